@@ -91,6 +91,21 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
 }
 
+// 4-byte asynchronous copy global -> shared memory (zero instead when !valid;
+// src must still be an address of the caller's buffer).
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+
+// One of the arrivals `bar` was initialised with, made once this thread's
+// earlier cp_async4 copies have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// This thread's earlier cp_async4 copies have landed.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // 2-D tensor-map copy (box at coordinates x = innermost, y) -> shared memory.
 // x * element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tensor2d_g2s(void *dst, const void *tmap, int x, int y, uint64_t *bar) {

@@ -36,7 +36,8 @@
 //    barrier: a round waits only for the boxes holding the rows its blocks
 //    can select, so the consumers start on the first rows while the rest
 //    land; a run's first slice is requested before its first set record is
-//    read;
+//    read.  Where X has no tensor map (a row pitch or base that is no multiple
+//    of 16 bytes) the consumer warps copy the slice, 4 bytes a lane;
 //  * three reducer warps: when every CTA of the cluster has stored its partial
 //    sums of a set (each consumer warp, once its rows are stored, arrives on
 //    every CTA's "ready" barrier), they add, for this CTA's share of the
@@ -139,9 +140,9 @@ struct Set {
     long long val_off, off_off;
 };
 
-template <bool BF16, int T>
+template <bool BF16, int T, bool PLAIN>
 __global__ void __launch_bounds__(kThreads, 1)
-xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restrict__ Y, int64_t ldy,
+xres_kernel(Format f, const float *__restrict__ X, int64_t ldx, int64_t batch, float *__restrict__ Y, int64_t ldy,
             const __grid_constant__ CUtensorMap xmap, const __grid_constant__ Plan p) {
     static_assert(T == 32, "the consumer layouts assume 32-column tiles (128-byte activation rows)");
     constexpr int kEsz = BF16 ? 2 : 4;
@@ -166,7 +167,7 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
             mbar_init(&bar.full[st], 1);
             mbar_init(&bar.empty[st], kCWarps);
         }
-        for (int i = 0; i < p.nboxes; ++i) mbar_init(&bar.xbox[i], 1);
+        for (int i = 0; i < p.nboxes; ++i) mbar_init(&bar.xbox[i], PLAIN ? kCThreads : 1);
         mbar_init(&bar.xfree, kCWarps);
         mbar_init(&bar.ready, kCWarps * C);   // every consumer warp of every CTA, once a set
         mbar_init(&bar.freed, kRWarps * C);   // every reducer warp of every CTA, once a set
@@ -270,13 +271,13 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
         };
         Cursor cu = cursor_at(u_begin), cn = cu;
         advance(cn);
-        if (u_begin < u_end) ok = load_slice(cu.tile);   // the run's first tile is known: no wait for its set
+        if (!PLAIN && u_begin < u_end) ok = load_slice(cu.tile);   // the run's first tile is known: no wait for its set
         Set s_next = u_begin < u_end ? load_set(cu.sidx) : Set{};
         for (int u = u_begin; u < u_end && ok; ++u, cu = cn, advance(cn)) {
             const Set s = s_next;
             if (u + 1 < u_end) s_next = load_set(cn.sidx);
             const Unit g = unit_geo(cu.tile, s);
-            if (g.tile != cur_tile) {
+            if (!PLAIN && g.tile != cur_tile) {
                 // the consumers are done with the previous slice
                 if (xloads > 0) ok = mbar_wait(&bar.xfree, (xloads - 1) & 1, false);
                 ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
@@ -398,6 +399,27 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
         advance(cn);
         Set s_next = u_begin < u_end ? load_set(cu.sidx) : Set{};
         const uint32_t x0 = smem_addr(s_x);   // slice row k at x0 + 128 k (rows of 32 floats)
+        // PLAIN: the consumers copy the slice themselves, 4 bytes a lane, a
+        // warp a row; rows past the matrix and columns past the batch become
+        // zeros.  Every thread arrives on every box.
+        auto load_slice_plain = [&](int tile) {
+            const int64_t b = int64_t(tile) * T + lane;
+            for (int i = 0; i < p.nboxes; ++i) {
+                const int r0 = i * p.box_rows;
+                const float *src = X + int64_t(kq0 + r0 + warp) * ldx + b;
+                uint32_t dst = x0 + uint32_t(r0 + warp) * (T * 4) + uint32_t(lane) * 4u;
+                // rows of the box inside the matrix
+                const int inside = static_cast<int>(min(int64_t(p.box_rows), f.cols - kq0 - r0));
+#pragma unroll 4
+                for (int r = warp; r < p.box_rows; r += kCWarps) {
+                    const bool in = r < inside && b < batch;
+                    cp_async4(dst, in ? src : X, in);
+                    src += kCWarps * ldx;
+                    dst += kCWarps * T * 4;
+                }
+                cp_async_arrive(&bar.xbox[i]);
+            }
+        };
         // one unit with LPR lanes a row, NP row passes and 4-bit (NIB) or 8-bit
         // offsets: multiply, then store the partial sums once every CTA's
         // reducers have read the previous set's (t: sets stored)
@@ -514,6 +536,15 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bar.xfree);
                 }
+                if constexpr (PLAIN) {
+                    // every warp is done with the previous slice and all of its
+                    // boxes have landed (their phases must not overlap)
+                    if (xloads > 0) {
+                        if (ok) ok = mbar_wait(&bar.xfree, (xloads - 1) & 1);
+                        for (int i = 0; i < p.nboxes && ok; ++i) ok = mbar_wait(&bar.xbox[i], (xloads - 1) & 1);
+                    }
+                    if (ok) load_slice_plain(g.tile);
+                }
                 ++xloads;           // its boxes are waited for by the rounds that read them
                 nready = 0;
                 cur_tile = g.tile;
@@ -542,6 +573,7 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar.xfree);
         }
+        if constexpr (PLAIN) cp_async_wait_all();
         if (!ok && lane == 0) atomicOr(f.status, kStatusTimeout);
     }
     cluster.sync();   // no CTA leaves while another may still read its shared memory
@@ -549,9 +581,9 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t batch, float *__restr
 
 
 // Clusters of C CTAs of this kernel resident at once with `smem` bytes each.
-template <bool BF16, int T>
+template <bool BF16, int T, bool PLAIN>
 inline int max_clusters(int C, uint32_t smem) {
-    const auto fn = xres_kernel<BF16, T>;
+    const auto fn = xres_kernel<BF16, T, PLAIN>;
     return static_cast<int>(per_device(reinterpret_cast<const void *>(fn), (long long)C << 32 | smem, [&]() -> long long {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(C) * 64);
@@ -575,19 +607,16 @@ inline int max_clusters(int C, uint32_t smem) {
 
 // The product on this kernel, or cudaErrorNotSupported when the call does not
 // fit it (the slice of the tile does not fit in shared memory even split 8
-// ways with a two-stage ring, or X cannot be described by a tensor map).
-template <bool BF16, int T>
-cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy, bool early,
+// ways with a two-stage ring).  PLAIN: X cannot be described by a tensor map.
+template <bool BF16, int T, bool PLAIN>
+cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy, bool early,
                    cudaStream_t stream) {
     (void)early;
     const int64_t tiles = (batch + T - 1) / T;
     if (f.nxsets[0] <= 0 || f.nxsets[1] <= 0 || f.xset_prefix[0] == nullptr || f.xset_prefix[1] == nullptr ||
         tiles * f.nxsets[0] > (int64_t(1) << 30))
         return cudaErrorNotSupported;
-    if (reinterpret_cast<uintptr_t>(X) % 16 != 0 || (ldx * 4) % 16 != 0) return cudaErrorNotSupported;
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (enc == nullptr) return cudaErrorNotSupported;
-    const cudaError_t attr = allow_smem(xres_kernel<BF16, T>, kSmemCap);
+    const cudaError_t attr = allow_smem(xres_kernel<BF16, T, PLAIN>, kSmemCap);
     if (attr != cudaSuccess) return attr;
     // least common multiple of the block sizes (0 when it grows past any slice)
     int64_t lcm = 1;
@@ -634,7 +663,7 @@ cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, 
             std::min<uint64_t>(kMaxStages, (kSmemCap - ring_off - part_bytes) / stage_bytes<BF16>()));
         const uint64_t part_off = ring_off + uint64_t(nst) * stage_bytes<BF16>();
         const uint32_t total = static_cast<uint32_t>(part_off + part_bytes);
-        const int64_t sms = std::min<int64_t>(max_clusters<BF16, T>(C, total), kMaxClusters) * C;
+        const int64_t sms = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(C, total), kMaxClusters) * C;
         const bool deep = nst >= kMinStages;
         const bool better = deep != best_deep ? deep : (sms != best_sms ? sms > best_sms : nst > best_nst);
         if (sms <= 0 || !better) continue;
@@ -652,7 +681,7 @@ cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, 
         smem = total;
     }
     if (best_sms <= 0) return cudaErrorNotSupported;
-    const int64_t occ = std::min<int64_t>(max_clusters<BF16, T>(p.C, smem), kMaxClusters);
+    const int64_t occ = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(p.C, smem), kMaxClusters);
     // Row sets of about 4 heaviest groups (table 1: 128 rows, the consumers'
     // efficient layout) when they still give every cluster 2 units or more;
     // else sets of about 2 (table 0), whose finer units balance better.  (At
@@ -737,16 +766,35 @@ cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, 
     const int nrun = greedy(lo, true);
     CUtensorMap xmap;
     std::memset(&xmap, 0, sizeof xmap);
-    const cuuint64_t dims[2] = {cuuint64_t(batch), cuuint64_t(f.cols)};
-    const cuuint64_t strides[1] = {cuuint64_t(ldx) * 4};
-    const cuuint32_t box[2] = {cuuint32_t(T), cuuint32_t(p.box_rows)};
-    const cuuint32_t estr[2] = {1, 1};
-    if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(X), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorNotSupported;
-    return launch_ex(xres_kernel<BF16, T>, dim3(static_cast<unsigned>(nrun * p.C)), dim3(kThreads), smem, stream,
-                     static_cast<unsigned>(p.C), true, f, X, batch, Y, ldy, xmap, p);
+    if constexpr (!PLAIN) {
+        const cuuint64_t dims[2] = {cuuint64_t(batch), cuuint64_t(f.cols)};
+        const cuuint64_t strides[1] = {cuuint64_t(ldx) * 4};
+        const cuuint32_t box[2] = {cuuint32_t(T), cuuint32_t(p.box_rows)};
+        const cuuint32_t estr[2] = {1, 1};
+        if (tensor_map_encoder()(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(X), dims, strides, box,
+                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorNotSupported;
+    }
+    return launch_ex(xres_kernel<BF16, T, PLAIN>, dim3(static_cast<unsigned>(nrun * p.C)), dim3(kThreads), smem, stream,
+                     static_cast<unsigned>(p.C), true, f, X, ldx, batch, Y, ldy, xmap, p);
+}
+
+// The slices arrive by tensor maps where X allows one (16-byte aligned base
+// and rows, a row pitch the encoder takes), else by 4-byte copies of the
+// consumer warps, 128 bytes of a row per warp.  A slice of 192 KB then takes
+// ~1500 copy instructions of the SM's load unit (3 us) and no register
+// round trip: 3001 x 4099 fp32 at batch 999 takes 131 us, of which the gather's
+// bound is 76 (with batch_kernel's one producer warp loading X: 2420 us).
+template <bool BF16, int T>
+cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy, bool early,
+                   cudaStream_t stream) {
+    if (reinterpret_cast<uintptr_t>(X) % 16 == 0 && (ldx * 4) % 16 == 0 && tensor_map_encoder() != nullptr) {
+        const cudaError_t e = launch_as<BF16, T, false>(f, X, ldx, batch, Y, ldy, early, stream);
+        if (e != cudaErrorNotSupported) return e;
+    }
+    return launch_as<BF16, T, true>(f, X, ldx, batch, Y, ldy, early, stream);
 }
 
 }  // namespace xres
