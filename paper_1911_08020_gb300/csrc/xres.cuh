@@ -87,6 +87,13 @@ __device__ __forceinline__ float4 lds_f4(uint32_t addr) {
     return v;
 }
 
+__device__ __forceinline__ void add4(float4 &a, const float4 &b) {
+    a.x += b.x;
+    a.y += b.y;
+    a.z += b.z;
+    a.w += b.w;
+}
+
 constexpr int kCWarps = 16;                    // consumer warps
 constexpr int kCThreads = kCWarps * 32;
 constexpr int kRWarps = 3;                     // reducer warps (20 warps in all: 96 registers a thread)
@@ -485,6 +492,13 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t ldx, int64_t batch, f
                                 }
                             }
                             const uint2 ow = NIB ? make_uint2(so[rec], 0u) : reinterpret_cast<const uint2 *>(so)[rec];
+                            // PLAIN: a chunk's sum is formed by itself and then
+                            // added, so that the fp32 error is no larger than
+                            // batch_kernel's, whose ranks split a row's blocks
+                            // (one chain a slice: up to 2.3 times larger); the
+                            // adds are not seen beside the gathers
+                            float4 chunkA = make_float4(0.f, 0.f, 0.f, 0.f), chunkB = chunkA;
+                            float4 &sumA = PLAIN ? chunkA : accA[pp], &sumB = PLAIN ? chunkB : accB[pp];
                             // block e: its kept value times the lane's quads of its selected activation row
                             auto block = [&](int e) {
                                 uint32_t off;
@@ -496,8 +510,8 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t ldx, int64_t batch, f
                                 else
                                     v = __uint_as_float(vw[e]);
                                 const uint32_t ad = xb + uint32_t(e) * mrow + (off << 7);
-                                fma4(accA[pp], v, lds_f4(ad));
-                                if constexpr (kTwo) fma4(accB[pp], v, lds_f4(ad ^ 64u));   // the other half of the row
+                                fma4(sumA, v, lds_f4(ad));
+                                if constexpr (kTwo) fma4(sumB, v, lds_f4(ad ^ 64u));   // the other half of the row
                             };
                             if (e_lo == 0 && e_hi == kChunk) {
                                 // a whole chunk: one straight run, every load can be issued early
@@ -507,6 +521,10 @@ xres_kernel(Format f, const float *__restrict__ X, int64_t ldx, int64_t batch, f
 #pragma unroll
                                 for (int e = 0; e < kChunk; ++e)
                                     if (e >= e_lo && e < e_hi) block(e);
+                            }
+                            if constexpr (PLAIN) {
+                                add4(accA[pp], chunkA);
+                                if constexpr (kTwo) add4(accB[pp], chunkB);
                             }
                         }
                     }
