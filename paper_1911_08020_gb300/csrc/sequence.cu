@@ -2,24 +2,43 @@
 // persistent, cooperative launch (the RNNs of Sec. 4.1 run many steps per
 // input; each step is the fused step of darb_lstm_step / darb_gru_step).
 //
-// Every CTA owns a contiguous range of hidden units and all gate rows of those
-// units (LSTM rows u, H+u, 2H+u, 3H+u; GRU rows u, H+u, 2H+u), so the cell of
-// a unit needs nothing from another CTA.  In the prologue a CTA decodes its
-// rows once into shared memory as packed (value, absolute column) words -- a
-// row's kept weights in column order -- and keeps them there for the whole
-// sequence, so W_darb leaves HBM/L2 once instead of once per step.  Per step
-// and per tile of batch columns it stages the stacked input [x_t; h_{t-1}] in
-// shared memory and forms its gate sums: a warp per gate row, the 32 lanes
-// split into 32/bt subgroups of bt batch columns, each subgroup taking every
-// (32/bt)-th kept weight, then a shuffle reduction over the subgroups.  The
-// cell is applied by the owning CTA, h_t goes to h_seq, c stays in a device
-// buffer that only its owner touches.  Steps are separated by a grid-wide
-// barrier (arrival counter in global memory, spun on with a 1 s limit; on
-// expiry the kernel records a timeout, raises an abort flag that ends every
-// other CTA's wait, and returns).  The launch is cooperative, so all CTAs are
-// resident and the barrier cannot starve.  No CTA touches another CTA's shared
-// memory, and no CTA leaves while a copy it issued may still be landing.
+// The batch columns are cut into tiles of bt <= 32 columns, and the CTAs into
+// column groups, each of which runs the recurrence of its own tiles: columns
+// are independent, so a group exchanges h only among its own CTAs, stages only
+// its own columns of it, and has a barrier of its own.  Within a group every CTA owns a contiguous range
+// of hidden units and all gate rows of those units (LSTM rows u, H+u, 2H+u,
+// 3H+u; GRU rows u, H+u, 2H+u), so the cell of a unit needs nothing from
+// another CTA.  In the prologue a CTA decodes its rows once into shared memory
+// as packed (value, staged row) words and keeps them there for the whole
+// sequence, so W_darb leaves HBM/L2 once instead of once per step.
+//
+// Per step and tile a CTA copies h_{t-1} (and x_t, unless the x parts of all
+// steps were one product up front) into shared memory and forms its gate
+// sums.  h_t goes to h_seq and to an exchange buffer laid out as the staged
+// tile is ([row][bt], two buffers by step parity), so that staging is a few
+// 1-D bulk copies whatever the batch's width and alignment.  A lane multiplies 4 columns (a
+// 16-byte load of the staged row its kept weight selects), bt / 4 lanes share
+// a weight, and the 128 / bt subgroups of a warp take the weights of a row in
+// turn; their sums meet in a shuffle reduction that leaves each lane one
+// column.  The owning CTA applies the cell.  Steps are separated by a barrier
+// over the group's CTAs (arrival counter in global memory, spun on with a 1 s
+// limit; on expiry the kernel records a timeout, raises an abort flag that
+// ends every other CTA's wait, and returns).  The launch is cooperative, so
+// all CTAs are resident and the barrier cannot starve.  No CTA touches another
+// CTA's shared memory, and no CTA leaves while a copy it issued may still be
+// landing.
+//
+// What bounds a step (cycle stamps, 6000 x 3000 bf16 at batch 20, tiles of 32,
+// ~14000 cycles): the gather and its reductions 6500, the barrier 2900, the
+// cell 2000, staging 1800.  One column group instead of one a tile stages every
+// column in every CTA: GRU 3072 x 2048 at batch 64 took 11.0 against 8.7 us a
+// step.  Against one lane a column, tensor-map staging and all CTAs in one
+// barrier, whole calls went from 3131 to 1606 us (that GRU, 200 steps), 507 to
+// 343 (the LSTM above, 35 steps), 520 to 399 (LSTM 4096 x 1280 fp32, batch 1,
+// 100 steps), and 2592 to 620 where the batch is no multiple of 4 (GRU 2100 x
+// 1000, batch 37, 100 steps).
 #include "darb_internal.h"
+#include "kernels_common.cuh"
 #include "launch.cuh"
 #include "rnn_epilogue.cuh"
 #include "tma.cuh"
@@ -34,33 +53,38 @@ namespace seq {
 constexpr int kThreads = 512;
 constexpr int kSeqWarps = kThreads / 32;
 constexpr int kMaxCtas = 256;
-constexpr size_t kSmemCap = 226 * 1024;   // dynamic shared memory, below the 227 KB opt-in with room for the static part
-constexpr int kMaxTile = 32;              // batch columns per tile, at most (one per lane)
+constexpr size_t kSmemCap = 226 * 1024 + 512;   // dynamic shared memory, below the 227 KB opt-in with room for the static part
+constexpr int kMaxLbt = 5;                // batch tiles of at most 2^5 columns
 constexpr size_t kCellOnChip = 16 * 1024; // LSTM cell state kept in shared memory up to this size
+constexpr int kBarWords = 32;             // words between the barrier counters of two groups (128 bytes)
+constexpr int kCopies = 8;                // bulk copies a staged tile is cut into, at most
 
 struct Ranges {
-    int32_t start[kMaxCtas + 1];   // CTA q owns hidden units [start[q], start[q+1])
+    int32_t start[kMaxCtas + 1];   // CTA q of a group owns hidden units [start[q], start[q+1])
 };
+
+// Where x_t comes from.
+constexpr int kXNone = 0;    // its products are precomputed (gx)
+constexpr int kXBulk = 1;    // tile-major rows (x_tiles), bulk copies
+constexpr int kXPlain = 2;   // the caller's x, plain loads (its tile-major copy would be too large)
 
 struct SeqArgs {
     int I, H, T;
-    int lbt;                // log2 of the batch tile width bt (bt <= 32)
-    int stage_mode;         // kStage*
+    int ngroups;            // column groups; CTA i is CTA i / ngroups of group i % ngroups
+    int ntiles;             // batch tiles; group g runs tiles g, g + ngroups, ...
+    int tpg;                // tiles of a group, at most
     int piece;              // kept weights per work item, at most
     int c_on_chip;          // LSTM: cell state in shared memory
-    // staged input rows: x_t at [0, I) (none when the x parts are precomputed),
-    // h_{t-1} from row ipad, a zero row at ipad + hpad
-    int ipad, hpad;
-    // tensor-map staging (tma != 0): boxes of {bt columns, bxh rows} over x_t
-    // (nbx of them) and {bt, bhh} over h_{t-1} (nbh), tile_bytes per tile in all
-    int tma, nbx, bxh, nbh, bhh;
-    uint32_t tile_bytes;
+    int x_mode;             // kX*
+    // staged input rows: x_t at [0, irows), h_{t-1} from row irows on (hrows of
+    // them), both rounded up to 4 rows; a zero row at irows + hrows
+    int irows, hrows;
     int64_t B;
     const float *gx;        // x parts of the gate sums of every step, rows x ldgx (row r, step t, column b
                             // at r * ldgx + t * B + b), or nullptr: x_t is staged with h_{t-1} instead
     int64_t ldgx;
-    const float *x;         // T x I x B
-    const float *h0;        // H x B
+    const float *x;         // T x I x B (kXPlain)
+    const float *x_tiles;   // T x ntiles x irows x bt (kXBulk)
     const float *c0;        // H x B (LSTM)
     const float *bias;      // LSTM [4H] or nullptr
     const float *b_ih;      // GRU [3H] or nullptr
@@ -69,16 +93,11 @@ struct SeqArgs {
     float *c_seq;           // T x H x B or nullptr (LSTM)
     float *c_state;         // H x B: the running cell state when it is not on chip (LSTM)
     float *c_last;          // H x B or nullptr (LSTM)
-    // a copy of h_t with rows of ldp columns (B rounded up to the batch tile,
-    // zeros past B) in two buffers by step parity, H x ldp each, or nullptr:
-    // h_{t-1} is then staged from h_seq.  Boxes over it are whole 128-byte
-    // aligned rows; boxes over B-column rows with a ragged tail are not
-    float *h_pad;
-    int64_t ldp;
-    unsigned *bar;          // arrival counter, zero at launch
+    float *h_x;             // the exchanged h_t, [t & 1][ntiles][hrows][bt]; h0 in buffer 1 at launch
+    unsigned *bar;          // arrival counters of the groups, kBarWords apart, zero at launch
     int *abort_flag;        // zero at launch
     int32_t *status;
-    unsigned long long barrier_ns;   // time limit of a grid-barrier wait (kWaitLimitNs unless a test shortens it)
+    unsigned long long barrier_ns;   // time limit of a barrier wait (kWaitLimitNs unless a test shortens it)
     int skip_cta;           // test hook: this CTA does not arrive at the first barrier (-1: none)
 };
 
@@ -89,7 +108,7 @@ struct SmemPlan {
 };
 
 inline SmemPlan smem_plan(int64_t kept_cap, int rows_cap, int items_cap, int units_cap, bool bf16, bool gru,
-                          int in_rows, int bt, int64_t B, bool c_on_chip, bool pre) {
+                          int in_rows, int bt, int tpg, bool c_on_chip, bool pre) {
     SmemPlan p{};
     p.items_cap = items_cap;
     size_t o = 0;
@@ -104,7 +123,7 @@ inline SmemPlan smem_plan(int64_t kept_cap, int rows_cap, int items_cap, int uni
     p.rowitem_off = take(size_t(rows_cap + 1) * 4);
     p.item_off = take(size_t(items_cap) * 16);
     p.bias_off = take(size_t(rows_cap) * 2 * 4);
-    p.c_off = take(c_on_chip ? size_t(units_cap) * size_t(B) * 4 : 0);
+    p.c_off = take(c_on_chip ? size_t(units_cap) * size_t(tpg) * bt * 4 : 0);
     p.gx_off = take(pre ? size_t(rows_cap) * bt * 4 : 0);
     p.in_off = take(size_t(in_rows) * bt * 4 + 128);   // rounded up to 128 bytes in the kernel
     p.part_off = take(size_t(gru ? 2 : 1) * items_cap * bt * 4);
@@ -127,44 +146,6 @@ template <> struct Packed<false> {  // fp32 bits, index
     static __device__ __forceinline__ float val(T w) { return __uint_as_float(w.x); }
     static __device__ __forceinline__ uint32_t col(T w) { return w.y; }
 };
-
-// Grid-wide barrier with a time limit; false if this CTA gave up or another
-// CTA did.  The CTA barrier orders every thread's h_t stores before thread 0's
-// arrival, a release reduction on the counter (no return trip, no separate
-// fence); thread 0 then polls with acquire loads.  An acquire that reads the
-// final count synchronises with every arrival (each is a read-modify-write in
-// the counter's release sequence), and the closing CTA barrier carries that
-// to the CTA's other threads.
-__device__ __forceinline__ bool grid_barrier(const SeqArgs &a, unsigned target, int *s_ok) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (!(int(blockIdx.x) == a.skip_cta && target == gridDim.x))
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
-        int ok = 1;
-        const unsigned long long t0 = global_timer_ns();
-        for (unsigned spin = 0;; ++spin) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
-            if (v >= target) break;
-            if ((spin & 63) == 63) {
-                if (*reinterpret_cast<volatile int *>(a.abort_flag)) {
-                    ok = 0;
-                    break;
-                }
-                if (global_timer_ns() - t0 > a.barrier_ns) {
-                    ok = 0;
-                    atomicExch(a.abort_flag, 1);
-                    atomicOr(a.status, kStatusTimeout);
-                    break;
-                }
-                __nanosleep(32);
-            }
-        }
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
 
 // On-chip layout of one row's kept weights: an x region, then an h region,
 // each padded with zero weights (pointing at the zero row of the staged input)
@@ -190,147 +171,209 @@ __host__ __device__ inline void row_regions(int n, int m, int I, bool pre, bool 
     }
 }
 
-// Sum over kept weights [pa, pb) of the CTA (multiples of 4), subgroup `sub`
-// taking every S-th group of 4 weights from pa + 4 sub, against one batch
-// column of the staged input: s_inc = s_in + that column, and a weight's
-// column field is the index of its staged row's first element, row * bt.
-template <class P>
-__device__ __forceinline__ float dot_range(const typename P::T *s_w, const float *s_inc, int pa, int pb, int sub,
-                                           int S) {
-    float acc0 = 0.0f, acc1 = 0.0f;
-#pragma unroll 2
-    for (int p = pa + 4 * sub; p < pb; p += 4 * S) {
-        typename P::T w[4];
-        if constexpr (sizeof(typename P::T) == 4) {
-            const uint4 q = *reinterpret_cast<const uint4 *>(s_w + p);
+// How the lanes of a warp share a tile of 2^LBT columns: a lane multiplies V
+// columns of a weight, L lanes share the weight, S subgroups of L lanes take
+// the weights of a row in turn, KW consecutive ones at a time (one load).
+template <int LBT>
+struct Lanes {
+    static constexpr int BT = 1 << LBT;
+    static constexpr int V = BT < 4 ? BT : 4;
+    static constexpr int L = BT / V;
+    static constexpr int S = 32 / L;
+    static constexpr int KW = S <= 4 ? 4 : S <= 8 ? 2 : 1;
+};
+
+template <class P, int KW>
+__device__ __forceinline__ void load_weights(const typename P::T *p, typename P::T (&w)[KW]) {
+    if constexpr (sizeof(typename P::T) == 4) {
+        if constexpr (KW == 4) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(p);
             w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+        } else if constexpr (KW == 2) {
+            const uint2 q = *reinterpret_cast<const uint2 *>(p);
+            w[0] = q.x; w[1] = q.y;
         } else {
-            const uint4 q0 = *reinterpret_cast<const uint4 *>(s_w + p);
-            const uint4 q1 = *reinterpret_cast<const uint4 *>(s_w + p + 2);
-            w[0] = make_uint2(q0.x, q0.y); w[1] = make_uint2(q0.z, q0.w);
-            w[2] = make_uint2(q1.x, q1.y); w[3] = make_uint2(q1.z, q1.w);
-        }
-        const float v0 = s_inc[P::col(w[0])], v1 = s_inc[P::col(w[1])];
-        const float v2 = s_inc[P::col(w[2])], v3 = s_inc[P::col(w[3])];
-        acc0 = fmaf(P::val(w[0]), v0, acc0);
-        acc1 = fmaf(P::val(w[1]), v1, acc1);
-        acc0 = fmaf(P::val(w[2]), v2, acc0);
-        acc1 = fmaf(P::val(w[3]), v3, acc1);
-    }
-    return acc0 + acc1;
-}
-
-// Input staging modes, chosen on the host from the shapes and alignments.
-constexpr int kStageScalar = 0;   // one float per load
-constexpr int kStageQuadCols = 1; // 4 batch columns per 16-byte load (B and bt multiples of 4, aligned)
-constexpr int kStageQuadRows = 2; // B == 1: 4 input rows per 16-byte load (I, H multiples of 4, aligned)
-constexpr int kStageUnroll = 8;   // loads a thread has in flight
-
-// s_in[k][j] = [x_t; h_{t-1}][k][b0 + j] for j < nb, 0 for nb <= j < bt, for
-// the K staged rows, of which the first I come from x_t (I = 0: h only).
-// h_{t-1} was written by other CTAs of this launch, so every load goes to L2
-// (ld.cg); the loads of a thread are issued together so that enough bytes are
-// in flight to cover the L2 latency, and each CTA starts its sweep at its own
-// offset so that the CTAs do not all ask for the same lines at once.
-__device__ __forceinline__ void stage_input(const SeqArgs &a, int I, int K, const float *xt, const float *hp,
-                                            int64_t b0, int nb, float *s_in) {
-    const int lbt = a.lbt, bt = 1 << lbt;
-    const int64_t B = a.B;
-    const int tid = threadIdx.x;
-    auto src = [&](int k) { return k < I ? xt + int64_t(k) * B : hp + int64_t(k - I) * B; };
-    if (a.stage_mode == kStageQuadCols) {
-        const int lq = lbt - 2, n = K << lq;   // quads
-        const int rot = static_cast<int>(int64_t(blockIdx.x) * n / gridDim.x);
-        for (int i0 = tid; i0 < n; i0 += kThreads * kStageUnroll) {
-            float4 v[kStageUnroll];
-#pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u) {
-                int i = i0 + u * kThreads;
-                v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (i < n) {
-                    i = i + rot < n ? i + rot : i + rot - n;
-                    const int k = i >> lq, j = (i & ((1 << lq) - 1)) * 4;
-                    if (j < nb) v[u] = __ldcg(reinterpret_cast<const float4 *>(src(k) + b0 + j));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u) {
-                const int i = i0 + u * kThreads;
-                if (i < n) reinterpret_cast<float4 *>(s_in)[i + rot < n ? i + rot : i + rot - n] = v[u];
-            }
-        }
-    } else if (a.stage_mode == kStageQuadRows) {
-        const int n = K >> 2;
-        const int rot = static_cast<int>(int64_t(blockIdx.x) * n / gridDim.x);
-        for (int i0 = tid; i0 < n; i0 += kThreads * kStageUnroll) {
-            float4 v[kStageUnroll];
-#pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u) {
-                int i = i0 + u * kThreads;
-                if (i < n) {
-                    i = i + rot < n ? i + rot : i + rot - n;
-                    v[u] = __ldcg(reinterpret_cast<const float4 *>(src(4 * i)));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u) {
-                const int i = i0 + u * kThreads;
-                if (i < n) reinterpret_cast<float4 *>(s_in)[i + rot < n ? i + rot : i + rot - n] = v[u];
-            }
+            w[0] = *p;
         }
     } else {
-        const int n = K << lbt;
-        for (int i0 = tid; i0 < n; i0 += kThreads * kStageUnroll) {
-            float v[kStageUnroll];
+        if constexpr (KW == 1) {
+            w[0] = *p;
+        } else {
 #pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u) {
-                const int i = i0 + u * kThreads;
-                const int k = i >> lbt, j = i & (bt - 1);
-                v[u] = 0.0f;
-                if (i < n && j < nb) v[u] = __ldcg(src(k) + b0 + j);
+            for (int i = 0; i < KW; i += 2) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(p + i);
+                w[i] = make_uint2(q.x, q.y);
+                w[i + 1] = make_uint2(q.z, q.w);
             }
-#pragma unroll
-            for (int u = 0; u < kStageUnroll; ++u)
-                if (i0 + u * kThreads < n) s_in[i0 + u * kThreads] = v[u];
         }
     }
 }
 
-template <bool BF16, int MODE>
+// Sums over kept weights [pa, pb) of the CTA (multiples of 4) against the
+// tile: subgroup `sub` takes every S-th run of KW weights from pa + KW sub,
+// s_inc = staged tile + the lane's first column.  The lane's V columns, each
+// from U * KW accumulators.
+template <class P, int LBT>
+__device__ __forceinline__ void dot_range(const typename P::T *s_w, const float *s_inc, int pa, int pb, int sub,
+                                          float (&acc)[Lanes<LBT>::V]) {
+    using G = Lanes<LBT>;
+    constexpr int V = G::V, KW = G::KW, U = KW < 4 ? 2 : 1, A = U * KW, kStep = KW * G::S;
+    float4 s[A];   // (V < 4: the first V of each)
+#pragma unroll
+    for (int i = 0; i < A; ++i) s[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int p = pa + KW * sub; p < pb; p += U * kStep) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = p + u * kStep;
+            if (u > 0 && q >= pb) continue;
+            typename P::T w[KW];
+            load_weights<P, KW>(s_w + q, w);
+#pragma unroll
+            for (int i = 0; i < KW; ++i) {
+                const float *x = s_inc + P::col(w[i]);
+                const float v = P::val(w[i]);
+                float4 &d = s[u * KW + i];
+                if constexpr (V == 4) {
+                    fma4(d, v, *reinterpret_cast<const float4 *>(x));
+                } else if constexpr (V == 2) {
+                    const float2 x2 = *reinterpret_cast<const float2 *>(x);
+                    d.x = fmaf(v, x2.x, d.x);
+                    d.y = fmaf(v, x2.y, d.y);
+                } else {
+                    d.x = fmaf(v, *x, d.x);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int h = A / 2; h >= 1; h /= 2)
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            s[i].x += s[i + h].x;
+            if constexpr (V > 1) s[i].y += s[i + h].y;
+            if constexpr (V > 2) s[i].z += s[i + h].z;
+            if constexpr (V > 2) s[i].w += s[i + h].w;
+        }
+    acc[0] = s[0].x;
+    if constexpr (V > 1) acc[1] = s[0].y;
+    if constexpr (V > 2) acc[2] = s[0].z;
+    if constexpr (V > 2) acc[3] = s[0].w;
+}
+
+// Add the subgroups' sums of an item and store them at part[0 .. BT): the
+// first exchanges halve the columns a lane keeps (from V to 1), the rest add
+// whole; a fixed order, so deterministic.
+template <int LBT>
+__device__ __forceinline__ void reduce_store(float (&acc)[Lanes<LBT>::V], int lane, float *part) {
+    using G = Lanes<LBT>;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    int col = (lane & (G::L - 1)) * G::V;
+    float v;
+    int o = 16;   // the lane bits from L up to 16 number the subgroups
+    if constexpr (G::V == 4) {
+        const bool up = lane & 16;
+        const float s0 = up ? acc[0] : acc[2], s1 = up ? acc[1] : acc[3];
+        const float k0 = (up ? acc[2] : acc[0]) + __shfl_xor_sync(kAll, s0, 16);
+        const float k1 = (up ? acc[3] : acc[1]) + __shfl_xor_sync(kAll, s1, 16);
+        const bool up8 = lane & 8;
+        v = (up8 ? k1 : k0) + __shfl_xor_sync(kAll, up8 ? k0 : k1, 8);
+        col += (up ? 2 : 0) + (up8 ? 1 : 0);
+        o = 4;
+    } else if constexpr (G::V == 2) {
+        const bool up = lane & 16;
+        v = (up ? acc[1] : acc[0]) + __shfl_xor_sync(kAll, up ? acc[0] : acc[1], 16);
+        col += up ? 1 : 0;
+        o = 8;
+    } else {
+        v = acc[0];
+    }
+    const int rest = 2 * o - G::L;   // lane bits still to add over: L .. o
+#pragma unroll
+    for (int b = o; b >= G::L; b >>= 1) v += __shfl_xor_sync(kAll, v, b);
+    if ((lane & rest) == 0) part[col] = v;
+}
+
+// Thread 0's wait for the arrivals of its group; false if it gave up or
+// another CTA did.  The CTA barrier before an arrival orders every thread's
+// h_t stores before it; the arrival is a release reduction on the counter (no
+// return trip, no separate fence).  An acquire that reads the final count
+// synchronises with every arrival (each is a read-modify-write in the
+// counter's release sequence).
+__device__ __forceinline__ bool wait_arrivals(const SeqArgs &a, const unsigned *bar, unsigned target) {
+    const unsigned long long t0 = global_timer_ns();
+    for (unsigned spin = 0;; ++spin) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        if (v >= target) return true;
+        if ((spin & 63) == 63) {
+            if (*reinterpret_cast<volatile int *>(a.abort_flag)) return false;
+            if (global_timer_ns() - t0 > a.barrier_ns) {
+                atomicExch(a.abort_flag, 1);
+                atomicOr(a.status, kStatusTimeout);
+                return false;
+            }
+            __nanosleep(32);
+        }
+    }
+}
+
+// A tile of `bytes` (a multiple of 16): one warp, each of its first kCopies
+// lanes a bulk copy that completes on `bar` (one thread issuing all of them
+// took 1400 cycles of a step).  Lane 0 arms `bar`
+// first.
+__device__ __forceinline__ void copy_tile(int lane, float *dst, const float *src, uint32_t bytes, uint64_t *bar) {
+    // every thread of this CTA is done with the previous tile (the barrier
+    // that ended it); order those reads, and what other CTAs published by
+    // generic stores, before the copies
+    fence_proxy_async_smem();
+    fence_proxy_async_global();
+    if (lane == 0) mbar_arrive_expect_tx(bar, bytes);
+    __syncwarp();
+    const uint32_t each = (bytes / kCopies + 127) & ~127u, at = uint32_t(lane) * each;
+    if (lane < kCopies && at < bytes)
+        bulk_g2s(reinterpret_cast<char *>(dst) + at, reinterpret_cast<const char *>(src) + at,
+                 lane == kCopies - 1 || bytes - at < each ? bytes - at : each, bar);
+}
+
+template <bool BF16, int MODE, int LBT>
 __global__ void __launch_bounds__(kThreads, 1)
-seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp, const __grid_constant__ CUtensorMap mx,
-           const __grid_constant__ CUtensorMap mh0, const __grid_constant__ CUtensorMap mhs) {
+seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
+    using G = Lanes<LBT>;
     constexpr int kGates = MODE == kModeLstm ? 4 : 3;
     constexpr bool kGru = MODE == kModeGru;
+    constexpr int bt = G::BT;
     using P = Packed<BF16>;
     using PT = typename P::T;
     extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int s_ok, s_nitems, s_staged, s_next;
-    __shared__ __align__(8) uint64_t s_full;   // the staged tile has landed
+    __shared__ int s_nitems, s_next, s_fail;
+    __shared__ __align__(8) uint64_t s_hfull, s_xfull;   // the staged h / x rows have landed
     PT *s_w = reinterpret_cast<PT *>(sm + sp.w_off);
     int *s_rowptr = reinterpret_cast<int *>(sm + sp.rowptr_off);
     int *s_mid = reinterpret_cast<int *>(sm + sp.mid_off);          // GRU: first kept weight of a row on h
     int *s_rowitem = reinterpret_cast<int *>(sm + sp.rowitem_off);  // items of local row lr: [s_rowitem[lr], s_rowitem[lr+1])
-    int4 *s_item = reinterpret_cast<int4 *>(sm + sp.item_off);      // (first, end, local row, first on h)
+    int4 *s_item = reinterpret_cast<int4 *>(sm + sp.item_off);      // (first, end, number (at first: local row), first on h)
     float *s_bias = reinterpret_cast<float *>(sm + sp.bias_off);    // [R] (GRU: [2R], b_ih then b_hh)
-    float *s_c = reinterpret_cast<float *>(sm + sp.c_off);          // [units][B] when on chip
+    float *s_c = reinterpret_cast<float *>(sm + sp.c_off);          // [units][tpg * bt] when on chip
     float *s_gx = reinterpret_cast<float *>(sm + sp.gx_off);        // [R][bt]: x parts of this tile
     float *s_in = reinterpret_cast<float *>(                          // [kin + 1][bt], row kin zero
         (reinterpret_cast<uintptr_t>(sm + sp.in_off) + 127) & ~uintptr_t(127));
     float *s_part = reinterpret_cast<float *>(sm + sp.part_off);    // [parts][items][bt]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int u0 = rg.start[blockIdx.x], nu = rg.start[blockIdx.x + 1] - u0;
+    const int group = int(blockIdx.x) % a.ngroups, member = int(blockIdx.x) / a.ngroups;
+    const unsigned members = gridDim.x / unsigned(a.ngroups);
+    unsigned *bar = a.bar + group * kBarWords;
+    const int u0 = rg.start[member], nu = rg.start[member + 1] - u0;
     const int R = kGates * nu;   // local row q*nu + i is matrix row q*H + u0 + i
     const int I = a.I, H = a.H;
-    const int lbt = a.lbt, bt = 1 << lbt, S = 32 >> lbt;
-    const int sub = lane >> lbt, col = lane & (bt - 1);
+    const int sub = lane / G::L, col = (lane % G::L) * G::V;
     const int64_t B = a.B;
     // with the x parts precomputed only h_{t-1} is staged and only the kept
     // weights of blocks that reach column I are kept on chip (columns shifted by I)
     const bool pre = a.gx != nullptr;
     // GRU without precomputed x parts keeps the x and h sums of each item apart
     const bool split = kGru && !pre;
-    const int kin = a.ipad + a.hpad;
+    const int kin = a.irows + a.hrows;
     auto grow = [&](int lr) { return (lr / nu) * H + u0 + lr % nu; };
 
     // ---- prologue: row sizes, biases, cell state, the zero row of the staged input
@@ -348,12 +391,18 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp, const __grid_constant__ 
             s_bias[lr] = a.bias ? a.bias[r] : 0.0f;
         }
     }
+    const int cw = a.tpg << LBT;   // columns of the on-chip cell state
     if constexpr (!kGru)
         if (a.c_on_chip)
-            for (int i = tid; i < nu * B; i += kThreads) s_c[i] = a.c0[int64_t(u0) * B + i];
-    for (int j = tid; j < bt; j += kThreads) s_in[(kin << lbt) + j] = 0.0f;
+            for (int i = tid; i < nu * cw; i += kThreads) {
+                const int64_t b = (int64_t(group + (i % cw >> LBT) * a.ngroups) << LBT) + (i & (bt - 1));
+                s_c[i] = b < B ? a.c0[int64_t(u0 + i / cw) * B + b] : 0.0f;
+            }
+    for (int j = tid; j < bt; j += kThreads) s_in[(kin << LBT) + j] = 0.0f;
     if (tid == 0) {
-        mbar_init(&s_full, 1);
+        mbar_init(&s_hfull, 1);
+        mbar_init(&s_xfull, 1);
+        s_fail = 0;
         fence_mbar_init();
     }
     __syncthreads();
@@ -374,7 +423,7 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp, const __grid_constant__ 
     }
     __syncthreads();
     // zero weights everywhere, then every kept weight as (value, staged row)
-    for (int p = tid; p < s_rowptr[R]; p += kThreads) s_w[p] = P::make(0u, uint32_t(kin) << lbt);
+    for (int p = tid; p < s_rowptr[R]; p += kThreads) s_w[p] = P::make(0u, uint32_t(kin) << LBT);
     __syncthreads();
     for (int lr = warp; lr < R; lr += kSeqWarps) {
         const int loc = f.rowloc[grow(lr)];
@@ -397,119 +446,147 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp, const __grid_constant__ 
             if (pre || kGru) at = on_h ? mid + j - jmid : base + j;   // h region from block jmid on
             else at = base + j;
             if (on_h) {
-                c = c - uint32_t(I) + uint32_t(a.ipad);   // staged row of h
+                c = c - uint32_t(I) + uint32_t(a.irows);   // staged row of h
             } else if (pre) {   // an x weight of block jmid: its product is in gx
                 bits = 0;
                 c = uint32_t(kin);
                 at = mid;
             }
-            s_w[at] = P::make(bits, c << lbt);   // (kin + 1) * bt floats fit in shared memory: < 2^16
+            s_w[at] = P::make(bits, c << LBT);   // (kin + 1) * bt floats fit in shared memory: < 2^16
         }
     }
     __syncthreads();
     const int NI = s_nitems;
-    if (tid == 0) s_next = 0;
-    for (int i = tid; i < NI; i += kThreads) {
-        int4 it = s_item[i];
-        it.w = split ? max(it.x, min(it.y, s_mid[it.z])) : it.y;
-        s_item[i] = it;
+    if (tid == 0) s_next = kSeqWarps;   // a warp's first item is its own index
+    // the items in descending order of their weights, so that the last ones
+    // handed out are short; z becomes the item's number (its partial sums)
+    for (int i0 = 0; i0 < NI; i0 += kThreads) {
+        const int i = i0 + tid;
+        int4 it = make_int4(0, 0, 0, 0);
+        int rank = 0;
+        if (i < NI) {
+            it = s_item[i];
+            it.w = split ? max(it.x, min(it.y, s_mid[it.z])) : it.y;
+            it.z = i;
+            const int n = it.y - it.x;
+            for (int o = 0; o < NI; ++o) {
+                const int2 other = *reinterpret_cast<const int2 *>(s_item + o);
+                rank += other.y - other.x > n || (other.y - other.x == n && o < i);
+            }
+        }
+        if (NI > kThreads) break;   // too many to sort in one pass: their order stays
+        __syncthreads();
+        if (i < NI) s_item[rank] = it;
     }
+    if (NI > kThreads)
+        for (int i = tid; i < NI; i += kThreads) {
+            s_item[i].w = split ? max(s_item[i].x, min(s_item[i].y, s_mid[s_item[i].z])) : s_item[i].y;
+            s_item[i].z = i;
+        }
     __syncthreads();
 
     // ---- the steps
-    int tile = 0;   // tiles staged so far: the parity of s_full
+    const uint32_t xbytes = uint32_t(a.irows) * bt * 4, hbytes = uint32_t(a.hrows) * bt * 4;
+    // x_t of one tile (the last warp): its rows are free once the tile before has been multiplied
+    auto copy_x = [&](int t, int tile) {
+        copy_tile(lane, s_in, a.x_tiles + (int64_t(t) * a.ntiles + tile) * (int64_t(a.irows) << LBT), xbytes, &s_xfull);
+    };
+    const bool xbulk = a.x_mode == kXBulk;
+    if (xbulk && warp == kSeqWarps - 1) copy_x(0, group);
+    int staged = 0;   // tiles staged so far: the parity of s_hfull and s_xfull
     float *c_run = kGru ? nullptr : (a.c_on_chip ? s_c : a.c_state + int64_t(u0) * B);
     for (int t = 0; t < a.T; ++t) {
-        const float *xt = a.x + int64_t(t) * I * B;
-        const float *hp = t == 0 ? a.h0 : a.h_seq + int64_t(t - 1) * H * B;
         float *ht = a.h_seq + int64_t(t) * H * B + int64_t(u0) * B;
         float *ct = a.c_seq ? a.c_seq + int64_t(t) * H * B + int64_t(u0) * B : nullptr;
-        const float *cp = kGru ? nullptr : (t == 0 && !a.c_on_chip ? a.c0 + int64_t(u0) * B : c_run);
-        for (int64_t b0 = 0; b0 < B; b0 += bt) {
+        for (int k = 0, tile = group; tile < a.ntiles; ++k, tile += a.ngroups, ++staged) {
+            const int64_t b0 = int64_t(tile) << LBT;
             const int nb = static_cast<int>(B - b0 < bt ? B - b0 : bt);
-            // stage [x_t; h_{t-1}] (or h_{t-1}) for columns [b0, b0 + nb), zeros past the batch
-            if (a.tma && tid == 0) {
-                // every thread of this CTA is done with the previous tile (the
-                // barrier that ended it); order those reads before the copies
-                fence_proxy_async_smem();
-                fence_proxy_async_global();   // h_{t-1} was published by generic stores
-                mbar_arrive_expect_tx(&s_full, a.tile_bytes);
-                for (int bx = 0; bx < a.nbx + a.nbh; ++bx) {
-                    const bool isx = bx < a.nbx;
-                    const int y = isx ? bx * a.bxh : (bx - a.nbx) * a.bhh;
-                    float *dst = s_in + (int64_t(isx ? y : a.ipad + y) << lbt);
-                    const CUtensorMap *m = isx ? &mx : (t == 0 ? &mh0 : &mhs);
-                    const int z = isx ? t : (t == 0 ? 0 : (a.h_pad ? (t - 1) & 1 : t - 1));
-                    tensor3d_g2s(dst, m, static_cast<int>(b0), y, z, &s_full);
+            if (pre)
+                for (int i = tid; i < R << LBT; i += kThreads) {
+                    const int lr = i >> LBT, j = i & (bt - 1);
+                    cp_async4(smem_addr(s_gx + i),
+                              a.gx + int64_t(grow(lr)) * a.ldgx + int64_t(t) * B + b0 + (j < nb ? j : 0), j < nb);
                 }
-                bool ok = mbar_wait(&s_full, tile & 1, false);
-                if (!ok) {
+            if (a.x_mode == kXPlain)
+                for (int i = tid; i < I << LBT; i += kThreads) {
+                    const int j = i & (bt - 1);
+                    s_in[i] = j < nb ? __ldg(a.x + (int64_t(t) * I + (i >> LBT)) * B + b0 + j) : 0.0f;
+                }
+            if (warp == 0) {
+                int go = 1;
+                if (lane == 0 && k == 0 && t > 0) go = wait_arrivals(a, bar, unsigned(t) * members);
+                if (__shfl_sync(0xFFFFFFFFu, go, 0)) {
+                    copy_tile(lane, s_in + (a.irows << LBT),
+                              a.h_x + (int64_t((t + 1) & 1) * a.ntiles + tile) * (int64_t(a.hrows) << LBT), hbytes,
+                              &s_hfull);
+                } else if (lane == 0) {
+                    s_fail = 1;
+                    mbar_arrive(&s_hfull);   // no copy comes: let the waiting threads see s_fail
+                }
+            }
+            if (a.x_mode == kXPlain) __syncthreads();
+            bool ok = mbar_wait(&s_hfull, staged & 1);
+            if (xbulk) ok = mbar_wait(&s_xfull, staged & 1) && ok;
+            // partial gate sums of the work items, handed out to warps as they come free
+            for (int ii = warp; ii < NI;) {
+                int next = 0;
+                if (lane == 0) next = atomicAdd(&s_next, 1);
+                const int4 it = s_item[ii];
+                float acc[G::V];
+                dot_range<P, LBT>(s_w, s_in + col, it.x, it.w, sub, acc);
+                reduce_store<LBT>(acc, lane, s_part + (it.z << LBT));
+                if (split) {
+                    dot_range<P, LBT>(s_w, s_in + col, it.w, it.y, sub, acc);
+                    reduce_store<LBT>(acc, lane, s_part + ((NI + it.z) << LBT));
+                }
+                ii = __shfl_sync(0xFFFFFFFFu, next, 0);
+            }
+            if (pre) cp_async_wait_all();
+            if (!__syncthreads_and(ok) || s_fail) {
+                // a wait gave up: end the other CTAs' waits too.  Copies of this
+                // CTA may still land: give them a second bounded wait before it leaves
+                if (tid == 0) {
                     atomicOr(a.status, kStatusTimeout);
                     atomicExch(a.abort_flag, 1);
-                    // the copies may still land: give them a second bounded wait
-                    // before this CTA leaves
-                    mbar_wait(&s_full, tile & 1, false);
+                    mbar_wait(&s_hfull, staged & 1);
+                    if (xbulk) mbar_wait(&s_xfull, staged & 1);
                 }
-                s_staged = ok;
+                return;
             }
-            if (pre)
-                for (int i = tid; i < R << lbt; i += kThreads) {
-                    const int lr = i >> lbt, j = i & (bt - 1);
-                    s_gx[i] = j < nb ? __ldg(a.gx + int64_t(grow(lr)) * a.ldgx + int64_t(t) * B + b0 + j) : 0.0f;
-                }
-            if (!a.tma) stage_input(a, pre ? 0 : I, kin, xt, hp, b0, nb, s_in);
-            __syncthreads();
-            if (a.tma) {
-                if (!s_staged) return;
-                mbar_wait(&s_full, tile & 1, false);   // completed: makes the copied data visible to this thread
+            if (warp == kSeqWarps - 1) {
+                if (lane == 0) s_next = kSeqWarps;   // for the next tile; every warp has left the loop
+                // the next tile's x rows, while the cell and the barrier run
+                const bool more = tile + a.ngroups < a.ntiles;
+                if (xbulk && (more || t + 1 < a.T)) copy_x(more ? t : t + 1, more ? tile + a.ngroups : group);
             }
-            // partial gate sums of the work items, handed out to warps as they come free
-            while (true) {
-                int ii = 0;
-                if (lane == 0) ii = atomicAdd(&s_next, 1);
-                ii = __shfl_sync(0xFFFFFFFFu, ii, 0);
-                if (ii >= NI) break;
-                const int4 it = s_item[ii];
-                float a0 = dot_range<P>(s_w, s_in + col, it.x, it.w, sub, S);
-                float a1 = 0.0f;
-                if (split) a1 = dot_range<P>(s_w, s_in + col, it.w, it.y, sub, S);
-                for (int o = 16; o >= bt; o >>= 1) {
-                    a0 += __shfl_xor_sync(0xFFFFFFFFu, a0, o);
-                    if (split) a1 += __shfl_xor_sync(0xFFFFFFFFu, a1, o);
-                }
-                if (sub == 0) {
-                    s_part[(ii << lbt) + col] = a0;
-                    if (split) s_part[((NI + ii) << lbt) + col] = a1;
-                }
-            }
-            __syncthreads();
-            if (tid == 0) s_next = 0;   // for the next tile; every warp has left the loop
             // the cells of the owned units for these columns
             // partial sums of local row lr: part 0 (everything, or the x part of a
             // split GRU row), part 1 (the h part of a split GRU row)
             auto sum = [&](int lr, int part, int j) {
                 float v = 0.0f;
-                for (int ii = s_rowitem[lr]; ii < s_rowitem[lr + 1]; ++ii) v += s_part[((part * NI + ii) << lbt) + j];
+                for (int ii = s_rowitem[lr]; ii < s_rowitem[lr + 1]; ++ii) v += s_part[((part * NI + ii) << LBT) + j];
                 return v;
             };
-            for (int i = tid; i < nu << lbt; i += kThreads) {
-                const int ui = i >> lbt, j = i & (bt - 1);
-                float *hq = a.h_pad ? a.h_pad + (int64_t(t & 1) * H + u0 + ui) * a.ldp + b0 + j : nullptr;
+            float *hx = a.h_x + ((int64_t(t & 1) * a.ntiles + tile) * a.hrows + u0) * bt;
+            for (int i = tid; i < nu << LBT; i += kThreads) {
+                const int ui = i >> LBT, j = i & (bt - 1);
                 if (j >= nb) {
-                    if (hq) *hq = 0.0f;
+                    hx[i] = 0.0f;
                     continue;
                 }
                 const int64_t e = int64_t(ui) * B + b0 + j;
-                auto xg = [&](int lr) { return pre ? s_gx[(lr << lbt) + j] : 0.0f; };
+                auto xg = [&](int lr) { return pre ? s_gx[(lr << LBT) + j] : 0.0f; };
                 if constexpr (MODE == kModeLstm) {
                     auto gate = [&](int lr) { return s_bias[lr] + sum(lr, 0, j) + xg(lr); };
                     const float pi = gate(ui), pf = gate(nu + ui), pg = gate(2 * nu + ui), po = gate(3 * nu + ui);
-                    const float c = sigm(pf) * cp[e] + sigm(pi) * tanhf(pg);
-                    c_run[e] = c;
-                    if (ct) ct[e] = c;
+                    const int64_t ec = a.c_on_chip ? ui * cw + (k << LBT) + j : e;
+                    const float cprev = t == 0 && !a.c_on_chip ? a.c0[int64_t(u0) * B + e] : c_run[ec];
+                    const float c = sigm(pf) * cprev + sigm(pi) * tanhf(pg);
                     const float hv = sigm(po) * tanhf(c);
+                    hx[i] = hv;
+                    c_run[ec] = c;
+                    if (ct) ct[e] = c;
                     ht[e] = hv;
-                    if (hq) *hq = hv;
                 } else {
                     // x part (b_ih + W_x x) and h part (b_hh + W_h h) of each gate
                     auto gx_ = [&](int lr) { return s_bias[lr] + (pre ? xg(lr) : sum(lr, 0, j)); };
@@ -517,19 +594,49 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp, const __grid_constant__ 
                     const float rr = sigm(gx_(ui) + gh_(ui));
                     const float zz = sigm(gx_(nu + ui) + gh_(nu + ui));
                     const float nn = tanhf(gx_(2 * nu + ui) + rr * gh_(2 * nu + ui));
-                    const float hv = (1.0f - zz) * nn + zz * s_in[((a.ipad + u0 + ui) << lbt) + j];
+                    const float hv = (1.0f - zz) * nn + zz * s_in[((a.irows + u0 + ui) << LBT) + j];
+                    hx[i] = hv;
                     ht[e] = hv;
-                    if (hq) *hq = hv;
                 }
             }
             __syncthreads();
-            ++tile;
         }
-        if (t + 1 < a.T && !grid_barrier(a, unsigned(t + 1) * gridDim.x, &s_ok)) return;
+        if (t + 1 < a.T && tid == 0 && !(int(blockIdx.x) == a.skip_cta && t == 0))
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     }
     if constexpr (!kGru)
         if (a.c_on_chip && a.c_last)
-            for (int i = tid; i < nu * B; i += kThreads) a.c_last[int64_t(u0) * B + i] = s_c[i];
+            for (int i = tid; i < nu * cw; i += kThreads) {
+                const int64_t b = (int64_t(group + (i % cw >> LBT) * a.ngroups) << LBT) + (i & (bt - 1));
+                if (b < B) a.c_last[int64_t(u0 + i / cw) * B + b] = s_c[i];
+            }
+}
+
+// What a call needs in place before seq_kernel: the barrier counters zero, h0
+// in the exchange buffer, and x_t of every step as tile-major rows (x_tiles)
+// or as the columns of one product input (xall[k][t * B + b] = x[t][k][b]).
+// A warp per row of h0 or of an x_t.
+__global__ void __launch_bounds__(256) prep_kernel(SeqArgs a, int lbt, const float *h0, float *x_tiles, float *xall,
+                                                   int64_t ldxall, int nwords) {
+    const int64_t B = a.B;
+    const int lane = threadIdx.x & 31;
+    for (int i = int(blockIdx.x) * 256 + int(threadIdx.x); i < nwords; i += int(gridDim.x) * 256) a.bar[i] = 0u;
+    const int bt = 1 << lbt;
+    const int64_t nrows = a.H + (x_tiles || xall ? int64_t(a.T) * a.I : 0);
+    for (int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); row < nrows; row += int64_t(gridDim.x) * 8) {
+        const int64_t xrow = row - a.H;
+        const int64_t t = xrow / a.I, k = xrow < 0 ? row : xrow % a.I;
+        if (xrow >= 0 && xall != nullptr) {
+            for (int64_t b = lane; b < B; b += 32) xall[k * ldxall + t * B + b] = __ldg(a.x + xrow * B + b);
+            continue;
+        }
+        const float *src = xrow < 0 ? h0 + row * B : a.x + xrow * B;
+        const int nr = xrow < 0 ? a.hrows : a.irows;   // rows of a tile
+        float *dst = (xrow < 0 ? a.h_x + ((int64_t(a.ntiles) * nr) << lbt) : x_tiles + ((t * a.ntiles * nr) << lbt)) +
+                     (k << lbt);
+        for (int64_t b = lane; b < (int64_t(a.ntiles) << lbt); b += 32)
+            dst[(((b >> lbt) * nr) << lbt) + (b & (bt - 1))] = b < B ? __ldg(src + b) : 0.0f;
+    }
 }
 
 }  // namespace seq
@@ -574,21 +681,15 @@ void split_units(const std::vector<int64_t> &kept, int G, seq::Ranges &rg, int64
     rg.start[G] = H;
 }
 
-}  // namespace
 
-// x_t of every step laid out as the columns of one product input:
-// xall[k][t * B + b] = x[t][k][b] for k < I (a warp per (t, k), lanes over b).
-__global__ void __launch_bounds__(256) gather_x_kernel(const float *x, int T, int I, int64_t B, float *xall,
-                                                       int64_t ldx) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nrows = int64_t(T) * I;
-    for (int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); row < nrows; row += int64_t(gridDim.x) * 8) {
-        const int64_t t = row / I, k = row % I;
-        const float *src = x + row * B;
-        float *dst = xall + k * ldx + t * B;
-        for (int64_t b = lane; b < B; b += 32) dst[b] = __ldg(src + b);
-    }
-}
+// A tile width and a number of column groups to try, and what a step is
+// expected to take (ns).
+struct Shape {
+    int lbt, ngroups, tpg;
+    double ns;
+};
+
+}  // namespace
 
 // Whether the x parts of all steps go through one darb_spmm-style product up
 // front: when x_t is a large share of the stacked input the per-step staging
@@ -598,7 +699,20 @@ inline bool precompute_x(int64_t T, int64_t I, int64_t H, int64_t B, size_t ws_b
 }
 
 template <bool BF16, int MODE>
-static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqArgs a, float *c_last,
+static auto seq_entry(int lbt) {
+    using namespace seq;
+    switch (lbt) {
+        case 0: return seq_kernel<BF16, MODE, 0>;
+        case 1: return seq_kernel<BF16, MODE, 1>;
+        case 2: return seq_kernel<BF16, MODE, 2>;
+        case 3: return seq_kernel<BF16, MODE, 3>;
+        case 4: return seq_kernel<BF16, MODE, 4>;
+        default: return seq_kernel<BF16, MODE, 5>;
+    }
+}
+
+template <bool BF16, int MODE>
+static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqArgs a, const float *h0, float *c_last,
                                 cudaStream_t stream) {
     using namespace seq;
     constexpr int kGates = MODE == kModeLstm ? 4 : 3;
@@ -618,93 +732,95 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
         return int64_t(xr + hr);
     };
     std::vector<int64_t> kept(static_cast<size_t>(H));
+    int64_t total = 0;
     for (int u = 0; u < H; ++u) {
         int64_t k = 0;
         for (int q = 0; q < kGates; ++q) k += row_kept(int64_t(q) * H + u);
         kept[static_cast<size_t>(u)] = k;
+        total += k;
     }
-    auto aligned = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-    const int xrows = pre ? 0 : I;   // staged rows that come from x_t
-    const bool ptrs = (xrows == 0 || aligned(a.x)) && aligned(a.h0) && aligned(a.h_seq);
-    // tensor-map staging needs 16-byte rows of every source (B a multiple of 4)
-    const bool tma_ok = ptrs && B % 4 == 0 && tensor_map_encoder() != nullptr;
-    const int G = std::max(1, std::min({sm_count(), H, kMaxCtas}));
-    Ranges rg{};
-    int64_t kept_cap = 0;
-    int units_cap = 0;
-    split_units(kept, G, rg, kept_cap, units_cap);
-    if (kept_cap > (int64_t(1) << 20)) return cudaErrorNotSupported;
-    const bool c_on_chip = !kGru && size_t(units_cap) * size_t(B) * 4 <= kCellOnChip;
-    // staged rows per box: at most 256, and a multiple of 32 / bt so that every
-    // box lands on a 128-byte boundary; as few padding rows as possible
-    auto box_rows = [](int n, int align, int &nbox, int &rows) {
-        nbox = (n + 255) / 256;
-        rows = nbox ? ((n + nbox - 1) / nbox + align - 1) / align * align : 0;
-        if (rows > 256) rows = 256 / align * align, nbox = (n + rows - 1) / rows;
-    };
-    int nbx = 0, bxh = 0, nbh = 0, bhh = 0;
-    // widest batch tile (a power of two, <= 32) whose staging still fits, with
-    // rows cut into work items of about kept_cap / (ipw * warps) weights (a
-    // multiple of 4, at least 2 loads of 4 weights per subgroup): ipw = 4 items
-    // per warp balances the warps best, fewer save the items' partial sums
-    int bt = 1;
-    while (bt < kMaxTile && bt < B) bt *= 2;
-    SmemPlan sp{};
-    int piece = 0;
-    for (bool fits = false; !fits; bt /= 2) {
-        if (bt == 0) return cudaErrorNotSupported;
-        const int S = kMaxTile / bt;
-        const bool tma = tma_ok && bt >= 4;
-        if (tma) {
-            box_rows(xrows, 32 / bt, nbx, bxh);
-            box_rows(H, 32 / bt, nbh, bhh);
+    a.irows = pre ? 0 : (I + 3) / 4 * 4;
+    a.hrows = (H + 3) / 4 * 4;
+    const int in_rows = a.irows + a.hrows + 1;
+    const int cmax = std::min({sm_count(), H, kMaxCtas});
+    // The tile widths and the group counts, by the time a step is expected to
+    // take: per tile a fixed part (barrier, cell, latencies: 2.5 us), the
+    // staging of in_rows rows and the gather of the CTA's kept weights.  A
+    // narrow tile stages less but keeps more weights a CTA, each of which
+    // costs its own share of a load, and a quarter-warp's staged rows then
+    // share banks (cycles per weight: measured on the gate matrices of
+    // 4096 x 1280 fp32 and 6000 x 3000 bf16).
+    Shape shapes[(kMaxLbt + 1) * 80];
+    int nshapes = 0;
+    for (int lbt = 0; lbt <= kMaxLbt && (lbt == 0 || (1 << (lbt - 1)) < B); ++lbt) {
+        const int bt = 1 << lbt;
+        const int64_t nt = (B + bt - 1) / bt;
+        static const double kCycles[kMaxLbt + 1] = {0.6, 0.75, 0.85, 1.1, 1.5, 1.9};
+        int64_t last = -1;
+        for (int64_t tpg = 1; tpg <= nt; tpg = tpg < 8 ? tpg + 1 : tpg * 2) {
+            const int64_t ng = (nt + tpg - 1) / tpg;
+            if (ng > cmax || ng == last) continue;
+            last = ng;
+            const int members = std::min<int>(std::max(1, sm_count() / static_cast<int>(ng)), std::min(H, kMaxCtas));
+            const double mine = double(total) / members;
+            const double tile = 2500.0 + double(in_rows) * bt * 4 / 150.0 + mine * kCycles[lbt] / 1.9;
+            shapes[nshapes++] = {lbt, static_cast<int>(ng), static_cast<int>((nt + ng - 1) / ng),
+                                 double((nt + ng - 1) / ng) * tile};
         }
-        const int in_rows = tma ? nbx * bxh + nbh * bhh + 1 : xrows + H + 1;
-        for (int ipw = 4; ipw >= 1 && !fits; ipw /= 2) {
-            piece = round4(static_cast<int>(
-                std::max<int64_t>(8 * S, (kept_cap + ipw * kSeqWarps - 1) / (ipw * kSeqWarps))));
+        if (last != 1) shapes[nshapes++] = {lbt, 1, static_cast<int>(nt), 1e18 / bt};   // always a candidate
+    }
+    std::sort(shapes, shapes + nshapes, [](const Shape &p, const Shape &q) { return p.ns < q.ns; });
+    Ranges rg{};
+    SmemPlan sp{};
+    Shape s{};
+    int members = 0;
+    bool fits = false;
+    for (int i = 0; i < nshapes && !fits; ++i) {
+        s = shapes[i];
+        const int bt = 1 << s.lbt;
+        members = std::max(1, std::min({sm_count() / s.ngroups, H, kMaxCtas}));
+        int64_t kept_cap = 0;
+        int units_cap = 0;
+        split_units(kept, members, rg, kept_cap, units_cap);
+        if (kept_cap > (int64_t(1) << 20)) continue;
+        const bool c_on_chip = !kGru && size_t(units_cap) * size_t(s.tpg) * bt * 4 <= kCellOnChip;
+        // work items: rows longer than a warp's share of the CTA's weights are
+        // cut (at least 2 loads per subgroup), or none where their partial sums
+        // do not fit.  Items handed out longest first balance the warps: four
+        // times as many, in row order, took 7.8 us against 6.5 a step on
+        // 4096 x 1280 fp32 at batch 32
+        const int S = bt < 4 ? 32 : 128 / bt, KW = S <= 4 ? 4 : S <= 8 ? 2 : 1;
+        for (int cut = 1; cut >= 0 && !fits; --cut) {
+            a.piece = round4(static_cast<int>(
+                cut ? std::max<int64_t>(2 * KW * S, (kept_cap + kSeqWarps - 1) / kSeqWarps) : kept_cap));
             int items_cap = 0;
-            for (int q = 0; q < G; ++q) {
+            for (int q = 0; q < members; ++q) {
                 int items = 0;
                 for (int g = 0; g < kGates; ++g)
                     for (int u = rg.start[q]; u < rg.start[q + 1]; ++u)
-                        items += static_cast<int>((row_kept(int64_t(g) * H + u) + piece - 1) / piece);
+                        items += static_cast<int>((row_kept(int64_t(g) * H + u) + a.piece - 1) / a.piece);
                 items_cap = std::max(items_cap, items);
             }
-            sp = smem_plan(kept_cap, kGates * units_cap, items_cap, units_cap, BF16, kGru && !pre, in_rows, bt, B,
+            sp = smem_plan(kept_cap, kGates * units_cap, items_cap, units_cap, BF16, kGru && !pre, in_rows, bt, s.tpg,
                            c_on_chip, pre);
             fits = sp.total <= kSmemCap;
         }
-        if (fits) break;
+        a.c_on_chip = c_on_chip ? 1 : 0;
     }
-    a.piece = piece;
-    a.c_on_chip = c_on_chip ? 1 : 0;
+    if (!fits) return cudaErrorNotSupported;
+    const int bt = 1 << s.lbt;
+    a.ngroups = s.ngroups;
+    a.tpg = s.tpg;
+    a.ntiles = static_cast<int>((B + bt - 1) / bt);
     a.c_last = c_last;
-    a.lbt = 0;
-    while ((1 << a.lbt) < bt) ++a.lbt;
-    a.tma = tma_ok && bt >= 4 ? 1 : 0;
-    if (a.tma) {
-        a.nbx = nbx;
-        a.bxh = bxh;
-        a.nbh = nbh;
-        a.bhh = bhh;
-        a.ipad = nbx * bxh;
-        a.hpad = nbh * bhh;
-        a.tile_bytes = static_cast<uint32_t>((a.ipad + a.hpad) * bt * 4);
-    } else {
-        a.ipad = xrows;
-        a.hpad = H;
-    }
-    a.stage_mode = kStageScalar;
-    if (ptrs && B % 4 == 0 && bt % 4 == 0) a.stage_mode = kStageQuadCols;
-    else if (ptrs && B == 1 && xrows % 4 == 0 && H % 4 == 0) a.stage_mode = kStageQuadRows;
-    const cudaError_t attr = allow_smem(seq_kernel<BF16, MODE>, kSmemCap);
+    const auto kernel = seq_entry<BF16, MODE>(s.lbt);
+    const cudaError_t attr = allow_smem(kernel, kSmemCap);
     if (attr != cudaSuccess) return attr;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(G));
+    cfg.gridDim = dim3(static_cast<unsigned>(members * s.ngroups));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = sp.total;
     cfg.stream = stream;
@@ -715,63 +831,46 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     a.barrier_ns = kWaitLimitNs;
     a.skip_cta = -1;
     sequence_test_hook(&a.barrier_ns, &a.skip_cta);
-    // workspace: barrier word and abort flag; the cell state when it is neither
-    // on chip nor in c_last; the x parts and the product input they come from;
-    // the padded copy of h_t
-    const size_t cbytes = kGru || c_on_chip || c_last ? 0 : up(size_t(H) * size_t(B) * 4);
-    const int64_t ldp = (B + bt - 1) / bt * bt;
-    const size_t pbytes = a.tma && ldp != B && T > 1 ? up(2 * size_t(H) * size_t(ldp) * 4) : 0;
-    const size_t ws_bytes = 256 + cbytes + (pre ? pre_bytes : 0) + pbytes;
+    // x_t is read in place when its rows are already tile-major; else from a
+    // tile-major copy, or by plain loads where that copy would be too large
+    const bool x_in_place = I % 4 == 0 && B == bt && reinterpret_cast<uintptr_t>(a.x) % 16 == 0;
+    const size_t xt_bytes = size_t(T) * size_t(a.ntiles) * size_t(a.irows) * bt * 4;
+    a.x_mode = pre || I == 0 ? kXNone : x_in_place || xt_bytes <= (size_t(1) << 30) ? kXBulk : kXPlain;
+    // workspace: barrier counters and abort flag; the cell state when it is
+    // neither on chip nor in c_last; the exchanged h; the x parts and the
+    // product input they come from, or the tile-major copy of x
+    const int nwords = (a.ngroups + 1) * kBarWords;
+    const size_t bar_bytes = up(size_t(nwords) * 4);
+    const size_t cbytes = kGru || a.c_on_chip || c_last ? 0 : up(size_t(H) * size_t(B) * 4);
+    const size_t hx_bytes = up(2 * size_t(a.ntiles) * size_t(a.hrows) * bt * 4);
+    const bool x_copy = a.x_mode == kXBulk && !x_in_place;
+    const size_t ws_bytes = bar_bytes + cbytes + hx_bytes + (pre ? pre_bytes : 0) + (x_copy ? up(xt_bytes) : 0);
     char *ws = nullptr;
     cudaError_t e = stream_alloc(reinterpret_cast<void **>(&ws), ws_bytes, stream);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(ws, 0, 16, stream);
     a.bar = reinterpret_cast<unsigned *>(ws);
-    a.abort_flag = reinterpret_cast<int *>(ws + 4);
-    a.c_state = kGru || c_on_chip ? nullptr : (c_last ? c_last : reinterpret_cast<float *>(ws + 256));
-    a.h_pad = pbytes ? reinterpret_cast<float *>(ws + ws_bytes - pbytes) : nullptr;
-    a.ldp = ldp;
-    if (pre && e == cudaSuccess) {
-        float *xall = reinterpret_cast<float *>(ws + 256 + cbytes);
-        float *gx = reinterpret_cast<float *>(ws + 256 + cbytes + up(size_t(I + H) * ldx * 4));
-        e = cudaMemsetAsync(xall + size_t(I) * ldx, 0, size_t(H) * ldx * 4, stream);
+    a.abort_flag = reinterpret_cast<int *>(ws + size_t(a.ngroups) * kBarWords * 4);
+    a.c_state = kGru || a.c_on_chip ? nullptr : (c_last ? c_last : reinterpret_cast<float *>(ws + bar_bytes));
+    a.h_x = reinterpret_cast<float *>(ws + bar_bytes + cbytes);
+    float *const xws = reinterpret_cast<float *>(ws + bar_bytes + cbytes + hx_bytes);
+    a.x_tiles = a.x_mode != kXBulk ? nullptr : x_in_place ? a.x : xws;
+    const int64_t warps = H + (pre || x_copy ? T * I : 0);
+    const unsigned grid = static_cast<unsigned>(std::min<int64_t>((warps + 7) / 8, int64_t(sm_count()) * 16));
+    prep_kernel<<<grid, 256, 0, stream>>>(a, s.lbt, h0, x_copy ? xws : nullptr, pre ? xws : nullptr, ldx, nwords);
+    e = cudaGetLastError();
+    if (pre) {
+        float *gx = reinterpret_cast<float *>(reinterpret_cast<char *>(xws) + up(size_t(I + H) * ldx * 4));
         if (e == cudaSuccess) {
-            const int64_t warps = T * I;
-            const unsigned grid = static_cast<unsigned>(std::min<int64_t>((warps + 7) / 8, int64_t(sm_count()) * 16));
-            gather_x_kernel<<<grid, 256, 0, stream>>>(a.x, a.T, I, B, xall, ldx);
-            e = cudaGetLastError();
+            e = launch_spmm_prefix(f, I, xws, ldx, T * B, gx, ldx, false, stream);
+            if (e == cudaErrorNotSupported) {   // the whole product then: the rows of h are zero
+                e = cudaMemsetAsync(xws + size_t(I) * ldx, 0, size_t(H) * ldx * 4, stream);
+                if (e == cudaSuccess) e = launch_spmm(f, xws, ldx, T * B, gx, ldx, false, DARB_PATH_AUTO, stream);
+            }
         }
-        // only the x columns: xall's h rows are zero
-        if (e == cudaSuccess) e = launch_spmm_prefix(f, I, xall, ldx, T * B, gx, ldx, false, stream);
         a.gx = gx;
         a.ldgx = ldx;
     }
-    // tensor maps of the staged sources: 3-D (batch, rows, step) so that a box
-    // running past the last row of a step reads zeros, never the next step;
-    // h_{t-1} from the padded copy when the last batch tile is ragged
-    CUtensorMap mx{}, mh0{}, mhs{};
-    if (a.tma && e == cudaSuccess) {
-        auto make = [&](CUtensorMap *m, const float *base, int64_t cols, int64_t rows, int64_t depth, int boxh) {
-            const cuuint64_t dims[3] = {cuuint64_t(cols), cuuint64_t(rows), cuuint64_t(depth)};
-            const cuuint64_t strides[2] = {cuuint64_t(cols) * 4, cuuint64_t(cols) * 4 * cuuint64_t(rows)};
-            const cuuint32_t box[3] = {cuuint32_t(bt), cuuint32_t(boxh), 1};
-            const cuuint32_t es[3] = {1, 1, 1};
-            return tensor_map_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims,
-                                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-        };
-        bool ok = make(&mh0, a.h0, B, H, 1, bhh) &&
-                  (a.h_pad ? make(&mhs, a.h_pad, a.ldp, H, 2, bhh) : make(&mhs, a.h_seq, B, H, T, bhh));
-        if (ok && nbx) ok = make(&mx, a.x, B, I, T, bxh);
-        if (!ok) {   // plain loads instead (the plan above has room for either)
-            a.tma = 0;
-            a.ipad = xrows;
-            a.hpad = H;
-            a.h_pad = nullptr;
-        }
-    }
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, seq_kernel<BF16, MODE>, f, a, rg, sp, mx, mh0, mhs);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kernel, f, a, rg, sp);
     const cudaError_t ef = cudaFreeAsync(ws, stream);
     return e != cudaSuccess ? e : ef;
 }
@@ -785,14 +884,13 @@ cudaError_t launch_lstm_sequence(const Format &f, const int32_t *row_m, int64_t 
     a.T = static_cast<int>(T);
     a.B = B;
     a.x = x;
-    a.h0 = h0;
     a.c0 = c0;
     a.bias = bias;
     a.h_seq = h_seq;
     a.c_seq = c_seq;
     a.status = f.status;
-    return f.bf16 ? launch_seq_t<true, kModeLstm>(f, row_m, a, c_last, stream)
-                  : launch_seq_t<false, kModeLstm>(f, row_m, a, c_last, stream);
+    return f.bf16 ? launch_seq_t<true, kModeLstm>(f, row_m, a, h0, c_last, stream)
+                  : launch_seq_t<false, kModeLstm>(f, row_m, a, h0, c_last, stream);
 }
 
 cudaError_t launch_gru_sequence(const Format &f, const int32_t *row_m, int64_t T, int64_t I, int64_t H, int64_t B,
@@ -804,13 +902,12 @@ cudaError_t launch_gru_sequence(const Format &f, const int32_t *row_m, int64_t T
     a.T = static_cast<int>(T);
     a.B = B;
     a.x = x;
-    a.h0 = h0;
     a.b_ih = b_ih;
     a.b_hh = b_hh;
     a.h_seq = h_seq;
     a.status = f.status;
-    return f.bf16 ? launch_seq_t<true, kModeGru>(f, row_m, a, nullptr, stream)
-                  : launch_seq_t<false, kModeGru>(f, row_m, a, nullptr, stream);
+    return f.bf16 ? launch_seq_t<true, kModeGru>(f, row_m, a, h0, nullptr, stream)
+                  : launch_seq_t<false, kModeGru>(f, row_m, a, h0, nullptr, stream);
 }
 
 }  // namespace darb

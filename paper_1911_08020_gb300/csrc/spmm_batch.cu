@@ -33,10 +33,10 @@ cudaError_t launch_spmm_prefix(const Format &f, int64_t col_limit, const float *
         fx.cols = col_limit;
         const cudaError_t e = f.bf16 ? xres::launch<true, 32>(fx, X, ldx, batch, Y, ldy, early, stream)
                                      : xres::launch<false, 32>(fx, X, ldx, batch, Y, ldy, early, stream);
-        if (e != cudaErrorNotSupported) return e;
-        cudaGetLastError();
+        if (e == cudaErrorNotSupported) cudaGetLastError();
+        return e;
     }
-    return launch_spmm(f, X, ldx, batch, Y, ldy, early, DARB_PATH_AUTO, stream);
+    return cudaErrorNotSupported;
 }
 
 }  // namespace darb

@@ -70,9 +70,7 @@ def _check_gru_sequence(h, ref, T, I, H, B, xs, h0, bi, bh, tol):
 
 
 # (I, H, B): one unit per CTA, ragged batch tiles, several tiles, I = 0, more
-# units than CTAs, a batch tile of one column; batches that are multiples of 4
-# stage through tensor maps (one CTA; a ragged last tile staged from the padded
-# copy of h, as one tile (B = 12) and as the second of two (B = 40))
+# units than CTAs, a batch tile of one column, ragged last tiles (B = 12, 40)
 SHAPES = [(0, 5, 1), (3, 4, 2), (7, 33, 3), (20, 40, 8), (64, 100, 9), (10, 70, 33), (16, 300, 1),
           (40, 200, 70), (5, 400, 17), (4, 1, 8), (6, 9, 4), (12, 36, 40), (0, 64, 12), (300, 260, 4)]
 
@@ -234,6 +232,61 @@ def test_sequence_deterministic_and_graph_capturable():
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(hs, outs[0])
+    finally:
+        darb.darb_destroy(h)
+
+
+# (cell, I, H, B): batches of several column groups; more tiles than a group
+# each (fewer units than tiles: a group runs several); x_t staged in place (a
+# whole tile) and from its tile-major copy, precomputed x parts on a ragged
+# last tile
+GROUPS = [("lstm", 16, 64, 32), ("lstm", 6, 500, 33), ("gru", 20, 700, 64), ("gru", 3, 2, 70), ("lstm", 0, 1, 40),
+          ("gru", 300, 200, 21), ("lstm", 7, 3, 129), ("gru", 8, 90, 2)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("cell,I,H,B", GROUPS)
+def test_sequence_column_groups(cell, I, H, B, dtype):
+    g = np.random.default_rng(46)
+    T = 4
+    gates = 4 if cell == "lstm" else 3
+    stored, m = _gate_matrix(g, gates, I, H, dtype, (1, 3, 8, 16))
+    h, ref = encode_both(stored, m, dtype)
+    try:
+        xs = synth.activations(T * max(I, 1), B, seed=8).reshape(T, max(I, 1), B)[:, :I].copy()
+        h0, c0 = synth.state(H, B, seed=9), synth.state(H, B, seed=10)
+        b1, b2 = synth.bias(gates * H, seed=1), synth.bias(gates * H, seed=2)
+        if cell == "lstm":
+            _check_lstm_sequence(h, ref, T, I, H, B, xs, h0, c0, b1, TOL[dtype])
+        else:
+            _check_gru_sequence(h, ref, T, I, H, B, xs, h0, b1, b2, TOL[dtype])
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
+def test_sequence_with_x_too_large_to_copy():
+    """Past 1 GiB x_t is neither precomputed nor copied to tile-major rows but
+    read in place; two calls of half the steps precompute.  A gate sum has 196
+    terms |w x| of some 0.14 * 0.8 (the largest of 256 weights): two orders of
+    fp32 addition differ by at most 196 * 2^-23 * 196 * 0.12 < 6e-4, and the
+    gates contract."""
+    g = np.random.default_rng(47)
+    I, H, B, T = 50000, 4, 14, 400
+    w = torch.from_numpy((0.05 * g.standard_normal((4 * H, I + H))).astype(np.float32)).to(dev())
+    h = darb.darb_encode(w, np.full(4 * H, 256, np.int32))
+    try:
+        xs = torch.randn((T, I, B), device=dev(), generator=torch.Generator(device=dev()).manual_seed(3))
+        z = torch.zeros((H, B), device=dev())
+        hs, cl = torch.empty((T, H, B), device=dev()), torch.empty((H, B), device=dev())
+        darb.darb_lstm_sequence(h, T, I, H, B, xs, z, z, None, hs, None, cl)
+        hs2, c1, c2 = torch.empty_like(hs), torch.empty_like(cl), torch.empty_like(cl)
+        half = T // 2
+        darb.darb_lstm_sequence(h, half, I, H, B, xs[:half], z, z, None, hs2[:half], None, c1)
+        darb.darb_lstm_sequence(h, half, I, H, B, xs[half:], hs2[half - 1].clone(), c1, None, hs2[half:], None, c2)
+        darb.darb_sync_status(h)
+        assert torch.max(torch.abs(hs - hs2)).item() < 6e-4
+        assert torch.max(torch.abs(cl - c2)).item() < 2e-3
     finally:
         darb.darb_destroy(h)
 
