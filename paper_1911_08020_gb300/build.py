@@ -22,7 +22,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdarb.so")
 BASE_LIB = os.path.join(PKG, "libdarb_baselines.so")
 BASE_SOURCES = ["baselines.cu"]
-SOURCES = ["darb_api.cu", "assign.cu", "encode.cu", "spmm.cu", "spmm_batch.cu", "spmm_tc.cu", "rnn.cu", "rnn_batch.cu",
+SOURCES = ["darb_api.cu", "assign.cu", "encode.cu", "spmm.cu", "spmm_batch.cu", "spmm_tc.cu", "rnn.cu", "rnn_batch.cu", "rnn_step.cu",
            "noalloc.cu", "sequence.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

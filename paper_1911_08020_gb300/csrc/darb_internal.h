@@ -201,6 +201,10 @@ struct RnnArgs;
 // Batch > 4 RNN steps (rnn_batch.cu); mode is kModeLstm or kModeGru.
 cudaError_t launch_rnn_batch(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream);
 
+// The same with the cell local to the CTA of a unit (rnn_step.cu);
+// cudaErrorNotSupported when the call does not fit it.
+cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream);
+
 // Batch-tile width the RNN step kernels use for a batch of B (sizes the counters).
 int rnn_batch_tile(int64_t B);
 

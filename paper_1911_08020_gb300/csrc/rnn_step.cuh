@@ -1,0 +1,458 @@
+// rnn_step.cuh -- one LSTM or GRU cell step with the cell local
+// to the CTA that owns a hidden unit (Sec. 3.2, Fig. 6(b) on the stacked input
+// [x_t; h_{t-1}], then the cell of Sec. 4.1).
+//
+// The batch columns are cut into tiles of bt columns, and the CTAs into one
+// group a tile; within a group every CTA owns a contiguous range of hidden
+// units with all their gate rows, so no gate sum leaves its CTA: no cluster,
+// no scratch, no counters.  A CTA
+//  * reads its rows' places in the format and, when the handle is complete,
+//    starts on their first records before the PDL wait;
+//  * stages the tile's columns of x_t and h_{t-1} whole (tensor-map boxes, or
+//    16- or 4-byte asynchronous copies), with its units' c_{t-1} and biases;
+//  * multiplies: bt / 4 lanes share a kept weight, 4 columns each (a 16-byte
+//    load of the staged row the weight selects).  The chunks of the CTA's rows
+//    form one stream that the 16 * 128 / bt lane groups share out evenly, a
+//    contiguous run each, so that rows of any length balance; the records come
+//    straight from L2, two chunks ahead of their use;
+//  * adds the runs' partial sums of each row in order (deterministic) and
+//    applies the cell.
+// A GRU row is two rows of the stream, its x part and its h part (r multiplies
+// only the h part of the candidate); a chunk that holds columns of both sides
+// of I, or runs past the row's last block, is in each with the other side's
+// weights as zeros on a zero row.
+//
+// What bounds it: the latency of its phases (staging, gather, cell; 3 to 4 us
+// with the launch) and, for wide matrices, the gather.  A step (us, in a graph
+// of steps) against the kernels whose gate sums meet through clusters, scratch
+// and counters (rowlane_kernel, batch_kernel): LSTM 4096 x 1280 fp32 at batch
+// 1 / 8 / 32 / 64: 6.2 / 5.9 / 7.8 / 11.1 against 7.8 / 17.0 / 25.0 / 30.3; GRU
+// 3072 x 2048 bf16 at batch 64: 11.5 against 32.3; LSTM 6000 x 3000 bf16 at
+// batch 20: 16.5 against 37.9, fp32 at batch 37: 30 against 212.  Those kernels
+// remain for inputs too tall to stage at 4 columns (some 14000 rows).
+#pragma once
+
+#include "kernels_common.cuh"
+#include "launch.cuh"
+#include "rnn_epilogue.cuh"
+#include "tma.cuh"
+
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cstring>
+
+namespace darb {
+namespace step {
+
+constexpr int kThreads = 512;
+constexpr int kStepWarps = kThreads / 32;
+constexpr size_t kSmemCap = 227 * 1024 - 256;   // dynamic shared memory, with room for the static part
+constexpr int kMinLbt = 2, kMaxLbt = 5;         // batch tiles of 4, 8, 16 or 32 columns
+constexpr int kAhead = 2;                       // chunks a lane group has requested ahead of its use
+
+// A row (GRU: a side of a row) of a CTA's stream of chunks.
+struct Row {
+    uint32_t rec, off;   // value record (8 values) and offset word of its chunk 0
+    int c0;              // first chunk in the stream
+    int m_nib;           // block size | 4-bit offsets << 16
+    int klo, khi;        // its columns [klo, khi)
+    int at;              // position of chunk c0 in the stream
+    int seg;             // partial sums: first index
+};
+
+constexpr int kStage4 = 0, kStage16 = 1, kStageBoxes = 2;
+
+struct Plan {
+    int ntiles, members;          // CTA i is CTA i / ntiles of tile i % ntiles
+    int staging, early;           // kStage*; the records may be read before the PDL wait
+    int nbx, bxh, nbh, bhh;       // boxes of x and h: their number and rows (the last one ends with the matrix)
+    uint32_t row_off, nseg_off, bias_off, c_off, in_off, part_off;
+};
+
+template <bool BF16, int MODE, int LBT>
+__global__ void __launch_bounds__(kThreads, 1)
+step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mh,
+            Plan p) {
+    constexpr int kGates = MODE == kModeLstm ? 4 : 3;
+    constexpr bool kGru = MODE == kModeGru;
+    constexpr int kSides = kGru ? 2 : 1;
+    constexpr int bt = 1 << LBT, L = bt / 4, S = 32 / L, kSubs = kStepWarps * S;
+    constexpr int kRowShift = LBT + 2;   // log2 of the bytes of a staged row
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ __align__(8) uint64_t s_full;
+    __shared__ int s_total;
+    Row *s_row = reinterpret_cast<Row *>(sm + p.row_off);      // [VR + 1]
+    int *s_nseg = reinterpret_cast<int *>(sm + p.nseg_off);    // [VR]
+    float *s_bias = reinterpret_cast<float *>(sm + p.bias_off);   // [VR]: GRU b_ih then b_hh
+    float *s_c = reinterpret_cast<float *>(sm + p.c_off);      // [units][bt]: c_{t-1} (LSTM)
+    float *s_in = reinterpret_cast<float *>(sm + p.in_off);    // [K + 1][bt], row K zero
+    float *s_part = reinterpret_cast<float *>(sm + p.part_off);   // [VR + kSubs][bt]
+
+    pdl_launch_dependents();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tile = int(blockIdx.x) % p.ntiles, member = int(blockIdx.x) / p.ntiles;
+    const int H = ra.H, I = ra.I, K = I + H;
+    const int64_t B = ra.B, b0 = int64_t(tile) << LBT;
+    const int nb = static_cast<int>(B - b0 < bt ? B - b0 : bt);
+    const int u0 = static_cast<int>(int64_t(H) * member / p.members);
+    const int nu = static_cast<int>(int64_t(H) * (member + 1) / p.members) - u0;
+    const int R = kGates * nu, VR = kSides * R;   // local row q*nu + i is matrix row q*H + u0 + i
+    auto grow = [&](int lr) { return (lr / nu) * H + u0 + lr % nu; };
+
+    // ---- the rows' places in the format (immutable: before the PDL wait)
+    for (int v = tid; v < VR; v += kThreads) {
+        const int lr = v < R ? v : v - R;
+        const int loc = f.rowloc[grow(lr)];
+        const Group g = f.groups[loc / kSlots];
+        const int slot = loc % kSlots;
+        const bool xside = kGru && v < R, hside = kGru && v >= R;
+        const int nch = (g.n + kChunk - 1) / kChunk, span = kChunk * g.m;
+        Row r;
+        r.rec = static_cast<uint32_t>(g.val_off / kChunk) + slot;
+        r.off = static_cast<uint32_t>(g.off_off) + slot * (g.nib ? 1 : 2);
+        r.m_nib = g.m | (g.nib ? 1 << 16 : 0);
+        r.klo = hside ? I : 0;
+        r.khi = xside ? I : K;
+        r.c0 = hside ? min(nch, I / span) : 0;
+        const int c1 = xside ? min(nch, (I + span - 1) / span) : nch;
+        r.at = c1 > r.c0 ? c1 - r.c0 : 0;   // its chunks, until the scan below
+        r.seg = 0;
+        s_row[v] = r;
+    }
+    for (int j = tid; j < bt; j += kThreads) s_in[(K << LBT) + j] = 0.0f;
+    if (tid == 0) {
+        mbar_init(&s_full, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (warp == 0) {   // where each row's chunks start in the stream
+        int base = 0;
+        for (int v0 = 0; v0 < VR; v0 += 32) {
+            const int n = v0 + lane < VR ? s_row[v0 + lane].at : 0;
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= o) incl += up;
+            }
+            if (v0 + lane < VR) s_row[v0 + lane].at = base + incl - n;
+            base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        }
+        if (lane == 0) {
+            s_row[VR].at = base;
+            s_total = base;
+        }
+    }
+    __syncthreads();
+    const int total = s_total;
+    const int N = max(1, (total + kSubs - 1) / kSubs);   // chunks of a lane group
+    // the lane groups that share a row are consecutive, and group + row is
+    // different for every (group, row) that meet: the index of a partial sum
+    for (int v = tid; v < VR; v += kThreads) {
+        const int a = s_row[v].at, b = s_row[v + 1].at;
+        s_row[v].seg = a / N + v;
+        s_nseg[v] = b > a ? (b - 1) / N - a / N + 1 : 0;
+    }
+
+    // ---- this lane group's run of chunks, [pos, end)
+    const int sub = warp * S + lane / L;
+    const uint32_t xl = smem_addr(s_in) + uint32_t(lane % L) * 16u;
+    const int pos = min(total, sub * N), end = min(total, pos + N);
+    constexpr int kW = BF16 ? 4 : 8;
+    struct Fetch {
+        uint32_t vw[kW];
+        uint2 ow;
+        int v, c;   // row of the stream (-1: none) and chunk
+    };
+    Fetch buf[kAhead];
+    int lv = 0;     // row of the next chunk to request
+    if (pos < end) {
+        int hi = VR;   // the last row that starts at or before pos
+        while (hi - lv > 1) {
+            const int mid = (lv + hi) / 2;
+            if (s_row[mid].at <= pos) lv = mid;
+            else hi = mid;
+        }
+    }
+    auto fetch = [&](int i, Fetch &b) {   // chunk i of the stream
+        b.v = -1;
+        if (i >= end) return;
+        while (s_row[lv + 1].at <= i) ++lv;
+        const uint4 *rw = reinterpret_cast<const uint4 *>(s_row + lv);
+        const uint4 q = rw[0];
+        const int at = s_row[lv].at;
+        const int c = int(q.z) + i - at;
+        const bool nib = q.w >> 16;
+        b.v = lv;
+        b.c = c;
+        const uint4 *pv = static_cast<const uint4 *>(f.vals) + int64_t(q.x + uint32_t(c) * kSlots) * (BF16 ? 1 : 2);
+        const uint4 w0 = __ldg(pv);
+        b.vw[0] = w0.x; b.vw[1] = w0.y; b.vw[2] = w0.z; b.vw[3] = w0.w;
+        if constexpr (!BF16) {
+            const uint4 w1 = __ldg(pv + 1);
+            b.vw[4] = w1.x; b.vw[5] = w1.y; b.vw[6] = w1.z; b.vw[7] = w1.w;
+        }
+        if (nib) {
+            const uint32_t w = __ldg(f.offs + q.y + uint32_t(c) * kSlots);
+            const uint32_t even = w & 0x0F0F0F0Fu, odd = (w >> 4) & 0x0F0F0F0Fu;
+            b.ow = make_uint2(__byte_perm(even, odd, 0x5140), __byte_perm(even, odd, 0x7362));
+        } else {
+            b.ow = __ldg(reinterpret_cast<const uint2 *>(f.offs + q.y + uint32_t(c) * (2 * kSlots)));
+        }
+    };
+    if (p.early) {
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) fetch(pos + i, buf[i]);
+    }
+
+    // ---- the inputs
+    pdl_wait_previous();
+    if (LBT == 5 && p.staging == kStageBoxes) {
+        if (warp == 0) {
+            if (lane == 0) mbar_arrive_expect_tx(&s_full, uint32_t(p.nbx * p.bxh + p.nbh * p.bhh) << kRowShift);
+            __syncwarp();
+            for (int i = lane; i < p.nbx + p.nbh; i += 32) {
+                const bool isx = i < p.nbx;
+                const int rows = isx ? I : H, bh = isx ? p.bxh : p.bhh;
+                const int y = min((isx ? i : i - p.nbx) * bh, rows - bh);
+                tensor2d_g2s(s_in + (int64_t((isx ? 0 : I) + y) << LBT), isx ? &mx : &mh, int(b0), y, &s_full);
+            }
+        }
+    } else if (p.staging == kStage16) {
+        constexpr int Q = bt / 4, kStep = kThreads / Q;
+        const int j = (tid & (Q - 1)) * 4;
+        const bool in = j < nb;   // B is a multiple of 4
+        uint32_t dst = smem_addr(s_in) + uint32_t(tid) * 16u;
+        const float *const sx = ra.x + b0 + (in ? j : 0), *const sh = ra.h + b0 + (in ? j : 0);
+#pragma unroll 4
+        for (int k = tid / Q; k < K; k += kStep, dst += kThreads * 16)
+            cp_async16(dst, k < I ? sx + int64_t(k) * B : sh + int64_t(k - I) * B, in);
+    } else {
+        constexpr int kStep = kThreads >> LBT;
+        const int j = tid & (bt - 1);
+        const bool in = j < nb;
+        uint32_t dst = smem_addr(s_in) + uint32_t(tid) * 4u;
+        const float *const sx = ra.x + b0 + (in ? j : 0), *const sh = ra.h + b0 + (in ? j : 0);
+#pragma unroll 4
+        for (int k = tid >> LBT; k < K; k += kStep, dst += kThreads * 4)
+            cp_async4(dst, k < I ? sx + int64_t(k) * B : sh + int64_t(k - I) * B, in);
+    }
+    for (int v = tid; v < VR; v += kThreads) {
+        const float *b = kGru ? (v < R ? ra.b_ih : ra.b_hh) : ra.bias;
+        cp_async4(smem_addr(s_bias + v), b ? b + grow(v < R ? v : v - R) : ra.h, b != nullptr);
+    }
+    if constexpr (!kGru)
+        for (int i = tid; i < nu << LBT; i += kThreads) {
+            const int j = i & (bt - 1);
+            cp_async4(smem_addr(s_c + i), ra.c_prev + int64_t(u0 + (i >> LBT)) * B + b0 + (j < nb ? j : 0), j < nb);
+        }
+    if (!p.early) {
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) fetch(pos + i, buf[i]);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    if (LBT == 5 && p.staging == kStageBoxes && !mbar_wait(&s_full, 0)) {
+        atomicOr(f.status, kStatusTimeout);
+        mbar_wait(&s_full, 0);   // the boxes may still land: before this CTA can leave
+    }
+
+    // ---- the products
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    int cur = -1;   // row of the sums in acc
+    auto flush = [&]() {
+        if (cur >= 0) reinterpret_cast<float4 *>(s_part)[(cur + sub) * L + lane % L] = acc;
+    };
+    auto multiply = [&](const Fetch &b) {
+        if (b.v < 0) return;
+        if (b.v != cur) {
+            flush();
+            acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            cur = b.v;
+        }
+        const int m = s_row[b.v].m_nib & 0xFFFF, klo = s_row[b.v].klo, khi = s_row[b.v].khi;
+        const int kb = b.c * kChunk * m;
+        // a chunk's products are added by themselves first: the chain of fp32
+        // additions of a run stays short
+        float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+        auto weight = [&](int e) {
+            if constexpr (BF16)
+                return __uint_as_float((e & 1) ? (b.vw[e >> 1] & 0xFFFF0000u) : (b.vw[e >> 1] << 16));
+            else return __uint_as_float(b.vw[e]);
+        };
+        auto load = [&](uint32_t ad) {
+            float4 x;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(ad));
+            return x;
+        };
+        if (kb >= klo && kb + kChunk * m <= khi) {
+            const uint32_t xb = xl + (uint32_t(kb) << kRowShift), step = uint32_t(m) << kRowShift;
+            float4 x[kChunk];
+#pragma unroll
+            for (int e = 0; e < kChunk; ++e)
+                x[e] = load(xb + uint32_t(e) * step + (((e < 4 ? b.ow.x : b.ow.y) >> (8 * (e & 3)) & 255u) << kRowShift));
+#pragma unroll
+            for (int e = 0; e < kChunk; ++e) fma4((e & 1) ? s1 : s0, weight(e), x[e]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < kChunk; ++e) {
+                const int k = kb + e * m + int((e < 4 ? b.ow.x : b.ow.y) >> (8 * (e & 3)) & 255u);
+                const bool in = k >= klo && k < khi;
+                fma4((e & 1) ? s1 : s0, in ? weight(e) : 0.0f, load(xl + (uint32_t(in ? k : K) << kRowShift)));
+            }
+        }
+        acc.x += s0.x + s1.x;
+        acc.y += s0.y + s1.y;
+        acc.z += s0.z + s1.z;
+        acc.w += s0.w + s1.w;
+    };
+    for (int i = pos; i < end; i += kAhead) {
+#pragma unroll
+        for (int a = 0; a < kAhead; ++a) {
+            const Fetch now = buf[a];
+            fetch(i + a + kAhead, buf[a]);
+            multiply(now);
+        }
+    }
+    flush();
+    __syncthreads();
+
+    // ---- the cells of the owned units
+    auto sum = [&](int v, int j) {
+        float r = 0.0f;
+        const int seg = s_row[v].seg, n = s_nseg[v];
+        for (int i = 0; i < n; ++i) r += s_part[((seg + i) << LBT) + j];
+        return r;
+    };
+    for (int i = tid; i < nu << LBT; i += kThreads) {
+        const int ui = i >> LBT, j = i & (bt - 1);
+        if (j >= nb) continue;
+        const int64_t e = int64_t(u0 + ui) * B + b0 + j;
+        if constexpr (!kGru) {
+            float pre[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) pre[q] = sum(q * nu + ui, j) + s_bias[q * nu + ui];
+            const float c = sigm(pre[1]) * s_c[i] + sigm(pre[0]) * tanhf(pre[2]);
+            ra.c_out[e] = c;
+            ra.h_out[e] = sigm(pre[3]) * tanhf(c);
+        } else {
+            float ax[3], bh[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int v = q * nu + ui;
+                ax[q] = sum(v, j) + s_bias[v];
+                bh[q] = sum(R + v, j) + s_bias[R + v];
+            }
+            const float rr = sigm(ax[0] + bh[0]);
+            const float zz = sigm(ax[1] + bh[1]);
+            const float nn = tanhf(ax[2] + rr * bh[2]);
+            ra.h_out[e] = (1.0f - zz) * nn + zz * s_in[((I + u0 + ui) << LBT) + j];
+        }
+    }
+}
+
+// Boxes of at most 256 rows over n rows: their number and rows.  The last one
+// ends with the matrix and repeats rows of the one before.
+inline void boxes(int n, int *nbox, int *rows) {
+    *rows = std::min(n, 256);
+    *nbox = n > 0 ? (n + *rows - 1) / *rows : 0;
+}
+
+template <bool BF16, int MODE, int LBT>
+cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem, cudaStream_t stream) {
+    constexpr int bt = 1 << LBT;
+    const auto kernel = step_kernel<BF16, MODE, LBT>;
+    const cudaError_t attr = allow_smem(kernel, kSmemCap);
+    if (attr != cudaSuccess) return attr;
+    CUtensorMap mx, mh;
+    std::memset(&mx, 0, sizeof mx);
+    std::memset(&mh, 0, sizeof mh);
+    // How the inputs are staged: whole 32-column tiles in tensor-map boxes (LSTM
+    // 4096 x 1280 at batch 32: 7.8 us against 8.3 by 16-byte copies), other
+    // aligned rows in 16-byte copies (boxes of short or ragged rows are slower:
+    // batch 8 6.0 against 7.3 us, 6000 x 3000 at batch 20 17.5 against 21.6),
+    // the rest 4 bytes at a time
+    const bool aligned = ra.B % 4 == 0 && (ra.I == 0 || reinterpret_cast<uintptr_t>(ra.x) % 16 == 0) &&
+                         reinterpret_cast<uintptr_t>(ra.h) % 16 == 0;
+    p.staging = aligned ? kStage16 : kStage4;
+    if (LBT == 5 && aligned && ra.B % bt == 0 && tensor_map_encoder() != nullptr) {
+        auto make = [&](CUtensorMap *m, const float *base, int rows, int boxh) {
+            if (rows == 0) return true;
+            const cuuint64_t dims[2] = {cuuint64_t(ra.B), cuuint64_t(rows)};
+            const cuuint64_t strides[1] = {cuuint64_t(ra.B) * 4};
+            const cuuint32_t box[2] = {cuuint32_t(bt), cuuint32_t(boxh)};
+            const cuuint32_t es[2] = {1, 1};
+            return tensor_map_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims,
+                                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        };
+        boxes(ra.I, &p.nbx, &p.bxh);
+        boxes(ra.H, &p.nbh, &p.bhh);
+        if (make(&mx, ra.x, ra.I, p.bxh) && make(&mh, ra.h, ra.H, p.bhh)) p.staging = kStageBoxes;
+    }
+    return launch_ex(kernel, dim3(static_cast<unsigned>(p.ntiles * p.members)), dim3(kThreads), smem, stream, 1, true,
+                     f, ra, mx, mh, p);
+}
+
+// The step on this kernel, or cudaErrorNotSupported when the staged tile does
+// not fit beside the CTA's rows even at 4 columns.
+template <bool BF16, int MODE>
+cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream) {
+    constexpr int kGates = MODE == kModeLstm ? 4 : 3;
+    const int64_t K = int64_t(ra.I) + ra.H;
+    if (K > 60000 || ra.B > 1024 || f.nitems[0][0] <= 0) return cudaErrorNotSupported;
+    // kept weights of the matrix, padded to whole groups and chunks
+    const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
+    const int sms = sm_count();
+    int lbt = -1;
+    size_t smem = 0;
+    Plan best{};
+    double best_ns = 1e300;
+    for (int l = kMinLbt; l <= kMaxLbt && (l == kMinLbt || (1 << (l - 1)) < ra.B); ++l) {
+        const int bt = 1 << l;
+        Plan p{};
+        p.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
+        p.members = std::max(1, std::min(sms / p.ntiles, ra.H));
+        const int units = (ra.H + p.members - 1) / p.members;
+        const int vr = (MODE == kModeGru ? 2 : 1) * kGates * units, subs = kStepWarps * 128 / bt;
+        size_t o = 0;
+        auto take = [&](size_t bytes) {
+            const size_t at = o;
+            o = (o + bytes + 127) / 128 * 128;
+            return static_cast<uint32_t>(at);
+        };
+        if (vr > 4096) continue;
+        p.in_off = take(size_t(K + 1) * bt * 4);
+        p.part_off = take(size_t(vr + subs) * bt * 4);
+        p.row_off = take(size_t(vr + 1) * sizeof(Row));
+        p.nseg_off = take(size_t(vr) * 4);
+        p.bias_off = take(size_t(vr) * 4);
+        p.c_off = take(MODE == kModeLstm ? size_t(units) * bt * 4 : 0);
+        if (o > kSmemCap) continue;
+        // the staging of K rows (70 bytes/ns an SM) and the gather; a narrow
+        // tile stages less, but its staged rows share banks and each CTA
+        // multiplies more weights (cycles fitted to the shapes above)
+        static const double kCycles[kMaxLbt - kMinLbt + 1] = {0.9, 1.0, 1.35, 1.5};
+        const int waves = (p.ntiles * p.members + sms - 1) / sms;
+        const double ns = waves * (double(K) * bt * 4 / 70.0 + kept / p.members * kCycles[l - kMinLbt] / 1.9);
+        if (ns < best_ns) {
+            best_ns = ns;
+            best = p;
+            lbt = l;
+            smem = o;
+        }
+    }
+    if (lbt < 0) return cudaErrorNotSupported;
+    best.early = early ? 1 : 0;
+    return lbt == 2   ? launch_tile<BF16, MODE, 2>(f, ra, best, smem, stream)
+           : lbt == 3 ? launch_tile<BF16, MODE, 3>(f, ra, best, smem, stream)
+           : lbt == 4 ? launch_tile<BF16, MODE, 4>(f, ra, best, smem, stream)
+                      : launch_tile<BF16, MODE, 5>(f, ra, best, smem, stream);
+}
+
+}  // namespace step
+}  // namespace darb

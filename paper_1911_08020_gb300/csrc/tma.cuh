@@ -97,6 +97,11 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool va
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
 }
 
+// The same, 16 bytes (both addresses 16-byte aligned).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+
 // One of the arrivals `bar` was initialised with, made once this thread's
 // earlier cp_async4 copies have landed.
 __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {

@@ -1,0 +1,89 @@
+"""One LSTM / GRU cell step (darb_lstm_step, darb_gru_step) against the CPU oracle
+over the tile widths, stagings and row splits of the step kernel, and past the
+widest input it stages.  Bounds as for every step (gpu_helpers)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1911_08020_gb300 import darb, synth
+
+from .gpu_helpers import TOL, dev, encode_both, gru_bound, lstm_bounds, t
+
+pytestmark = pytest.mark.gpu
+
+
+def _buf(a, shift):
+    """Device copy of `a` whose base is `shift` floats past a 16-byte boundary."""
+    b = torch.empty(a.size + shift, device=dev())
+    v = b[shift:].view(a.shape)
+    v.copy_(torch.from_numpy(a))
+    return v
+
+
+# (I, H, B, block sizes, shift): tiles of 4 to 32 columns, whole, ragged and
+# several; rows shorter than a chunk and longer than a lane group's run; blocks
+# and chunks across I; no x; one unit; bases 4 bytes past a boundary; inputs too
+# tall for the kernel (15000 rows)
+SHAPES = [
+    (5, 7, 1, (1, 2, 3), 0), (33, 40, 3, (3, 8, 16), 0), (64, 200, 4, (4, 30), 0), (64, 200, 4, (4, 30), 1),
+    (0, 64, 8, (8, 64), 0), (100, 300, 7, (2, 10, 20), 0), (96, 160, 16, (4, 16, 40), 0), (50, 77, 13, (8, 256), 0),
+    (256, 300, 32, (4, 8, 32), 0), (300, 256, 32, (4, 8, 32), 1), (40, 500, 64, (8, 16), 0), (600, 30, 96, (5, 50), 0),
+    (31, 1, 33, (1, 7, 64), 0), (700, 900, 45, (10, 15, 30), 0), (15000, 4, 2, (16, 64), 0), (15000, 4, 6, (16, 64), 0),
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("cell", ["lstm", "gru"])
+@pytest.mark.parametrize("I,H,B,mset,shift", SHAPES)
+def test_step(cell, I, H, B, mset, shift, dtype):
+    g = np.random.default_rng(80)
+    gates = 4 if cell == "lstm" else 3
+    w = (0.3 * g.standard_normal((gates * H, I + H))).astype(np.float32)
+    stored = synth.f32_to_bf16_bits(w) if dtype == "bf16" else w
+    m = g.choice(np.asarray(mset, np.int32), size=gates * H)
+    h, ref = encode_both(stored, m, dtype)
+    try:
+        x = synth.activations(max(I, 1), B, seed=1)[:I].copy()
+        hp, cp = synth.state(H, B, seed=2), synth.state(H, B, seed=3)
+        b1, b2 = synth.bias(gates * H, seed=4), synth.bias(gates * H, seed=5)
+        xd = _buf(x, shift) if I else None
+        ho, co = torch.empty((H, B), device=dev()), torch.empty((H, B), device=dev())
+        Wd = t(stored.view(np.int16)).view(torch.bfloat16) if dtype == "bf16" else t(stored)
+        for _ in range(2):   # with the records read early, and right after a re-encode
+            if cell == "lstm":
+                darb.darb_lstm_step(h, I, H, B, xd, _buf(hp, shift), _buf(cp, shift), t(b1), ho, co)
+                hr, cr, ga = oracle.lstm_step(ref, I, H, x if I else None, hp, cp, b1)
+                bc, bh = lstm_bounds(ga, cp, TOL[dtype])
+                assert np.all(np.abs(co.cpu().numpy() - cr) <= bc)
+                assert np.all(np.abs(ho.cpu().numpy() - hr) <= bh)
+            else:
+                darb.darb_gru_step(h, I, H, B, xd, _buf(hp, shift), t(b1), t(b2), ho)
+                hr, ga = oracle.gru_step(ref, I, H, x if I else None, hp, b1, b2)
+                assert np.all(np.abs(ho.cpu().numpy() - hr) <= gru_bound(ga, hp, hr, TOL[dtype]))
+            ho.fill_(float("nan"))
+            co.fill_(float("nan"))
+            darb.darb_reencode(h, Wd)
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
+def test_gru_step_infinite_weight_in_a_block_across_the_boundary():
+    """Block [4, 8) of a row holds x columns 4, 5 and h columns 6, 7 (I = 6); an
+    infinite weight on one side must not meet the other side's zeros."""
+    I, H, B = 6, 6, 3
+    w = np.full((3 * H, I + H), 0.1, np.float32)
+    w[:, 4] = np.inf        # every row keeps column 4 of that block
+    m = np.full(3 * H, 4, np.int32)
+    h = darb.darb_encode(t(w), m)
+    try:
+        x, hp = np.ones((I, B), np.float32), np.full((H, B), 0.5, np.float32)
+        ho = torch.empty((H, B), device=dev())
+        darb.darb_gru_step(h, I, H, B, t(x), t(hp), None, None, ho)
+        # r = z = 1 (their sums are +inf), n = tanh(inf): h = (1 - 1) * 1 + 1 * h
+        np.testing.assert_array_equal(ho.cpu().numpy(), hp)
+    finally:
+        darb.darb_destroy(h)
