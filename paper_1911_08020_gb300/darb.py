@@ -44,6 +44,9 @@ class _Info(ctypes.Structure):
 def lib():
     """The loaded libdarb.so (raises if it has not been built)."""
     global _lib
+    L = _lib
+    if L is not None:
+        return L
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -92,16 +95,40 @@ def _check(status: int, call: str):
         raise DarbError(status, call)
 
 
+# The small calls of this module are bound by the host: a cell step runs 8 us on
+# the device.  So what every call does is kept cheap: torch is looked up once,
+# and the current stream's handle is read without building a Stream object
+# (0.2 us against 3.0).
+_torch = None
+_raw_stream = None
+
+
+def _load_torch():
+    global _torch, _raw_stream
+    import torch
+    get, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+    def raw():
+        if get is None or device is None or not torch.cuda.is_initialized():
+            return int(torch.cuda.current_stream().cuda_stream)
+        return get(device())
+
+    _raw_stream = raw
+    _torch = torch
+    return torch
+
+
 def _ptr(t) -> int | None:
     if t is None:
         return None
-    return int(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream) -> int | None:
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if _raw_stream is None:
+            _load_torch()
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return int(stream.cuda_stream)
@@ -117,10 +144,9 @@ def _dtype_code(t) -> int:
 
 
 def _require_cuda_f32(t, name):
-    import torch
     if t is None:
         return
-    if not t.is_cuda or t.dtype != torch.float32:
+    if not t.is_cuda or t.dtype != (_torch or _load_torch()).float32:
         raise DarbError(ERR_INVALID_ARG, f"{name} must be a CUDA float32 tensor")
 
 
@@ -207,22 +233,23 @@ def darb_spmm(h: Handle, X, Y=None, stream=None):
 
 def darb_spmm_ex(h: Handle, X, Y=None, path: int = PATH_AUTO, stream=None):
     """darb_spmm with the kernel family chosen (PATH_AUTO, PATH_CUDA_CORES, PATH_TENSOR_CORES)."""
-    import torch
     _require_cuda_f32(X, "X")
     if X.dim() == 1:
         X = X.view(-1, 1)
-    if X.stride(1) != 1 and X.shape[1] > 1:
+    shape, strides = X.shape, X.stride()
+    batch = shape[1]
+    if strides[1] != 1 and batch > 1:
         raise DarbError(ERR_INVALID_ARG, "darb_spmm: X must have a contiguous batch dimension")
-    batch = X.shape[1]
     if Y is None:
-        Y = torch.empty((h.rows, batch), dtype=torch.float32, device=X.device)
-    _require_cuda_f32(Y, "Y")
-    ldx = X.stride(0) if X.shape[0] > 1 else batch
+        Y = _torch.empty((h.rows, batch), dtype=_torch.float32, device=X.device)
+    else:
+        _require_cuda_f32(Y, "Y")
+    ldx = strides[0] if shape[0] > 1 else batch
     ldy = Y.stride(0) if Y.shape[0] > 1 else batch
     if path == PATH_AUTO:
-        _check(lib().darb_spmm(h.ptr, _ptr(X), ldx, batch, _ptr(Y), ldy, _stream(stream)), "darb_spmm")
+        _check(lib().darb_spmm(h.ptr, X.data_ptr(), ldx, batch, Y.data_ptr(), ldy, _stream(stream)), "darb_spmm")
     else:
-        _check(lib().darb_spmm_ex(h.ptr, _ptr(X), ldx, batch, _ptr(Y), ldy, int(path), _stream(stream)),
+        _check(lib().darb_spmm_ex(h.ptr, X.data_ptr(), ldx, batch, Y.data_ptr(), ldy, int(path), _stream(stream)),
                "darb_spmm_ex")
     return Y
 
