@@ -205,6 +205,11 @@ cudaError_t launch_rnn_batch(const Format &f, const RnnArgs &ra, int mode, bool 
 // cudaErrorNotSupported when the call does not fit it.
 cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream);
 
+// The product on the same kernel (rnn_step.cu); cudaErrorNotSupported when it
+// does not fit or is not expected to take less than limit_ns.
+cudaError_t launch_spmm_rows(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,
+                             bool early, double limit_ns, cudaStream_t stream);
+
 // Batch-tile width the RNN step kernels use for a batch of B (sizes the counters).
 int rnn_batch_tile(int64_t B);
 

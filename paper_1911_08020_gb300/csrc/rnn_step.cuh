@@ -1,6 +1,6 @@
-// rnn_step.cuh -- one LSTM or GRU cell step with the cell local
-// to the CTA that owns a hidden unit (Sec. 3.2, Fig. 6(b) on the stacked input
-// [x_t; h_{t-1}], then the cell of Sec. 4.1).
+// rnn_step.cuh -- one LSTM or GRU cell step, or a plain product, local
+// to the CTA that owns a hidden unit or a row (Sec. 3.2, Fig. 6(b) on the
+// stacked input [x_t; h_{t-1}], then the cell of Sec. 4.1; or on X).
 //
 // The batch columns are cut into tiles of bt columns, and the CTAs into one
 // group a tile; within a group every CTA owns a contiguous range of hidden
@@ -30,6 +30,15 @@
 // 3072 x 2048 bf16 at batch 64: 11.5 against 32.3; LSTM 6000 x 3000 bf16 at
 // batch 20: 16.5 against 37.9, fp32 at batch 37: 30 against 212.  Those kernels
 // remain for inputs too tall to stage at 4 columns (some 14000 rows).
+//
+// A plain product (kModeY; the rows are the units, X the whole input) takes
+// this kernel from batch 5 on while it is expected to be faster than the
+// kernels that stream through clusters, whose fixed part is larger but whose
+// gather is cheaper: us against batch_kernel (batch 6, 8) and xres (the
+// others), 1024 x 1024 fp32 at batch 6 / 8 / 24 / 64: 3.9 / 3.7 / 3.9 / 4.4
+// against 27.6 / 4.9 / 10.2 / 10.2; 6000 x 3000 fp32 at 6 / 8 / 16: 8.7 / 7.4 /
+// 9.7 against 80 / 15 / 14, but 16.2 against 11.8 at 32; 2000 x 2500 fp32 at
+// 24 / 64 / 100: 6.7 / 9.2 / 13.4 against 12.2 / 11.8 / 13.0.
 #pragma once
 
 #include "kernels_common.cuh"
@@ -66,6 +75,7 @@ constexpr int kStage4 = 0, kStage16 = 1, kStageBoxes = 2;
 
 struct Plan {
     int ntiles, members;          // CTA i is CTA i / ntiles of tile i % ntiles
+    int64_t ldx, ldy;             // kModeY: pitches of X and Y
     int staging, early;           // kStage*; the records may be read before the PDL wait
     int nbx, bxh, nbh, bhh;       // boxes of x and h: their number and rows (the last one ends with the matrix)
     uint32_t row_off, nseg_off, bias_off, c_off, in_off, part_off;
@@ -75,7 +85,7 @@ template <bool BF16, int MODE, int LBT>
 __global__ void __launch_bounds__(kThreads, 1)
 step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mh,
             Plan p) {
-    constexpr int kGates = MODE == kModeLstm ? 4 : 3;
+    constexpr int kGates = MODE == kModeLstm ? 4 : MODE == kModeGru ? 3 : 1;
     constexpr bool kGru = MODE == kModeGru;
     constexpr int kSides = kGru ? 2 : 1;
     constexpr int bt = 1 << LBT, L = bt / 4, S = 32 / L, kSubs = kStepWarps * S;
@@ -93,8 +103,8 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
     pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tile = int(blockIdx.x) % p.ntiles, member = int(blockIdx.x) / p.ntiles;
-    const int H = ra.H, I = ra.I, K = I + H;
-    const int64_t B = ra.B, b0 = int64_t(tile) << LBT;
+    const int H = ra.H, I = ra.I, K = MODE == kModeY ? I : I + H;   // kModeY: H rows, I columns
+    const int64_t B = ra.B, ldx = MODE == kModeY ? p.ldx : B, b0 = int64_t(tile) << LBT;
     const int nb = static_cast<int>(B - b0 < bt ? B - b0 : bt);
     const int u0 = static_cast<int>(int64_t(H) * member / p.members);
     const int nu = static_cast<int>(int64_t(H) * (member + 1) / p.members) - u0;
@@ -228,7 +238,7 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
         const float *const sx = ra.x + b0 + (in ? j : 0), *const sh = ra.h + b0 + (in ? j : 0);
 #pragma unroll 4
         for (int k = tid / Q; k < K; k += kStep, dst += kThreads * 16)
-            cp_async16(dst, k < I ? sx + int64_t(k) * B : sh + int64_t(k - I) * B, in);
+            cp_async16(dst, MODE == kModeY || k < I ? sx + int64_t(k) * ldx : sh + int64_t(k - I) * B, in);
     } else {
         constexpr int kStep = kThreads >> LBT;
         const int j = tid & (bt - 1);
@@ -237,13 +247,14 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
         const float *const sx = ra.x + b0 + (in ? j : 0), *const sh = ra.h + b0 + (in ? j : 0);
 #pragma unroll 4
         for (int k = tid >> LBT; k < K; k += kStep, dst += kThreads * 4)
-            cp_async4(dst, k < I ? sx + int64_t(k) * B : sh + int64_t(k - I) * B, in);
+            cp_async4(dst, MODE == kModeY || k < I ? sx + int64_t(k) * ldx : sh + int64_t(k - I) * B, in);
     }
+    if constexpr (MODE != kModeY)
     for (int v = tid; v < VR; v += kThreads) {
         const float *b = kGru ? (v < R ? ra.b_ih : ra.b_hh) : ra.bias;
         cp_async4(smem_addr(s_bias + v), b ? b + grow(v < R ? v : v - R) : ra.h, b != nullptr);
     }
-    if constexpr (!kGru)
+    if constexpr (MODE == kModeLstm)
         for (int i = tid; i < nu << LBT; i += kThreads) {
             const int j = i & (bt - 1);
             cp_async4(smem_addr(s_c + i), ra.c_prev + int64_t(u0 + (i >> LBT)) * B + b0 + (j < nb ? j : 0), j < nb);
@@ -322,16 +333,26 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
 
     // ---- the cells of the owned units
     auto sum = [&](int v, int j) {
-        float r = 0.0f;
         const int seg = s_row[v].seg, n = s_nseg[v];
-        for (int i = 0; i < n; ++i) r += s_part[((seg + i) << LBT) + j];
-        return r;
+        float r0 = 0.0f, r1 = 0.0f;
+        if constexpr (MODE != kModeY) {   // few: the lane groups' runs are long
+            for (int i = 0; i < n; ++i) r0 += s_part[((seg + i) << LBT) + j];
+            return r0;
+        }
+        for (int i = 0; i + 1 < n; i += 2) {
+            r0 += s_part[((seg + i) << LBT) + j];
+            r1 += s_part[((seg + i + 1) << LBT) + j];
+        }
+        if (n & 1) r0 += s_part[((seg + n - 1) << LBT) + j];
+        return r0 + r1;
     };
     for (int i = tid; i < nu << LBT; i += kThreads) {
         const int ui = i >> LBT, j = i & (bt - 1);
         if (j >= nb) continue;
         const int64_t e = int64_t(u0 + ui) * B + b0 + j;
-        if constexpr (!kGru) {
+        if constexpr (MODE == kModeY) {
+            ra.h_out[int64_t(u0 + ui) * p.ldy + b0 + j] = sum(ui, j);
+        } else if constexpr (!kGru) {
             float pre[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) pre[q] = sum(q * nu + ui, j) + s_bias[q * nu + ui];
@@ -375,14 +396,15 @@ cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem,
     // aligned rows in 16-byte copies (boxes of short or ragged rows are slower:
     // batch 8 6.0 against 7.3 us, 6000 x 3000 at batch 20 17.5 against 21.6),
     // the rest 4 bytes at a time
-    const bool aligned = ra.B % 4 == 0 && (ra.I == 0 || reinterpret_cast<uintptr_t>(ra.x) % 16 == 0) &&
-                         reinterpret_cast<uintptr_t>(ra.h) % 16 == 0;
+    const int64_t ldx = MODE == kModeY ? p.ldx : ra.B;
+    const bool aligned = ra.B % 4 == 0 && ldx % 4 == 0 && (ra.I == 0 || reinterpret_cast<uintptr_t>(ra.x) % 16 == 0) &&
+                         (MODE == kModeY || reinterpret_cast<uintptr_t>(ra.h) % 16 == 0);
     p.staging = aligned ? kStage16 : kStage4;
     if (LBT == 5 && aligned && ra.B % bt == 0 && tensor_map_encoder() != nullptr) {
-        auto make = [&](CUtensorMap *m, const float *base, int rows, int boxh) {
+        auto make = [&](CUtensorMap *m, const float *base, int rows, int boxh, int64_t ld) {
             if (rows == 0) return true;
             const cuuint64_t dims[2] = {cuuint64_t(ra.B), cuuint64_t(rows)};
-            const cuuint64_t strides[1] = {cuuint64_t(ra.B) * 4};
+            const cuuint64_t strides[1] = {cuuint64_t(ld) * 4};
             const cuuint32_t box[2] = {cuuint32_t(bt), cuuint32_t(boxh)};
             const cuuint32_t es[2] = {1, 1};
             return tensor_map_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims,
@@ -391,19 +413,22 @@ cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem,
                                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
         };
         boxes(ra.I, &p.nbx, &p.bxh);
-        boxes(ra.H, &p.nbh, &p.bhh);
-        if (make(&mx, ra.x, ra.I, p.bxh) && make(&mh, ra.h, ra.H, p.bhh)) p.staging = kStageBoxes;
+        boxes(MODE == kModeY ? 0 : ra.H, &p.nbh, &p.bhh);
+        if (make(&mx, ra.x, ra.I, p.bxh, ldx) && (MODE == kModeY || make(&mh, ra.h, ra.H, p.bhh, ra.B)))
+            p.staging = kStageBoxes;
     }
     return launch_ex(kernel, dim3(static_cast<unsigned>(p.ntiles * p.members)), dim3(kThreads), smem, stream, 1, true,
                      f, ra, mx, mh, p);
 }
 
-// The step on this kernel, or cudaErrorNotSupported when the staged tile does
-// not fit beside the CTA's rows even at 4 columns.
+// The step (or product) on this kernel, or cudaErrorNotSupported when the
+// staged tile does not fit beside the CTA's rows even at 4 columns, or no tile
+// width is expected to take less than limit_ns.
 template <bool BF16, int MODE>
-cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream) {
-    constexpr int kGates = MODE == kModeLstm ? 4 : 3;
-    const int64_t K = int64_t(ra.I) + ra.H;
+cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream, int64_t ldx = 0,
+                   int64_t ldy = 0, double limit_ns = 1e300) {
+    constexpr int kGates = MODE == kModeLstm ? 4 : MODE == kModeGru ? 3 : 1;
+    const int64_t K = MODE == kModeY ? ra.I : int64_t(ra.I) + ra.H;
     if (K > 60000 || ra.B > 1024 || f.nitems[0][0] <= 0) return cudaErrorNotSupported;
     // kept weights of the matrix, padded to whole groups and chunks
     const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
@@ -411,7 +436,7 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
     int lbt = -1;
     size_t smem = 0;
     Plan best{};
-    double best_ns = 1e300;
+    double best_ns = limit_ns;
     for (int l = kMinLbt; l <= kMaxLbt && (l == kMinLbt || (1 << (l - 1)) < ra.B); ++l) {
         const int bt = 1 << l;
         Plan p{};
@@ -433,12 +458,17 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
         p.bias_off = take(size_t(vr) * 4);
         p.c_off = take(MODE == kModeLstm ? size_t(units) * bt * 4 : 0);
         if (o > kSmemCap) continue;
-        // the staging of K rows (70 bytes/ns an SM) and the gather; a narrow
-        // tile stages less, but its staged rows share banks and each CTA
-        // multiplies more weights (cycles fitted to the shapes above)
-        static const double kCycles[kMaxLbt - kMinLbt + 1] = {0.9, 1.0, 1.35, 1.5};
+        // launch and latencies, the staging of K rows, the gather, and a
+        // product's outputs.  A narrow tile stages less, but its staged rows
+        // share banks and each CTA multiplies more weights.  (Cycles a kept
+        // weight and staging rates fitted to steps, whose rows are long, and to
+        // products of 300 to 9216 columns at batch 2 to 256.)
+        static const double kCycles[2][kMaxLbt - kMinLbt + 1] = {{0.9, 1.0, 1.35, 1.5}, {0.9, 0.95, 1.45, 2.4}};
         const int waves = (p.ntiles * p.members + sms - 1) / sms;
-        const double ns = waves * (double(K) * bt * 4 / 70.0 + kept / p.members * kCycles[l - kMinLbt] / 1.9);
+        const double bytes = double(K) * bt * 4;
+        const double staging = MODE == kModeY ? bytes / 250.0 + std::max(0.0, bytes - 98304.0) / 100.0 : bytes / 70.0;
+        const double ns = 3200.0 + waves * (staging + kept / p.members * kCycles[MODE == kModeY][l - kMinLbt] / 1.9 +
+                                            (MODE == kModeY ? double(units) * bt / kThreads * 250.0 : 0.0));
         if (ns < best_ns) {
             best_ns = ns;
             best = p;
@@ -448,6 +478,8 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
     }
     if (lbt < 0) return cudaErrorNotSupported;
     best.early = early ? 1 : 0;
+    best.ldx = ldx;
+    best.ldy = ldy;
     return lbt == 2   ? launch_tile<BF16, MODE, 2>(f, ra, best, smem, stream)
            : lbt == 3 ? launch_tile<BF16, MODE, 3>(f, ra, best, smem, stream)
            : lbt == 4 ? launch_tile<BF16, MODE, 4>(f, ra, best, smem, stream)

@@ -1,8 +1,8 @@
 // spmm.cu -- y = W_darb X on the GPU (Sec. 3.2, Fig. 6(b)): the entry the C
 // ABI calls.  Batch 1 runs the one-group-per-CTA kernel (gemv.cuh) when x fits
 // in shared memory, batch <= 4 otherwise the row-per-lane kernel (rowlane.cuh:
-// the HBM-bound regime, values and offsets stream once), wider batches the
-// batch-per-lane kernel (batch.cuh, instantiated in spmm_batch.cu).  All of
+// the HBM-bound regime, values and offsets stream once), wider batches one of
+// three kernels (spmm_batch.cu).  All of
 // them evaluate exactly the per-block selection and sum of Fig. 6(b) on the
 // CUDA cores and allocate nothing.  The tensor-core kernel (tc.cuh, in
 // spmm_tc.cu) runs only when the caller asks for it by name.  All accumulate

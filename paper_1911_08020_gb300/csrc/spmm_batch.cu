@@ -1,9 +1,12 @@
-// spmm_batch.cu -- the batch > 4 product for plain Y: from 17 columns on the
-// kernel with the activation tile resident in shared memory (xres.cuh) when
-// the call fits it, else the streaming batch kernel (batch.cuh).  At 16
-// columns or fewer the resident tile is one 16-column tile, whose 64-byte rows
-// put two rows in each quarter-warp's 128-byte read (half of them conflict),
-// and the streaming kernel measured faster (FC6 11.9 us against 16.8).
+// spmm_batch.cu -- the batch > 4 product for plain Y, on one of three kernels.
+// Small and middling products take the kernel whose CTAs own rows and stage
+// the whole input (rnn_step.cuh) while it is expected to be faster than the
+// others, which split the columns over clusters: from 17 columns on, and for
+// any batch whose X no tensor map can describe (FC6 at batch 13: 15 us against
+// 26), the one with the activation tile resident in shared memory (xres.cuh)
+// when the call fits it, else the streaming batch kernel (batch.cuh).  At 16
+// columns or fewer xres's tile is half empty or more, and the streaming
+// kernel measured faster (FC6 11.4 us against 12.6).
 #include "batch.cuh"
 #include "xres.cuh"
 
@@ -11,9 +14,22 @@ namespace darb {
 
 cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y,
                               int64_t ldy, bool early, cudaStream_t stream) {
-    if (batch > 16) {
-        const cudaError_t e = f.bf16 ? xres::launch<true, 32>(f, X, ldx, batch, Y, ldy, early, stream)
-                                     : xres::launch<false, 32>(f, X, ldx, batch, Y, ldy, early, stream);
+    // what the cluster kernels take: a fixed part (for xres larger with the
+    // columns, and with plain copies of unaligned X) and 1.5 times the time of
+    // the gather at 128 bytes a clock and SM, over whole 32-column tiles.
+    // (Fitted to products of 300 to 9216 columns.  Where the two estimates meet
+    // the kernels differ by up to 4% the other way: 700 x 6000 fp32 at batch
+    // 16 takes 8.0 us against 7.7.)
+    const bool aligned = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
+    const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
+    const double gather_ns = kept * double((batch + 31) / 32) * 128.0 / (128.0 * 2.0 * sm_count());
+    const double others_ns = (batch > 16 ? 6500.0 + 0.3 * double(f.cols) : 5500.0) + (aligned ? 0.0 : 1500.0) + 1.5 * gather_ns;
+    cudaError_t e = launch_spmm_rows(f, X, ldx, batch, Y, ldy, early, others_ns, stream);
+    if (e != cudaErrorNotSupported) return e;
+    cudaGetLastError();
+    if (batch > 16 || !aligned) {
+        e = f.bf16 ? xres::launch<true, 32>(f, X, ldx, batch, Y, ldy, early, stream)
+                   : xres::launch<false, 32>(f, X, ldx, batch, Y, ldy, early, stream);
         if (e != cudaErrorNotSupported) return e;
         cudaGetLastError();
     }

@@ -69,6 +69,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 #include <vector>
@@ -107,6 +108,7 @@ constexpr int kMaxGroups = kXresMaxGroups;     // groups of a row set, at most
 constexpr int kMaxClusters = 160;
 constexpr int kUnitCost = 10;                  // fixed cost of a unit, in group-chunks
 constexpr int kSwitchCost = 40;                // a run's move to another batch tile, in group-chunks
+constexpr int kClusterCost = 20;               // of clusters of several CTAs, in group-chunks
 constexpr size_t kSmemCap = 227 * 1024;        // dynamic shared memory, at most (the kernel has no static part)
 
 template <bool BF16>
@@ -657,12 +659,23 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
     // fits (up to kMaxStages) and the partial sums of the largest set.  Of the
     // splits with kMinStages or more, the one whose clusters occupy the most
     // SMs, then the deeper ring, then the smaller split; a shallower ring only
-    // when no split has that.
-    Plan p{};
-    uint32_t smem = 0;
-    int64_t best_sms = 0;
-    int best_nst = 0;
-    bool best_deep = false;
+    // when no split has that.  Where that leaves its clusters with fewer than
+    // two units, most SMs idle while a unit runs: the split that is expected to
+    // take the least time then, if it is well below (in group-chunks of
+    // multiplying, 137 ns: the load of the slice, and the units of a cluster,
+    // each its share of the set's work and a fixed cost; more where partial sums
+    // cross CTAs).  512 x 4000 bf16 at
+    // batch 64: 9.0 us against 13.8, 2000 x 2500 fp32 at 64: 8.9 against 11.8.
+    // By that estimate alone 5000 x 700 at batch 256 went from 18.0 to 20.1.
+    struct Split {
+        Plan p;
+        uint32_t smem;
+        int64_t sms;
+        bool deep;
+        double cost;
+    };
+    Split most{}, least{};   // most SMs; least expected time
+    bool few = false;
     for (int C = 1; C <= 8; ++C) {
         int64_t S = (f.cols + C - 1) / C;
         int64_t rows = S + f.m_max - 1;
@@ -670,34 +683,41 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
             const int64_t Sa = (S + lcm - 1) / lcm * lcm;
             if (Sa <= rows) S = rows = Sa;
         }
-        const int nboxes = static_cast<int>((rows + 255) / 256);
-        const int box_rows = static_cast<int>((rows + nboxes - 1) / nboxes);
-        const uint64_t x_bytes = uint64_t(nboxes) * box_rows * T * 4;
-        if (nboxes > kMaxBoxes) continue;
+        Split s{};
+        s.p.C = C;
+        s.p.S = static_cast<int>(S);
+        s.p.nboxes = static_cast<int>((rows + 255) / 256);
+        if (s.p.nboxes > kMaxBoxes) continue;
+        s.p.box_rows = static_cast<int>((rows + s.p.nboxes - 1) / s.p.nboxes);
+        const uint64_t x_bytes = uint64_t(s.p.nboxes) * s.p.box_rows * T * 4;
         const uint64_t ring_off = kBarBytes + x_bytes;
         const uint64_t part_bytes = uint64_t(kMaxGroups) * kSlots * T * 4;
         if (ring_off + 2 * stage_bytes<BF16>() + part_bytes > kSmemCap) continue;
-        const int nst = static_cast<int>(
+        s.p.nst = static_cast<int>(
             std::min<uint64_t>(kMaxStages, (kSmemCap - ring_off - part_bytes) / stage_bytes<BF16>()));
-        const uint64_t part_off = ring_off + uint64_t(nst) * stage_bytes<BF16>();
-        const uint32_t total = static_cast<uint32_t>(part_off + part_bytes);
-        const int64_t sms = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(C, total), kMaxClusters) * C;
-        const bool deep = nst >= kMinStages;
-        const bool better = deep != best_deep ? deep : (sms != best_sms ? sms > best_sms : nst > best_nst);
-        if (sms <= 0 || !better) continue;
-        best_sms = sms;
-        best_nst = nst;
-        best_deep = deep;
-        p.C = C;
-        p.S = static_cast<int>(S);
-        p.nst = nst;
-        p.box_rows = box_rows;
-        p.nboxes = nboxes;
-        p.x_bytes = static_cast<uint32_t>(x_bytes);
-        p.ring_off = static_cast<uint32_t>(ring_off);
-        p.part_off = static_cast<uint32_t>(part_off);
-        smem = total;
+        s.p.x_bytes = static_cast<uint32_t>(x_bytes);
+        s.p.ring_off = static_cast<uint32_t>(ring_off);
+        s.p.part_off = static_cast<uint32_t>(ring_off + uint64_t(s.p.nst) * stage_bytes<BF16>());
+        s.smem = static_cast<uint32_t>(s.p.part_off + part_bytes);
+        s.sms = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(C, s.smem), kMaxClusters) * C;
+        s.deep = s.p.nst >= kMinStages;
+        if (s.sms <= 0) continue;
+        const double ncl = double(s.sms / C);
+        const int tb = double(tiles) * f.nxsets[1] >= 2 * ncl ? 1 : 0;
+        const double nsets = f.nxsets[tb], work = double(f.xset_prefix[tb][f.nxsets[tb]]);
+        s.cost = double(rows) * (T * 4 / (77.0 * 137.0)) +
+                 std::ceil(double(tiles) * nsets / ncl) * (work / (C * nsets) + 2 + kUnitCost) +
+                 (C > 1 ? kClusterCost : 0);
+        if (most.sms == 0 || (s.deep != most.deep ? s.deep : s.sms != most.sms ? s.sms > most.sms : s.p.nst > most.p.nst)) {
+            most = s;
+            few = double(tiles) * nsets < 2 * ncl;
+        }
+        if (least.sms == 0 || (s.deep != least.deep ? s.deep : s.cost < least.cost)) least = s;
     }
+    const Split &best = few && least.deep == most.deep && least.cost < 0.85 * most.cost ? least : most;
+    Plan p = best.p;
+    const uint32_t smem = best.smem;
+    const int64_t best_sms = best.sms;
     if (best_sms <= 0) return cudaErrorNotSupported;
     const int64_t occ = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(p.C, smem), kMaxClusters);
     // Row sets of about 4 heaviest groups (table 1: 128 rows, the consumers'
