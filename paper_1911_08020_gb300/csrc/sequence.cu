@@ -21,21 +21,23 @@
 // a weight, and the 128 / bt subgroups of a warp take the weights of a row in
 // turn; their sums meet in a shuffle reduction that leaves each lane one
 // column.  The owning CTA applies the cell.  Steps are separated by a barrier
-// over the group's CTAs (arrival counter in global memory, spun on with a 1 s
-// limit; on expiry the kernel records a timeout, raises an abort flag that
-// ends every other CTA's wait, and returns).  The launch is cooperative, so
-// all CTAs are resident and the barrier cannot starve.  No CTA touches another
+// over the group's CTAs (arrival counter in global memory) or, where a tile of
+// h is small, by the values of h themselves, which carry the number of their
+// step; both are spun on with a 1 s limit (on expiry the kernel records a
+// timeout, raises an abort flag that ends every other CTA's wait, and
+// returns).  The launch is cooperative, so all CTAs are resident and no wait
+// can starve.  No CTA touches another
 // CTA's shared memory, and no CTA leaves while a copy it issued may still be
 // landing.
 //
 // What bounds a step (cycle stamps, 6000 x 3000 bf16 at batch 20, tiles of 32,
-// ~14000 cycles): the gather and its reductions 6500, the barrier 2900, the
-// cell 2000, staging 1800.  One column group instead of one a tile stages every
-// column in every CTA: GRU 3072 x 2048 at batch 64 took 11.0 against 8.7 us a
-// step.  Against one lane a column, tensor-map staging and all CTAs in one
-// barrier, whole calls went from 3131 to 1606 us (that GRU, 200 steps), 507 to
-// 343 (the LSTM above, 35 steps), 520 to 399 (LSTM 4096 x 1280 fp32, batch 1,
-// 100 steps), and 2592 to 620 where the batch is no multiple of 4 (GRU 2100 x
+// ~13000 cycles): the gather and its reductions 5900, the barrier 2700,
+// staging 2500, the cell 1800.  One column group instead of one a tile stages
+// every column in every CTA: GRU 3072 x 2048 at batch 64 took 11.0 against 8.7
+// us a step.  Against one lane a column, tensor-map staging and all CTAs in one
+// barrier, whole calls went from 3131 to 1512 us (that GRU, 200 steps), 507 to
+// 332 (the LSTM above, 35 steps), 520 to 321 (LSTM 4096 x 1280 fp32, batch 1,
+// 100 steps), and 2592 to 588 where the batch is no multiple of 4 (GRU 2100 x
 // 1000, batch 37, 100 steps).
 #include "darb_internal.h"
 #include "kernels_common.cuh"
@@ -57,6 +59,7 @@ constexpr size_t kSmemCap = 226 * 1024 + 512;   // dynamic shared memory, below 
 constexpr int kMaxLbt = 5;                // batch tiles of at most 2^5 columns
 constexpr size_t kCellOnChip = 16 * 1024; // LSTM cell state kept in shared memory up to this size
 constexpr int kBarWords = 32;             // words between the barrier counters of two groups (128 bytes)
+constexpr size_t kTaggedBytes = 32 * 1024;  // h tiles up to this size are exchanged with tags, without barriers
 constexpr int kCopies = 8;                // bulk copies a staged tile is cut into, at most
 
 struct Ranges {
@@ -76,6 +79,7 @@ struct SeqArgs {
     int piece;              // kept weights per work item, at most
     int c_on_chip;          // LSTM: cell state in shared memory
     int x_mode;             // kX*
+    int tagged;             // h is exchanged as (value, tag) pairs, without barriers
     // staged input rows: x_t at [0, irows), h_{t-1} from row irows on (hrows of
     // them), both rounded up to 4 rows; a zero row at irows + hrows
     int irows, hrows;
@@ -93,7 +97,10 @@ struct SeqArgs {
     float *c_seq;           // T x H x B or nullptr (LSTM)
     float *c_state;         // H x B: the running cell state when it is not on chip (LSTM)
     float *c_last;          // H x B or nullptr (LSTM)
-    float *h_x;             // the exchanged h_t, [t & 1][ntiles][hrows][bt]; h0 in buffer 1 at launch
+    // the exchanged h_t, [t & 1][ntiles][hrows][bt]; h0 in buffer 1 at launch.
+    // Tagged: 8-byte pairs of a value and the number of the step that reads it,
+    // plus 1; at launch 1 with h0, 0 in buffer 0 and ~0 in rows past H
+    float *h_x;
     unsigned *bar;          // arrival counters of the groups, kBarWords apart, zero at launch
     int *abort_flag;        // zero at launch
     int32_t *status;
@@ -318,6 +325,64 @@ __device__ __forceinline__ bool wait_arrivals(const SeqArgs &a, const unsigned *
     }
 }
 
+// One (value, tag) pair of an exchanged h: a single 8-byte access, so that the
+// tag vouches for the value next to it without any ordering.
+__device__ __forceinline__ void put_tagged(float *h_x, int64_t i, float v, uint32_t tag) {
+    const uint64_t w = (uint64_t(tag) << 32) | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(reinterpret_cast<uint64_t *>(h_x) + i), "l"(w) : "memory");
+}
+__device__ __forceinline__ ulonglong2 get_tagged2(const uint64_t *p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
+// Stage n2 pairs of tagged elements, waiting for each to carry `tag` (or a
+// later one); false if this thread gave up or another CTA did.  A buffer is
+// written again two steps later, when every CTA of the group has published the
+// step in between, i.e. has read this one.  U: loads a thread has in flight.
+template <int U>
+__device__ __forceinline__ bool stage_tagged(const SeqArgs &a, const float *h_x, int64_t first, int n2, uint32_t tag,
+                                             float *dst) {
+    const uint64_t *src = reinterpret_cast<const uint64_t *>(h_x) + first;
+    unsigned long long t0 = 0;
+    unsigned spin = 0;
+    for (int i0 = threadIdx.x; i0 < n2; i0 += kThreads * U) {
+        ulonglong2 v[U];
+        unsigned wanted = 0;   // bit u: element u has not come yet
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * kThreads < n2) wanted |= 1u << u;
+        const unsigned all = wanted;
+        while (true) {   // all that is missing is asked for again at once
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (wanted >> u & 1) v[u] = get_tagged2(src + 2 * (i0 + u * kThreads));
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if ((wanted >> u & 1) && uint32_t(v[u].x >> 32) >= tag && uint32_t(v[u].y >> 32) >= tag)
+                    wanted &= ~(1u << u);
+            if (wanted == 0) break;
+            if ((++spin & 63) == 0) {
+                if (*reinterpret_cast<volatile int *>(a.abort_flag)) return false;
+                const unsigned long long now = global_timer_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > a.barrier_ns) {
+                    atomicExch(a.abort_flag, 1);
+                    atomicOr(a.status, kStatusTimeout);
+                    return false;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (all >> u & 1)
+                reinterpret_cast<float2 *>(dst)[i0 + u * kThreads] =
+                    make_float2(__uint_as_float(uint32_t(v[u].x)), __uint_as_float(uint32_t(v[u].y)));
+    }
+    return true;
+}
+
 // A tile of `bytes` (a multiple of 16): one warp, each of its first kCopies
 // lanes a bulk copy that completes on `bar` (one thread issuing all of them
 // took 1400 cycles of a step).  Lane 0 arms `bar`
@@ -336,7 +401,7 @@ __device__ __forceinline__ void copy_tile(int lane, float *dst, const float *src
                  lane == kCopies - 1 || bytes - at < each ? bytes - at : each, bar);
 }
 
-template <bool BF16, int MODE, int LBT>
+template <bool BF16, int MODE, int LBT, bool TAGGED>
 __global__ void __launch_bounds__(kThreads, 1)
 seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
     using G = Lanes<LBT>;
@@ -351,7 +416,7 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
     PT *s_w = reinterpret_cast<PT *>(sm + sp.w_off);
     int *s_rowptr = reinterpret_cast<int *>(sm + sp.rowptr_off);
     int *s_mid = reinterpret_cast<int *>(sm + sp.mid_off);          // GRU: first kept weight of a row on h
-    int *s_rowitem = reinterpret_cast<int *>(sm + sp.rowitem_off);  // items of local row lr: [s_rowitem[lr], s_rowitem[lr+1])
+    uint32_t *s_rowitem = reinterpret_cast<uint32_t *>(sm + sp.rowitem_off);   // a row's first item | their number << 16 (>= 1)
     int4 *s_item = reinterpret_cast<int4 *>(sm + sp.item_off);      // (first, end, number (at first: local row), first on h)
     float *s_bias = reinterpret_cast<float *>(sm + sp.bias_off);    // [R] (GRU: [2R], b_ih then b_hh)
     float *s_c = reinterpret_cast<float *>(sm + sp.c_off);          // [units][tpg * bt] when on chip
@@ -413,12 +478,12 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
             const int n = s_rowptr[lr + 1];
             s_rowptr[lr] = p;
             s_mid[lr] += p;
-            s_rowitem[lr] = ni;
+            const int first = ni;
             for (int q = 0; q < n; q += a.piece) s_item[ni++] = make_int4(p + q, p + min(n, q + a.piece), lr, 0);
+            s_rowitem[lr] = uint32_t(first) | uint32_t(ni - first) << 16;
             p += n;
         }
         s_rowptr[R] = p;
-        s_rowitem[R] = ni;
         s_nitems = ni;
     }
     __syncthreads();
@@ -512,7 +577,16 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                     const int j = i & (bt - 1);
                     s_in[i] = j < nb ? __ldg(a.x + (int64_t(t) * I + (i >> LBT)) * B + b0 + j) : 0.0f;
                 }
-            if (warp == 0) {
+            bool ok = true;
+            if constexpr (TAGGED) {
+                const int64_t first = (int64_t((t + 1) & 1) * a.ntiles + tile) * (int64_t(a.hrows) << LBT);
+                const int n2 = a.hrows * bt / 2;   // up to 8 a thread (kTaggedBytes)
+                float *dst = s_in + (a.irows << LBT);
+                const uint32_t tag = uint32_t(t) + 1u;
+                ok = n2 <= kThreads       ? stage_tagged<1>(a, a.h_x, first, n2, tag, dst)
+                     : n2 <= 4 * kThreads ? stage_tagged<4>(a, a.h_x, first, n2, tag, dst)
+                                          : stage_tagged<8>(a, a.h_x, first, n2, tag, dst);
+            } else if (warp == 0) {
                 int go = 1;
                 if (lane == 0 && k == 0 && t > 0) go = wait_arrivals(a, bar, unsigned(t) * members);
                 if (__shfl_sync(0xFFFFFFFFu, go, 0)) {
@@ -524,8 +598,8 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                     mbar_arrive(&s_hfull);   // no copy comes: let the waiting threads see s_fail
                 }
             }
-            if (a.x_mode == kXPlain) __syncthreads();
-            bool ok = mbar_wait(&s_hfull, staged & 1);
+            if (TAGGED || a.x_mode == kXPlain) __syncthreads();
+            if (!TAGGED) ok = mbar_wait(&s_hfull, staged & 1);
             if (xbulk) ok = mbar_wait(&s_xfull, staged & 1) && ok;
             // partial gate sums of the work items, handed out to warps as they come free
             for (int ii = warp; ii < NI;) {
@@ -548,7 +622,7 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                 if (tid == 0) {
                     atomicOr(a.status, kStatusTimeout);
                     atomicExch(a.abort_flag, 1);
-                    mbar_wait(&s_hfull, staged & 1);
+                    if (!TAGGED) mbar_wait(&s_hfull, staged & 1);
                     if (xbulk) mbar_wait(&s_xfull, staged & 1);
                 }
                 return;
@@ -560,18 +634,24 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                 if (xbulk && (more || t + 1 < a.T)) copy_x(more ? t : t + 1, more ? tile + a.ngroups : group);
             }
             // the cells of the owned units for these columns
+            const int64_t hx0 = ((int64_t(t & 1) * a.ntiles + tile) * a.hrows + u0) * bt;
+            auto publish = [&](int i, float v) {
+                if (!TAGGED) a.h_x[hx0 + i] = v;
+                else if (!(int(blockIdx.x) == a.skip_cta && t == 0)) put_tagged(a.h_x, hx0 + i, v, uint32_t(t) + 2u);
+            };
             // partial sums of local row lr: part 0 (everything, or the x part of a
             // split GRU row), part 1 (the h part of a split GRU row)
             auto sum = [&](int lr, int part, int j) {
-                float v = 0.0f;
-                for (int ii = s_rowitem[lr]; ii < s_rowitem[lr + 1]; ++ii) v += s_part[((part * NI + ii) << LBT) + j];
+                const uint32_t it = s_rowitem[lr];
+                const float *sp = s_part + (((it & 0xFFFFu) + part * NI) << LBT) + j;
+                float v = sp[0];
+                for (uint32_t o = 1; o < it >> 16; ++o) v += sp[o << LBT];
                 return v;
             };
-            float *hx = a.h_x + ((int64_t(t & 1) * a.ntiles + tile) * a.hrows + u0) * bt;
             for (int i = tid; i < nu << LBT; i += kThreads) {
                 const int ui = i >> LBT, j = i & (bt - 1);
                 if (j >= nb) {
-                    hx[i] = 0.0f;
+                    publish(i, 0.0f);
                     continue;
                 }
                 const int64_t e = int64_t(ui) * B + b0 + j;
@@ -583,7 +663,7 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                     const float cprev = t == 0 && !a.c_on_chip ? a.c0[int64_t(u0) * B + e] : c_run[ec];
                     const float c = sigm(pf) * cprev + sigm(pi) * tanhf(pg);
                     const float hv = sigm(po) * tanhf(c);
-                    hx[i] = hv;
+                    publish(i, hv);
                     c_run[ec] = c;
                     if (ct) ct[e] = c;
                     ht[e] = hv;
@@ -595,13 +675,13 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                     const float zz = sigm(gx_(nu + ui) + gh_(nu + ui));
                     const float nn = tanhf(gx_(2 * nu + ui) + rr * gh_(2 * nu + ui));
                     const float hv = (1.0f - zz) * nn + zz * s_in[((a.irows + u0 + ui) << LBT) + j];
-                    hx[i] = hv;
+                    publish(i, hv);
                     ht[e] = hv;
                 }
             }
             __syncthreads();
         }
-        if (t + 1 < a.T && tid == 0 && !(int(blockIdx.x) == a.skip_cta && t == 0))
+        if (!TAGGED && t + 1 < a.T && tid == 0 && !(int(blockIdx.x) == a.skip_cta && t == 0))
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     }
     if constexpr (!kGru)
@@ -623,6 +703,14 @@ __global__ void __launch_bounds__(256) prep_kernel(SeqArgs a, int lbt, const flo
     for (int i = int(blockIdx.x) * 256 + int(threadIdx.x); i < nwords; i += int(gridDim.x) * 256) a.bar[i] = 0u;
     const int bt = 1 << lbt;
     const int64_t nrows = a.H + (x_tiles || xall ? int64_t(a.T) * a.I : 0);
+    if (a.tagged) {   // tags of buffer 0, and of the rows past H in both
+        const int64_t n = int64_t(a.ntiles) * a.hrows << lbt;
+        for (int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x; i < n; i += int64_t(gridDim.x) * 256) {
+            const bool pad = (i >> lbt) % a.hrows >= a.H;
+            reinterpret_cast<uint64_t *>(a.h_x)[i] = pad ? ~uint64_t(0) << 32 : 0;
+            if (pad) reinterpret_cast<uint64_t *>(a.h_x)[n + i] = ~uint64_t(0) << 32;
+        }
+    }
     for (int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); row < nrows; row += int64_t(gridDim.x) * 8) {
         const int64_t xrow = row - a.H;
         const int64_t t = xrow / a.I, k = xrow < 0 ? row : xrow % a.I;
@@ -634,6 +722,13 @@ __global__ void __launch_bounds__(256) prep_kernel(SeqArgs a, int lbt, const flo
         const int nr = xrow < 0 ? a.hrows : a.irows;   // rows of a tile
         float *dst = (xrow < 0 ? a.h_x + ((int64_t(a.ntiles) * nr) << lbt) : x_tiles + ((t * a.ntiles * nr) << lbt)) +
                      (k << lbt);
+        if (xrow < 0 && a.tagged) {
+            uint64_t *d = reinterpret_cast<uint64_t *>(a.h_x) + ((int64_t(a.ntiles) * nr) << lbt) + (k << lbt);
+            for (int64_t b = lane; b < (int64_t(a.ntiles) << lbt); b += 32)
+                d[(((b >> lbt) * nr) << lbt) + (b & (bt - 1))] =
+                    uint64_t(1) << 32 | (b < B ? __float_as_uint(__ldg(src + b)) : 0u);
+            continue;
+        }
         for (int64_t b = lane; b < (int64_t(a.ntiles) << lbt); b += 32)
             dst[(((b >> lbt) * nr) << lbt) + (b & (bt - 1))] = b < B ? __ldg(src + b) : 0.0f;
     }
@@ -698,16 +793,16 @@ inline bool precompute_x(int64_t T, int64_t I, int64_t H, int64_t B, size_t ws_b
     return I > 0 && 2 * I >= H && T * B >= 64 && T * B <= (int64_t(1) << 19) && ws_bytes <= (size_t(1) << 30);
 }
 
-template <bool BF16, int MODE>
+template <bool BF16, int MODE, bool TAGGED>
 static auto seq_entry(int lbt) {
     using namespace seq;
     switch (lbt) {
-        case 0: return seq_kernel<BF16, MODE, 0>;
-        case 1: return seq_kernel<BF16, MODE, 1>;
-        case 2: return seq_kernel<BF16, MODE, 2>;
-        case 3: return seq_kernel<BF16, MODE, 3>;
-        case 4: return seq_kernel<BF16, MODE, 4>;
-        default: return seq_kernel<BF16, MODE, 5>;
+        case 0: return seq_kernel<BF16, MODE, 0, TAGGED>;
+        case 1: return seq_kernel<BF16, MODE, 1, TAGGED>;
+        case 2: return seq_kernel<BF16, MODE, 2, TAGGED>;
+        case 3: return seq_kernel<BF16, MODE, 3, TAGGED>;
+        case 4: return seq_kernel<BF16, MODE, 4, TAGGED>;
+        default: return seq_kernel<BF16, MODE, 5, TAGGED>;
     }
 }
 
@@ -813,7 +908,12 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     a.tpg = s.tpg;
     a.ntiles = static_cast<int>((B + bt - 1) / bt);
     a.c_last = c_last;
-    const auto kernel = seq_entry<BF16, MODE>(s.lbt);
+    // small tiles are exchanged as tagged pairs: a reader waits for the values
+    // themselves, not for a barrier and then for them (us a step: LSTM 4096 x
+    // 1280 at batch 1 / 8 4.2 / 4.9 -> 3.5 / 4.6, H = 200 at 13 3.5 -> 2.7); twice
+    // the bytes cost more than that on tiles of 128 KB (batch 32: 6.3 -> 8.1)
+    a.tagged = size_t(a.hrows) * bt * 4 <= kTaggedBytes ? 1 : 0;
+    const auto kernel = a.tagged ? seq_entry<BF16, MODE, true>(s.lbt) : seq_entry<BF16, MODE, false>(s.lbt);
     const cudaError_t attr = allow_smem(kernel, kSmemCap);
     if (attr != cudaSuccess) return attr;
     cudaLaunchAttribute at[1];
@@ -842,7 +942,7 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     const int nwords = (a.ngroups + 1) * kBarWords;
     const size_t bar_bytes = up(size_t(nwords) * 4);
     const size_t cbytes = kGru || a.c_on_chip || c_last ? 0 : up(size_t(H) * size_t(B) * 4);
-    const size_t hx_bytes = up(2 * size_t(a.ntiles) * size_t(a.hrows) * bt * 4);
+    const size_t hx_bytes = up(2 * size_t(a.ntiles) * size_t(a.hrows) * bt * (a.tagged ? 8 : 4));
     const bool x_copy = a.x_mode == kXBulk && !x_in_place;
     const size_t ws_bytes = bar_bytes + cbytes + hx_bytes + (pre ? pre_bytes : 0) + (x_copy ? up(xt_bytes) : 0);
     char *ws = nullptr;

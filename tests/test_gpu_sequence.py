@@ -354,3 +354,9 @@ def test_barrier_timeout_is_reported_and_the_device_stays_usable(cell, I, H, B, 
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
+
+
+def test_barrier_timeout_of_a_wide_tile(monkeypatch):
+    """The same where h is exchanged behind the barrier (tiles of more than 32 KB)
+    instead of with tags."""
+    test_barrier_timeout_is_reported_and_the_device_stays_usable("lstm", 20, 1100, 8, monkeypatch)
