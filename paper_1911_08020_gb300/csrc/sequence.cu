@@ -301,8 +301,8 @@ __device__ __forceinline__ void reduce_store(float (&acc)[Lanes<LBT>::V], int la
     if ((lane & rest) == 0) part[col] = v;
 }
 
-// Thread 0's wait for the arrivals of its group; false if it gave up or
-// another CTA did.  The CTA barrier before an arrival orders every thread's
+// A warp's wait for the arrivals of its group; false if it gave up or another
+// CTA did.  The CTA barrier before an arrival orders every thread's
 // h_t stores before it; the arrival is a release reduction on the counter (no
 // return trip, no separate fence).  An acquire that reads the final count
 // synchronises with every arrival (each is a read-modify-write in the
@@ -385,20 +385,24 @@ __device__ __forceinline__ bool stage_tagged(const SeqArgs &a, const float *h_x,
 
 // A tile of `bytes` (a multiple of 16): one warp, each of its first kCopies
 // lanes a bulk copy that completes on `bar` (one thread issuing all of them
-// took 1400 cycles of a step).  Lane 0 arms `bar`
-// first.
-__device__ __forceinline__ void copy_tile(int lane, float *dst, const float *src, uint32_t bytes, uint64_t *bar) {
+// took 1400 cycles of a step).  `ready` is called by the whole warp between
+// arming `bar` and the copies: what only has to be done is done before it.
+template <class Ready>
+__device__ __forceinline__ void copy_tile(int lane, float *dst, const float *src, uint32_t bytes, uint64_t *bar,
+                                          Ready ready) {
     // every thread of this CTA is done with the previous tile (the barrier
-    // that ended it); order those reads, and what other CTAs published by
-    // generic stores, before the copies
+    // that ended it); order those reads before the copies
     fence_proxy_async_smem();
-    fence_proxy_async_global();
     if (lane == 0) mbar_arrive_expect_tx(bar, bytes);
-    __syncwarp();
     const uint32_t each = (bytes / kCopies + 127) & ~127u, at = uint32_t(lane) * each;
-    if (lane < kCopies && at < bytes)
-        bulk_g2s(reinterpret_cast<char *>(dst) + at, reinterpret_cast<const char *>(src) + at,
-                 lane == kCopies - 1 || bytes - at < each ? bytes - at : each, bar);
+    const bool has = lane < kCopies && at < bytes;
+    const uint32_t size = lane == kCopies - 1 || bytes - at < each ? bytes - at : each;
+    char *d = reinterpret_cast<char *>(dst) + at;
+    const char *s = reinterpret_cast<const char *>(src) + at;
+    __syncwarp();
+    ready();
+    fence_proxy_async_global();   // what other CTAs published by generic stores, too
+    if (has) bulk_g2s(d, s, size, bar);
 }
 
 template <bool BF16, int MODE, int LBT, bool TAGGED>
@@ -554,7 +558,8 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
     const uint32_t xbytes = uint32_t(a.irows) * bt * 4, hbytes = uint32_t(a.hrows) * bt * 4;
     // x_t of one tile (the last warp): its rows are free once the tile before has been multiplied
     auto copy_x = [&](int t, int tile) {
-        copy_tile(lane, s_in, a.x_tiles + (int64_t(t) * a.ntiles + tile) * (int64_t(a.irows) << LBT), xbytes, &s_xfull);
+        copy_tile(lane, s_in, a.x_tiles + (int64_t(t) * a.ntiles + tile) * (int64_t(a.irows) << LBT), xbytes, &s_xfull,
+                  [] {});
     };
     const bool xbulk = a.x_mode == kXBulk;
     if (xbulk && warp == kSeqWarps - 1) copy_x(0, group);
@@ -587,16 +592,13 @@ seq_kernel(Format f, SeqArgs a, Ranges rg, SmemPlan sp) {
                      : n2 <= 4 * kThreads ? stage_tagged<4>(a, a.h_x, first, n2, tag, dst)
                                           : stage_tagged<8>(a, a.h_x, first, n2, tag, dst);
             } else if (warp == 0) {
-                int go = 1;
-                if (lane == 0 && k == 0 && t > 0) go = wait_arrivals(a, bar, unsigned(t) * members);
-                if (__shfl_sync(0xFFFFFFFFu, go, 0)) {
-                    copy_tile(lane, s_in + (a.irows << LBT),
-                              a.h_x + (int64_t((t + 1) & 1) * a.ntiles + tile) * (int64_t(a.hrows) << LBT), hbytes,
-                              &s_hfull);
-                } else if (lane == 0) {
-                    s_fail = 1;
-                    mbar_arrive(&s_hfull);   // no copy comes: let the waiting threads see s_fail
-                }
+                // a wait that gives up sets s_fail; its copies are harmless and let
+                // the waiting threads get there
+                copy_tile(lane, s_in + (a.irows << LBT),
+                          a.h_x + (int64_t((t + 1) & 1) * a.ntiles + tile) * (int64_t(a.hrows) << LBT), hbytes, &s_hfull,
+                          [&] {
+                              if (k == 0 && t > 0 && !wait_arrivals(a, bar, unsigned(t) * members)) s_fail = 1;
+                          });
             }
             if (TAGGED || a.x_mode == kXPlain) __syncthreads();
             if (!TAGGED) ok = mbar_wait(&s_hfull, staged & 1);
