@@ -34,11 +34,11 @@
 // A plain product (kModeY; the rows are the units, X the whole input) takes
 // this kernel from batch 5 on while it is expected to be faster than the
 // kernels that stream through clusters, whose fixed part is larger but whose
-// gather is cheaper: us against batch_kernel (batch 6, 8) and xres (the
-// others), 1024 x 1024 fp32 at batch 6 / 8 / 24 / 64: 3.9 / 3.7 / 3.9 / 4.4
-// against 27.6 / 4.9 / 10.2 / 10.2; 6000 x 3000 fp32 at 6 / 8 / 16: 8.7 / 7.4 /
-// 9.7 against 80 / 15 / 14, but 16.2 against 11.8 at 32; 2000 x 2500 fp32 at
-// 24 / 64 / 100: 6.7 / 9.2 / 13.4 against 12.2 / 11.8 / 13.0.
+// gather is cheaper.  us against what those took: 1024 x 1024 fp32 at batch 6 /
+// 8 / 24 / 64: 4.0 / 3.7 / 4.0 / 4.4 against 27.6 / 4.9 / 10.2 / 10.1; 6000 x
+// 3000 fp32 at 6 / 8 / 16: 8.7 / 7.4 / 9.7 against 80 / 15 / 14, but 16.2 against
+// 11.8 at 32; 2000 x 2500 fp32 at 24 / 64: 6.3 / 9.1 against 12.2 / 11.7, but
+// 13.4 against 13.0 at 100; 4096 x 4096 bf16 at 8: 5.6 against 8.2.
 #pragma once
 
 #include "kernels_common.cuh"
@@ -466,7 +466,9 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
         static const double kCycles[2][kMaxLbt - kMinLbt + 1] = {{0.9, 1.0, 1.35, 1.5}, {0.9, 0.95, 1.45, 2.4}};
         const int waves = (p.ntiles * p.members + sms - 1) / sms;
         const double bytes = double(K) * bt * 4;
-        const double staging = MODE == kModeY ? bytes / 250.0 + std::max(0.0, bytes - 98304.0) / 100.0 : bytes / 70.0;
+        const double half_sectors = l == 2 && ra.B > 4 && ra.B % 4 == 0 ? bytes / 100.0 : 0.0;   // 16 of 32 bytes a row
+        const double staging = MODE == kModeY ? bytes / 250.0 + half_sectors + std::max(0.0, bytes - 98304.0) / 100.0
+                                              : bytes / 70.0;
         const double ns = 3200.0 + waves * (staging + kept / p.members * kCycles[MODE == kModeY][l - kMinLbt] / 1.9 +
                                             (MODE == kModeY ? double(units) * bt / kThreads * 250.0 : 0.0));
         if (ns < best_ns) {

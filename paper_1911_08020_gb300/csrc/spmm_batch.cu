@@ -10,24 +10,32 @@
 #include "batch.cuh"
 #include "xres.cuh"
 
+#include <algorithm>
+
 namespace darb {
 
 cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y,
                               int64_t ldy, bool early, cudaStream_t stream) {
-    // what the cluster kernels take: a fixed part (for xres larger with the
-    // columns, and with plain copies of unaligned X) and 1.5 times the time of
-    // the gather at 128 bytes a clock and SM, over whole 32-column tiles.
-    // (Fitted to products of 300 to 9216 columns.  Where the two estimates meet
-    // the kernels differ by up to 4% the other way: 700 x 6000 fp32 at batch
-    // 16 takes 8.0 us against 7.7.)
+    // What the cluster kernels take, fitted to products of 300 to 9216 columns
+    // (where two estimates meet, the kernels differ by a few percent either
+    // way), from the time of the gather at 128 bytes a clock and SM over whole
+    // 32-column tiles.  batch_kernel: a fixed part and 1.5 times the gather (2.3
+    // times for fp32 weights).  xres: a fixed part, the load of a slice of the
+    // columns (slower by plain copies) and the longer of its share of the
+    // gather and of its heaviest unit, two groups of the smallest block size.
     const bool aligned = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
+    const bool streams = batch <= 16 && aligned;   // batch_kernel, else xres
     const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
     const double gather_ns = kept * double((batch + 31) / 32) * 128.0 / (128.0 * 2.0 * sm_count());
-    const double others_ns = (batch > 16 ? 6500.0 + 0.3 * double(f.cols) : 5500.0) + (aligned ? 0.0 : 1500.0) + 1.5 * gather_ns;
+    const double slices = double((f.cols + 1399) / 1400);
+    const double unit_ns = 0.75 * 137.0 * (2.0 * f.nch_max / slices + 12.0);
+    const double others_ns = streams ? 4600.0 + (f.bf16 ? 1.5 : 2.3) * gather_ns
+                                     : 0.95 * (3000.0 + (aligned ? 0.0 : 2500.0) + 1.66 * double(f.cols) / slices +
+                                               std::max(unit_ns, 1.6 * gather_ns));
     cudaError_t e = launch_spmm_rows(f, X, ldx, batch, Y, ldy, early, others_ns, stream);
     if (e != cudaErrorNotSupported) return e;
     cudaGetLastError();
-    if (batch > 16 || !aligned) {
+    if (!streams) {
         e = f.bf16 ? xres::launch<true, 32>(f, X, ldx, batch, Y, ldy, early, stream)
                    : xres::launch<false, 32>(f, X, ldx, batch, Y, ldy, early, stream);
         if (e != cudaErrorNotSupported) return e;

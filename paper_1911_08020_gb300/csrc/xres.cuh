@@ -660,13 +660,14 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
     // splits with kMinStages or more, the one whose clusters occupy the most
     // SMs, then the deeper ring, then the smaller split; a shallower ring only
     // when no split has that.  Where that leaves its clusters with fewer than
-    // two units, most SMs idle while a unit runs: the split that is expected to
-    // take the least time then, if it is well below (in group-chunks of
+    // two units, most SMs idle while a unit runs: a finer split that is expected
+    // to take the least time then, if it is well below (in group-chunks of
     // multiplying, 137 ns: the load of the slice, and the units of a cluster,
     // each its share of the set's work and a fixed cost; more where partial sums
-    // cross CTAs).  512 x 4000 bf16 at
-    // batch 64: 9.0 us against 13.8, 2000 x 2500 fp32 at 64: 8.9 against 11.8.
-    // By that estimate alone 5000 x 700 at batch 256 went from 18.0 to 20.1.
+    // cross CTAs).  1000 x 7000 bf16 at batch 24: 8.5 us against 10.8, 2000 x
+    // 5000 at 64: 10.4 against 11.2.  By that estimate alone 5000 x 700 at
+    // batch 256 went from 18.0 to 20.1, and a coarser split has longer chains
+    // of fp32 additions (1500 x 1500 at 100: 1.38 times the error).
     struct Split {
         Plan p;
         uint32_t smem;
@@ -714,7 +715,7 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
         }
         if (least.sms == 0 || (s.deep != least.deep ? s.deep : s.cost < least.cost)) least = s;
     }
-    const Split &best = few && least.deep == most.deep && least.cost < 0.85 * most.cost ? least : most;
+    const Split &best = few && least.p.C > most.p.C && least.deep == most.deep && least.cost < 0.85 * most.cost ? least : most;
     Plan p = best.p;
     const uint32_t smem = best.smem;
     const int64_t best_sms = best.sms;
