@@ -120,16 +120,6 @@ __device__ __forceinline__ void tensor2d_g2s(void *dst, const void *tmap, int x,
         ::"r"(smem_addr(dst)), "l"(tmap), "r"(x), "r"(y), "r"(smem_addr(bar)) : "memory");
 }
 
-// 3-D tensor-map copy (box at coordinates x = innermost, y, z) -> this CTA's
-// shared memory, completing on `bar`.  x * element size must be a multiple of
-// 16 bytes; dst 128-byte aligned.
-__device__ __forceinline__ void tensor3d_g2s(void *dst, const void *tmap, int x, int y, int z, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_addr(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar)) : "memory");
-}
-
 // Order this thread's earlier generic-proxy view of global memory (e.g. data
 // other CTAs published through a release/acquire handshake) before its later
 // async-proxy (TMA) reads.
@@ -174,12 +164,6 @@ __device__ __forceinline__ bool mbar_wait_acq_cluster(uint64_t *bar, uint32_t pa
             if (sleep_ns < 512) sleep_ns <<= 1;
         }
     }
-}
-
-// Named barrier `id` (1..15) over `threads` threads of the CTA (a multiple of
-// 32; the warps that take part all call it with the same id and count).
-__device__ __forceinline__ void named_sync(uint32_t id, uint32_t threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // Programmatic dependent launch: let the next kernel on the stream start its
