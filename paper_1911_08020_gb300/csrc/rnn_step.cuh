@@ -432,6 +432,7 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
     if (K > 60000 || ra.B > 1024 || f.nitems[0][0] <= 0) return cudaErrorNotSupported;
     // kept weights of the matrix, padded to whole groups and chunks
     const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
+    if (kept > 8e9) return cudaErrorNotSupported;   // Row's indices of records and offset words are 32-bit
     const int sms = sm_count();
     int lbt = -1;
     size_t smem = 0;
