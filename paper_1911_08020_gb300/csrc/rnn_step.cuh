@@ -26,9 +26,9 @@
 // with the launch) and, for wide matrices, the gather.  A step (us, in a graph
 // of steps) against the kernels whose gate sums meet through clusters, scratch
 // and counters (rowlane_kernel, batch_kernel): LSTM 4096 x 1280 fp32 at batch
-// 1 / 8 / 32 / 64: 6.2 / 5.9 / 7.8 / 11.1 against 7.8 / 17.0 / 25.0 / 30.3; GRU
-// 3072 x 2048 bf16 at batch 64: 11.5 against 32.3; LSTM 6000 x 3000 bf16 at
-// batch 20: 16.5 against 37.9, fp32 at batch 37: 30 against 212.  Those kernels
+// 1 / 8 / 32 / 64: 6.3 / 5.8 / 7.6 / 10.5 against 7.8 / 17.0 / 25.0 / 30.3; GRU
+// 3072 x 2048 bf16 at batch 64: 10.9 against 32.3; LSTM 6000 x 3000 bf16 at
+// batch 20: 16.0 against 37.9, fp32 at batch 37: 27.5 against 212.  Those kernels
 // remain for inputs too tall to stage at 4 columns (some 14000 rows).
 //
 // A plain product (kModeY; the rows are the units, X the whole input) takes
@@ -174,7 +174,9 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
     struct Fetch {
         uint32_t vw[kW];
         uint2 ow;
-        int v, c;   // row of the stream (-1: none) and chunk
+        int v;          // row of the stream (-1: none)
+        int m, kb;      // its block size and the chunk's first column
+        bool whole;     // all of the chunk's blocks lie inside the row's columns
     };
     Fetch buf[kAhead];
     int lv = 0;     // row of the next chunk to request
@@ -186,18 +188,25 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
             else hi = mid;
         }
     }
+    // the row of the next chunk to request stays in registers (read from shared
+    // memory for each chunk: GRU 3072 x 2048 at batch 64 11.5 us against 10.9)
+    Row row = s_row[lv];
+    int row_end = s_row[lv + 1].at;
     auto fetch = [&](int i, Fetch &b) {   // chunk i of the stream
         b.v = -1;
         if (i >= end) return;
-        while (s_row[lv + 1].at <= i) ++lv;
-        const uint4 *rw = reinterpret_cast<const uint4 *>(s_row + lv);
-        const uint4 q = rw[0];
-        const int at = s_row[lv].at;
-        const int c = int(q.z) + i - at;
-        const bool nib = q.w >> 16;
+        if (i >= row_end) {
+            do row_end = s_row[++lv + 1].at;
+            while (i >= row_end);
+            row = s_row[lv];
+        }
+        const int c = row.c0 + i - row.at, m = row.m_nib & 0xFFFF;
+        const bool nib = row.m_nib >> 16;
         b.v = lv;
-        b.c = c;
-        const uint4 *pv = static_cast<const uint4 *>(f.vals) + int64_t(q.x + uint32_t(c) * kSlots) * (BF16 ? 1 : 2);
+        b.m = m;
+        b.kb = c * kChunk * m;
+        b.whole = b.kb >= row.klo && b.kb + kChunk * m <= row.khi;
+        const uint4 *pv = static_cast<const uint4 *>(f.vals) + int64_t(row.rec + uint32_t(c) * kSlots) * (BF16 ? 1 : 2);
         const uint4 w0 = __ldg(pv);
         b.vw[0] = w0.x; b.vw[1] = w0.y; b.vw[2] = w0.z; b.vw[3] = w0.w;
         if constexpr (!BF16) {
@@ -205,11 +214,11 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
             b.vw[4] = w1.x; b.vw[5] = w1.y; b.vw[6] = w1.z; b.vw[7] = w1.w;
         }
         if (nib) {
-            const uint32_t w = __ldg(f.offs + q.y + uint32_t(c) * kSlots);
+            const uint32_t w = __ldg(f.offs + row.off + uint32_t(c) * kSlots);
             const uint32_t even = w & 0x0F0F0F0Fu, odd = (w >> 4) & 0x0F0F0F0Fu;
             b.ow = make_uint2(__byte_perm(even, odd, 0x5140), __byte_perm(even, odd, 0x7362));
         } else {
-            b.ow = __ldg(reinterpret_cast<const uint2 *>(f.offs + q.y + uint32_t(c) * (2 * kSlots)));
+            b.ow = __ldg(reinterpret_cast<const uint2 *>(f.offs + row.off + uint32_t(c) * (2 * kSlots)));
         }
     };
     if (p.early) {
@@ -283,8 +292,7 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
             acc = make_float4(0.f, 0.f, 0.f, 0.f);
             cur = b.v;
         }
-        const int m = s_row[b.v].m_nib & 0xFFFF, klo = s_row[b.v].klo, khi = s_row[b.v].khi;
-        const int kb = b.c * kChunk * m;
+        const int m = b.m, kb = b.kb;
         // a chunk's products are added by themselves first: the chain of fp32
         // additions of a run stays short
         float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
@@ -299,7 +307,7 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
                          : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(ad));
             return x;
         };
-        if (kb >= klo && kb + kChunk * m <= khi) {
+        if (b.whole) {
             const uint32_t xb = xl + (uint32_t(kb) << kRowShift), step = uint32_t(m) << kRowShift;
             float4 x[kChunk];
 #pragma unroll
@@ -308,6 +316,7 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
 #pragma unroll
             for (int e = 0; e < kChunk; ++e) fma4((e & 1) ? s1 : s0, weight(e), x[e]);
         } else {
+            const int klo = s_row[b.v].klo, khi = s_row[b.v].khi;
 #pragma unroll
             for (int e = 0; e < kChunk; ++e) {
                 const int k = kb + e * m + int((e < 4 ? b.ow.x : b.ow.y) >> (8 * (e & 3)) & 255u);
