@@ -35,9 +35,9 @@
 // staging 2500, the cell 1800.  One column group instead of one a tile stages
 // every column in every CTA: GRU 3072 x 2048 at batch 64 took 11.0 against 8.7
 // us a step.  Against one lane a column, tensor-map staging and all CTAs in one
-// barrier, whole calls went from 3131 to 1512 us (that GRU, 200 steps), 507 to
-// 332 (the LSTM above, 35 steps), 520 to 321 (LSTM 4096 x 1280 fp32, batch 1,
-// 100 steps), and 2592 to 588 where the batch is no multiple of 4 (GRU 2100 x
+// barrier, whole calls went from 3131 to 1505 us (that GRU, 200 steps), 507 to
+// 329 (the LSTM above, 35 steps), 520 to 309 (LSTM 4096 x 1280 fp32, batch 1,
+// 100 steps), and 2592 to 545 where the batch is no multiple of 4 (GRU 2100 x
 // 1000, batch 37, 100 steps).
 #include "darb_internal.h"
 #include "kernels_common.cuh"
@@ -228,7 +228,9 @@ __device__ __forceinline__ void dot_range(const typename P::T *s_w, const float 
     float4 s[A];   // (V < 4: the first V of each)
 #pragma unroll
     for (int i = 0; i < A; ++i) s[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
+    // (not unrolled further: a step runs through its code once, and the fetch of
+    // more of it costs more than the overlap gives; by 2: 1 to 5% slower)
+#pragma unroll 1
     for (int p = pa + KW * sub; p < pb; p += U * kStep) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
