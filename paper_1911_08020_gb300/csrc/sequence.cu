@@ -43,6 +43,7 @@
 #include "kernels_common.cuh"
 #include "launch.cuh"
 #include "rnn_epilogue.cuh"
+#include "sequence_rows.h"
 #include "tma.cuh"
 
 #include <algorithm>
@@ -716,18 +717,18 @@ __global__ void __launch_bounds__(256) prep_kernel(SeqArgs a, int lbt, const flo
         }
     }
     for (int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5); row < nrows; row += int64_t(gridDim.x) * 8) {
+        const PrepRow r = prep_row(row, a.H, a.I);
         const int64_t xrow = row - a.H;
-        const int64_t t = xrow / a.I, k = xrow < 0 ? row : xrow % a.I;
-        if (xrow >= 0 && xall != nullptr) {
-            for (int64_t b = lane; b < B; b += 32) xall[k * ldxall + t * B + b] = __ldg(a.x + xrow * B + b);
+        if (r.of_x && xall != nullptr) {
+            for (int64_t b = lane; b < B; b += 32) xall[r.k * ldxall + r.t * B + b] = __ldg(a.x + xrow * B + b);
             continue;
         }
-        const float *src = xrow < 0 ? h0 + row * B : a.x + xrow * B;
-        const int nr = xrow < 0 ? a.hrows : a.irows;   // rows of a tile
-        float *dst = (xrow < 0 ? a.h_x + ((int64_t(a.ntiles) * nr) << lbt) : x_tiles + ((t * a.ntiles * nr) << lbt)) +
-                     (k << lbt);
-        if (xrow < 0 && a.tagged) {
-            uint64_t *d = reinterpret_cast<uint64_t *>(a.h_x) + ((int64_t(a.ntiles) * nr) << lbt) + (k << lbt);
+        const float *src = r.of_x ? a.x + xrow * B : h0 + row * B;
+        const int nr = r.of_x ? a.irows : a.hrows;   // rows of a tile
+        float *dst = (r.of_x ? x_tiles + ((r.t * a.ntiles * nr) << lbt) : a.h_x + ((int64_t(a.ntiles) * nr) << lbt)) +
+                     (r.k << lbt);
+        if (!r.of_x && a.tagged) {
+            uint64_t *d = reinterpret_cast<uint64_t *>(a.h_x) + ((int64_t(a.ntiles) * nr) << lbt) + (r.k << lbt);
             for (int64_t b = lane; b < (int64_t(a.ntiles) << lbt); b += 32)
                 d[(((b >> lbt) * nr) << lbt) + (b & (bt - 1))] =
                     uint64_t(1) << 32 | (b < B ? __float_as_uint(__ldg(src + b)) : 0u);
