@@ -41,6 +41,7 @@ struct darb_handle_s {
     int32_t xset_first[darb::kXresTables] = {}, nxsets[darb::kXresTables] = {};
     std::vector<int64_t> xset_prefix[darb::kXresTables];
     darb::SetGeo *d_xsets = nullptr;
+    darb::UnitSplits splits[darb::kUnitKinds];            // of rnn_step.cuh
     int64_t val_elems = 0, off_words = 0;
     // device memory: one allocation holding the layout, values and offsets
     void *dmem = nullptr;
@@ -154,6 +155,21 @@ void build_layout(darb_handle_s *h, const int32_t *m) {
     h->val_elems = val;
     h->off_words = off;
     build_work_tables(h);
+    // a row costs its chunks, and about one more to form its outputs
+    std::vector<int32_t> row_cost(static_cast<size_t>(rows));
+    for (int64_t r = 0; r < rows; ++r)
+        row_cost[static_cast<size_t>(r)] =
+            (h->groups[static_cast<size_t>(h->rowloc[static_cast<size_t>(r)] / kSlots)].n + kChunk - 1) / kChunk + 1;
+    for (int kind = 0; kind < darb::kUnitKinds; ++kind) {
+        const int64_t gates = kind == darb::kUnitRow ? 1 : kind == darb::kUnitLstm ? 4 : 3;
+        if (rows % gates != 0) continue;
+        const int64_t units = rows / gates;
+        h->splits[kind].build(units, [&](int64_t u) {
+            int64_t c = 0;
+            for (int64_t q = 0; q < gates; ++q) c += row_cost[static_cast<size_t>(q * units + u)];
+            return c;
+        });
+    }
     // tiles of tb(m) blocks, every row in order; tb a multiple of the chunk
     auto tiles_of = [h, rows, cols](std::vector<darb::EncTile> &out, int (*tb_of)(int)) {
         out.clear();
@@ -389,6 +405,7 @@ Format format_of(const darb_handle_s *h) {
         f.xset_prefix[i] = h->xset_prefix[i].data();
         f.xsets_host[i] = h->xsets.data() + h->xset_first[i];
     }
+    for (int k = 0; k < darb::kUnitKinds; ++k) f.splits[k] = &h->splits[k];
     f.ngroups = static_cast<int32_t>(h->groups.size());
     f.bf16 = h->wtype == DARB_BF16 ? 1 : 0;
     f.m_max = h->groups.empty() ? 1 : h->groups.back().m;   // groups are sorted by block size

@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include "darb.h"
+#include "unit_split.h"
 
 namespace darb {
 
@@ -84,6 +85,10 @@ constexpr int kXresTables = 2;   // row-set tables of xres: 2 and 4 groups of th
 constexpr int kXresMaxGroups = 4;
 constexpr int kWorkSplits = 4;   // clusters of 1, 2, 4, 8 CTAs
 
+// What a unit of rnn_step.cuh is: a row, or a hidden unit of an LSTM (4 gate
+// rows) or a GRU (3).
+constexpr int kUnitRow = 0, kUnitLstm = 1, kUnitGru = 2, kUnitKinds = 3;
+
 // Everything a kernel needs to read an encoded matrix.
 struct Format {
     const Group *groups;
@@ -111,6 +116,9 @@ struct Format {
     int32_t nxsets[kXresTables];
     const int64_t *xset_prefix[kXresTables];
     const SetGeo *xsets_host[kXresTables];   // HOST copies of xsets
+    // HOST: the units' costs and splits, by kUnit* (of a cell: only when the rows
+    // divide by its gates)
+    const UnitSplits *splits[kUnitKinds];
     int32_t ngroups;
     int32_t bf16;            // value dtype: 0 fp32, 1 bf16
     int32_t m_max;           // largest block size of any row

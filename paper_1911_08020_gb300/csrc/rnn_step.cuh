@@ -5,7 +5,10 @@
 // The batch columns are cut into tiles of bt columns, and the CTAs into one
 // group a tile; within a group every CTA owns a contiguous range of hidden
 // units with all their gate rows, so no gate sum leaves its CTA: no cluster,
-// no scratch, no counters.  A CTA
+// no scratch, no counters.  The ranges cost about the same (unit_split.h; with
+// equal numbers of units instead, 6000 x 3000 fp32 at batch 16 with its first
+// tenth of the rows in blocks of 4 and the rest of 64 took 28.0 us against 8.2,
+// and rows of mixed blocks 5% more).  A CTA
 //  * reads its rows' places in the format and, when the handle is complete,
 //    starts on their first records before the PDL wait;
 //  * stages the tile's columns of x_t and h_{t-1} whole (tensor-map boxes, or
@@ -79,12 +82,14 @@ struct Plan {
     int staging, early;           // kStage*; the records may be read before the PDL wait
     int nbx, bxh, nbh, bhh;       // boxes of x and h: their number and rows (the last one ends with the matrix)
     uint32_t row_off, nseg_off, bias_off, c_off, in_off, part_off;
+    int by_cost;                  // the members' units: start's ranges, else equal numbers (unit_split.h)
+    int start[kMaxMembers + 1];
 };
 
 template <bool BF16, int MODE, int LBT>
 __global__ void __launch_bounds__(kThreads, 1)
 step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mh,
-            Plan p) {
+            const __grid_constant__ Plan p) {
     constexpr int kGates = MODE == kModeLstm ? 4 : MODE == kModeGru ? 3 : 1;
     constexpr bool kGru = MODE == kModeGru;
     constexpr int kSides = kGru ? 2 : 1;
@@ -106,8 +111,8 @@ step_kernel(Format f, RnnArgs ra, const __grid_constant__ CUtensorMap mx, const 
     const int H = ra.H, I = ra.I, K = MODE == kModeY ? I : I + H;   // kModeY: H rows, I columns
     const int64_t B = ra.B, ldx = MODE == kModeY ? p.ldx : B, b0 = int64_t(tile) << LBT;
     const int nb = static_cast<int>(B - b0 < bt ? B - b0 : bt);
-    const int u0 = static_cast<int>(int64_t(H) * member / p.members);
-    const int nu = static_cast<int>(int64_t(H) * (member + 1) / p.members) - u0;
+    const int u0 = p.by_cost ? p.start[member] : static_cast<int>(int64_t(H) * member / p.members);
+    const int nu = (p.by_cost ? p.start[member + 1] : static_cast<int>(int64_t(H) * (member + 1) / p.members)) - u0;
     const int R = kGates * nu, VR = kSides * R;   // local row q*nu + i is matrix row q*H + u0 + i
     auto grow = [&](int lr) { return (lr / nu) * H + u0 + lr % nu; };
 
@@ -391,6 +396,36 @@ inline void boxes(int n, int *nbox, int *rows) {
     *nbox = n > 0 ? (n + *rows - 1) / *rows : 0;
 }
 
+// Whether x and h_{t-1} (or X) can be staged by copies of 16 bytes.
+inline bool aligned16(const RnnArgs &ra, bool product, int64_t ldx) {
+    return ra.B % 4 == 0 && ldx % 4 == 0 && (ra.I == 0 || reinterpret_cast<uintptr_t>(ra.x) % 16 == 0) &&
+           (product || reinterpret_cast<uintptr_t>(ra.h) % 16 == 0);
+}
+
+// What a tile is expected to take, ns: a fixed part (launch, latencies), the
+// staged bytes by the way they are copied (4 or 16 bytes at a time, or boxes;
+// 16-byte copies cost more where the last tile is ragged, or where the tile is
+// part of a row), the kept weights of the busiest member (8 a chunk of its
+// cost), and its outputs (cell updates of a step).  A narrow tile stages less,
+// but its staged rows share banks and each CTA multiplies more weights.
+struct TileCost {
+    double fixed, stage4, stage16, boxes, ragged, part, weight, output;
+};
+// Fitted to the forced tiles of 47 product shapes (128 to 6000 rows of 300 to
+// 9216 columns, block sizes mixed and in runs) at 26 batches from 5 to 256, and
+// of 36 gate matrices (192 to 20000 rows, inputs of 192 to 13024 rows) at 27
+// batches from 1 to 128: 6 to 9% root mean square, at worst a third off.
+constexpr TileCost kProductCost[kMaxLbt - kMinLbt + 1] = {
+    {3156, 0.0189, 0.0272, 0, 0, 0, 0.304, 0.358},
+    {3098, 0.0173, 0.0035, 0, 0.0089, 0.0089, 0.445, 0.181},
+    {3031, 0.0165, 0.0048, 0, 0.0073, 0, 0.682, 0.118},
+    {3143, 0.0141, 0, 0.0039, 0.0048, 0, 1.247, 0.017}};
+constexpr TileCost kStepCost[kMaxLbt - kMinLbt + 1] = {
+    {4407, 0.0286, 0.0085, 0, 0, 0.0282, 0.270, 3.23},
+    {4425, 0.0253, 0.0043, 0, 0.0047, 0.0123, 0.395, 1.93},
+    {4509, 0.0227, 0.0043, 0, 0.0043, 0, 0.573, 1.86},
+    {4389, 0.0241, 0, 0.0013, 0.0058, 0.0013, 0.768, 2.81}};
+
 template <bool BF16, int MODE, int LBT>
 cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem, cudaStream_t stream) {
     constexpr int bt = 1 << LBT;
@@ -406,8 +441,7 @@ cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem,
     // batch 8 6.0 against 7.3 us, 6000 x 3000 at batch 20 17.5 against 21.6),
     // the rest 4 bytes at a time
     const int64_t ldx = MODE == kModeY ? p.ldx : ra.B;
-    const bool aligned = ra.B % 4 == 0 && ldx % 4 == 0 && (ra.I == 0 || reinterpret_cast<uintptr_t>(ra.x) % 16 == 0) &&
-                         (MODE == kModeY || reinterpret_cast<uintptr_t>(ra.h) % 16 == 0);
+    const bool aligned = aligned16(ra, MODE == kModeY, ldx);
     p.staging = aligned ? kStage16 : kStage4;
     if (LBT == 5 && aligned && ra.B % bt == 0 && tensor_map_encoder() != nullptr) {
         auto make = [&](CUtensorMap *m, const float *base, int rows, int boxh, int64_t ld) {
@@ -440,55 +474,71 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
     const int64_t K = MODE == kModeY ? ra.I : int64_t(ra.I) + ra.H;
     if (K > 60000 || ra.B > 1024 || f.nitems[0][0] <= 0) return cudaErrorNotSupported;
     // kept weights of the matrix, padded to whole groups and chunks
-    const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
-    if (kept > 8e9) return cudaErrorNotSupported;   // Row's indices of records and offset words are 32-bit
+    if (double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk > 8e9) return cudaErrorNotSupported;   // Row's indices of records and offset words are 32-bit
+    const UnitSplits &splits = *f.splits[MODE == kModeLstm ? kUnitLstm : MODE == kModeGru ? kUnitGru : kUnitRow];
     const int sms = sm_count();
+    const bool aligned = aligned16(ra, MODE == kModeY, MODE == kModeY ? ldx : ra.B);
     int lbt = -1;
     size_t smem = 0;
     Plan best{};
     double best_ns = limit_ns;
-    for (int l = kMinLbt; l <= kMaxLbt && (l == kMinLbt || (1 << (l - 1)) < ra.B); ++l) {
-        const int bt = 1 << l;
-        Plan p{};
-        p.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
-        p.members = std::max(1, std::min(sms / p.ntiles, ra.H));
-        const int units = (ra.H + p.members - 1) / p.members;
+    // the places of a CTA's shared memory for members of up to `units` units, and
+    // its bytes (0: more rows than the kernel handles)
+    auto lay_out = [&](Plan &p, int units, int bt) -> size_t {
         const int vr = (MODE == kModeGru ? 2 : 1) * kGates * units, subs = kStepWarps * 128 / bt;
+        if (units > 4096 || vr > 4096) return 0;
         size_t o = 0;
         auto take = [&](size_t bytes) {
             const size_t at = o;
             o = (o + bytes + 127) / 128 * 128;
             return static_cast<uint32_t>(at);
         };
-        if (vr > 4096) continue;
         p.in_off = take(size_t(K + 1) * bt * 4);
         p.part_off = take(size_t(vr + subs) * bt * 4);
         p.row_off = take(size_t(vr + 1) * sizeof(Row));
         p.nseg_off = take(size_t(vr) * 4);
         p.bias_off = take(size_t(vr) * 4);
         p.c_off = take(MODE == kModeLstm ? size_t(units) * bt * 4 : 0);
-        if (o > kSmemCap) continue;
-        // launch and latencies, the staging of K rows, the gather, and a
-        // product's outputs.  A narrow tile stages less, but its staged rows
-        // share banks and each CTA multiplies more weights.  (Cycles a kept
-        // weight and staging rates fitted to steps, whose rows are long, and to
-        // products of 300 to 9216 columns at batch 2 to 256.)
-        static const double kCycles[2][kMaxLbt - kMinLbt + 1] = {{0.9, 1.0, 1.35, 1.5}, {0.9, 0.95, 1.45, 2.4}};
-        const int waves = (p.ntiles * p.members + sms - 1) / sms;
-        const double bytes = double(K) * bt * 4;
-        const double half_sectors = l == 2 && ra.B > 4 && ra.B % 4 == 0 ? bytes / 100.0 : 0.0;   // 16 of 32 bytes a row
-        const double staging = MODE == kModeY ? bytes / 250.0 + half_sectors + std::max(0.0, bytes - 98304.0) / 100.0
-                                              : bytes / 70.0;
-        const double ns = 3200.0 + waves * (staging + kept / p.members * kCycles[MODE == kModeY][l - kMinLbt] / 1.9 +
-                                            (MODE == kModeY ? double(units) * bt / kThreads * 250.0 : 0.0));
-        if (ns < best_ns) {
-            best_ns = ns;
-            best = p;
-            lbt = l;
-            smem = o;
+        return o;
+    };
+    for (int l = kMinLbt; l <= kMaxLbt && (l == kMinLbt || (1 << (l - 1)) < ra.B); ++l) {
+        const int bt = 1 << l;
+        Plan p{};
+        p.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
+        p.members = std::max(1, std::min({sms / p.ntiles, ra.H, kMaxMembers}));
+        UnitSplit local;
+        const UnitSplit &split = splits.get(p.members, local);
+        // ranges by cost give some members many light units, whose rows and partial
+        // sums may not fit; equal numbers then
+        for (int by_cost = split.prefer_by_cost ? 1 : 0; by_cost >= 0; --by_cost) {
+            const UnitRanges &r = by_cost ? split.by_cost : split.equal;
+            const size_t bytes = lay_out(p, r.most_units, bt);
+            if (bytes == 0 || bytes > kSmemCap) continue;
+            p.by_cost = by_cost;
+            const TileCost &cost = (MODE == kModeY ? kProductCost : kStepCost)[l - kMinLbt];
+            const bool ragged = ra.B % bt != 0;
+            const double per_byte = !aligned            ? cost.stage4
+                                    : l == 5 && !ragged ? cost.boxes
+                                                        : cost.stage16 + (ragged ? cost.ragged : 0) +
+                                                              (p.ntiles > 1 ? cost.part : 0);
+            const int waves = (p.ntiles * p.members + sms - 1) / sms;
+            const double ns = cost.fixed + waves * (double(K) * bt * 4 * per_byte + double(r.busiest) * kChunk * cost.weight +
+                                                    double(r.most_units) * bt * cost.output);
+            if (ns < best_ns) {
+                best_ns = ns;
+                best = p;
+                lbt = l;
+                smem = bytes;
+            }
+            break;
         }
     }
     if (lbt < 0) return cudaErrorNotSupported;
+    if (best.by_cost) {
+        UnitSplit local;
+        const UnitSplit &split = splits.get(best.members, local);
+        std::copy(split.start, split.start + best.members + 1, best.start);
+    }
     best.early = early ? 1 : 0;
     best.ldx = ldx;
     best.ldy = ldy;

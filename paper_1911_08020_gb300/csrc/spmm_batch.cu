@@ -16,23 +16,32 @@ namespace darb {
 
 cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y,
                               int64_t ldy, bool early, cudaStream_t stream) {
-    // What the cluster kernels take, fitted to products of 300 to 9216 columns
-    // (where two estimates meet, the kernels differ by a few percent either
-    // way), from the time of the gather at 128 bytes a clock and SM over whole
+    // What the cluster kernels take, fitted to products of 300 to 9216 columns,
+    // from the time of the gather at 128 bytes a clock and SM over whole
     // 32-column tiles.  batch_kernel: a fixed part and 1.5 times the gather (2.3
-    // times for fp32 weights).  xres: a fixed part, the load of a slice of the
-    // columns (slower by plain copies) and the longer of its share of the
+    // times for fp32 weights).  xres: the lesser of two readings, one from its
+    // split (xres::expected_ns) and one of a fixed part, the load of a slice of
+    // the columns (slower by plain copies) and the longer of its share of the
     // gather and of its heaviest unit, two groups of the smallest block size.
+    // The rows kernel has to be expected to take 5% less.  Over 611 products of
+    // 47 shapes, block sizes mixed and in runs, at 26 batches from 5 to 256,
+    // each timed on every kernel, the choice is on average 2% above the fastest;
+    // 9 were more than 3% above the cluster kernel, the worst 14% (4096 x 4096
+    // fp32 at batch 16, half the rows in blocks of 8 and half of 64: 12.3 us
+    // against 11.0).
     const bool aligned = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
     const bool streams = batch <= 16 && aligned;   // batch_kernel, else xres
     const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
     const double gather_ns = kept * double((batch + 31) / 32) * 128.0 / (128.0 * 2.0 * sm_count());
     const double slices = double((f.cols + 1399) / 1400);
     const double unit_ns = 0.75 * 137.0 * (2.0 * f.nch_max / slices + 12.0);
-    const double others_ns = streams ? 4600.0 + (f.bf16 ? 1.5 : 2.3) * gather_ns
-                                     : 0.95 * (3000.0 + (aligned ? 0.0 : 2500.0) + 1.66 * double(f.cols) / slices +
-                                               std::max(unit_ns, 1.6 * gather_ns));
-    cudaError_t e = launch_spmm_rows(f, X, ldx, batch, Y, ldy, early, others_ns, stream);
+    const double others_ns =
+        streams ? 4600.0 + (f.bf16 ? 1.5 : 2.3) * gather_ns
+                : std::min(0.95 * (3000.0 + (aligned ? 0.0 : 2500.0) + 1.66 * double(f.cols) / slices +
+                                   std::max(unit_ns, 1.6 * gather_ns)),
+                           f.bf16 ? xres::expected_ns<true, 32>(f, batch, aligned)
+                                  : xres::expected_ns<false, 32>(f, batch, aligned));
+    cudaError_t e = launch_spmm_rows(f, X, ldx, batch, Y, ldy, early, 0.95 * others_ns, stream);
     if (e != cudaErrorNotSupported) return e;
     cudaGetLastError();
     if (!streams) {

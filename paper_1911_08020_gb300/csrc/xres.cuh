@@ -820,6 +820,48 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
                      static_cast<unsigned>(p.C), true, f, X, ldx, batch, Y, ldy, xmap, p);
 }
 
+// What the product is expected to take here, ns (infinite where no split fits),
+// without the occupancy queries of launch_as: the load of a slice, the gather
+// of a cluster's share (at least its heaviest set) and a fixed part a unit, for
+// the split that launch_as is about to choose.  Fitted to 611 products of 47
+// shapes: 12% root mean square.
+template <bool BF16, int T>
+double expected_ns(const Format &f, int64_t batch, bool aligned) {
+    static constexpr int kResident[8] = {152, 76, 48, 36, 28, 23, 18, 15};   // clusters of C CTAs on 152 SMs
+    struct Split {
+        double slice, gather, units, cost;   // in group-chunks of multiplying (137 ns), units in number
+        int C, sms, nst;
+        bool few;
+    } most{}, least{};
+    const double tiles = double((batch + T - 1) / T);
+    for (int C = 1; C <= 8; ++C) {
+        const int64_t rows = (f.cols + C - 1) / C + f.m_max - 1;
+        const int64_t room = int64_t(kSmemCap) - kBarBytes - rows * (T * 4) - kMaxGroups * kSlots * T * 4;
+        const int nst = static_cast<int>(std::min<int64_t>(kMaxStages, room / int64_t(stage_bytes<BF16>())));
+        if (room < 0 || nst < 2) continue;
+        const double ncl = kResident[C - 1];
+        const int tb = tiles * f.nxsets[1] >= 2 * ncl ? 1 : 0;
+        const double nsets = f.nxsets[tb], work = double(f.xset_prefix[tb][f.nxsets[tb]]);
+        // groups of the heaviest set: as many as the bin of the smallest blocks fills
+        const double heaviest = double(f.xset_prefix[tb][1]);
+        Split s{};
+        s.slice = double(rows) * (T * 4 / (77.0 * 137.0));
+        s.gather = std::max(tiles * work / (C * ncl), heaviest / C);
+        s.units = std::ceil(tiles * nsets / ncl);
+        s.cost = s.slice + s.units * (work / (C * nsets) + 2 + kUnitCost) + (C > 1 ? kClusterCost : 0);
+        s.C = C;
+        s.sms = static_cast<int>(ncl) * C;
+        s.nst = nst;
+        s.few = tiles * nsets < 2 * ncl;
+        const bool deep = nst >= kMinStages, most_deep = most.nst >= kMinStages;
+        if (most.C == 0 || (deep != most_deep ? deep : s.sms != most.sms ? s.sms > most.sms : nst > most.nst)) most = s;
+        if (least.C == 0 || s.cost < least.cost) least = s;
+    }
+    if (most.C == 0) return 1e300;
+    const Split &s = most.few && least.C > most.C && least.cost < 0.85 * most.cost ? least : most;
+    return 2854.0 + (123.8 + (aligned ? 0.0 : 106.5)) * s.slice + 148.9 * s.gather + 1480.0 * s.units;
+}
+
 // The slices arrive by tensor maps where X allows one (16-byte aligned base
 // and rows, a row pitch the encoder takes), else by 4-byte copies of the
 // consumer warps, 128 bytes of a row per warp.  A slice of 192 KB then takes

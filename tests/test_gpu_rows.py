@@ -71,3 +71,25 @@ def test_unselected_activations_do_not_matter(B):
         assert_product_close(Y, Yr, A, TOL["f32"])
     finally:
         darb.darb_destroy(h)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rows,cols,sizes,B", [
+    (1024, 600, ((4, 102), (64, 922)), 8),       # the dense rows first: many rows for most CTAs, few for some
+    (700, 900, ((256, 500), (2, 200)), 33),      # and last, on several column tiles
+    (161, 400, ((1, 1), (256, 160)), 6),         # one row with most of the work; more rows than CTAs by a few
+])
+def test_product_of_rows_sorted_by_block_size(rows, cols, sizes, B, dtype):
+    """The CTAs' row ranges follow the rows' cost (unit_split.h)."""
+    g = np.random.default_rng(92)
+    w = (0.05 * g.standard_normal((rows, cols))).astype(np.float32)
+    stored = synth.f32_to_bf16_bits(w) if dtype == "bf16" else w
+    h, ref = encode_both(stored, np.concatenate([np.full(n, m, np.int32) for m, n in sizes]), dtype)
+    try:
+        X = synth.activations(cols, B, seed=B)
+        Y = darb.darb_spmm(h, t(X)).cpu().numpy()
+        darb.darb_sync_status(h)
+        Yr, A = oracle.darb_spmm(ref, X, with_absdot=True)
+        assert_product_close(Y, Yr, A, TOL["f32"])
+    finally:
+        darb.darb_destroy(h)

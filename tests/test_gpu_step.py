@@ -71,6 +71,34 @@ def test_step(cell, I, H, B, mset, shift, dtype):
         darb.darb_destroy(h)
 
 
+@pytest.mark.parametrize("cell,I,H,B", [("lstm", 60, 400, 8), ("gru", 90, 500, 3), ("gru", 0, 200, 40)])
+def test_step_of_units_sorted_by_block_size(cell, I, H, B):
+    """The CTAs' unit ranges follow the units' cost (unit_split.h)."""
+    g = np.random.default_rng(81)
+    gates = 4 if cell == "lstm" else 3
+    w = (0.3 * g.standard_normal((gates * H, I + H))).astype(np.float32)
+    m = np.tile(np.r_[np.full(H // 10, 2, np.int32), np.full(H - H // 10, 64, np.int32)], gates)
+    h, ref = encode_both(w, m, "f32")
+    try:
+        x = synth.activations(max(I, 1), B, seed=1)[:I].copy()
+        hp, cp = synth.state(H, B, seed=2), synth.state(H, B, seed=3)
+        ho, co = torch.empty((H, B), device=dev()), torch.empty((H, B), device=dev())
+        xd = t(x) if I else None
+        if cell == "lstm":
+            darb.darb_lstm_step(h, I, H, B, xd, t(hp), t(cp), None, ho, co)
+            hr, cr, ga = oracle.lstm_step(ref, I, H, x if I else None, hp, cp, None)
+            bc, bh = lstm_bounds(ga, cp, TOL["f32"])
+            assert np.all(np.abs(co.cpu().numpy() - cr) <= bc)
+            assert np.all(np.abs(ho.cpu().numpy() - hr) <= bh)
+        else:
+            darb.darb_gru_step(h, I, H, B, xd, t(hp), None, None, ho)
+            hr, ga = oracle.gru_step(ref, I, H, x if I else None, hp, None, None)
+            assert np.all(np.abs(ho.cpu().numpy() - hr) <= gru_bound(ga, hp, hr, TOL["f32"]))
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
 def test_gru_step_infinite_weight_in_a_block_across_the_boundary():
     """Block [4, 8) of a row holds x columns 4, 5 and h columns 6, 7 (I = 6); an
     infinite weight on one side must not meet the other side's zeros."""
