@@ -2,7 +2,8 @@
 
 Each CUDA translation unit compiles in parallel to an object under ``_build/``
 and the objects link into ``paper_1911_08020_gb300/libdarb.so``, which exports
-only the C ABI declared in ``include/darb.h``.  ``libdarb_baselines.so`` holds
+only the C ABI declared in ``include/darb.h`` and, for the tests, the
+``darb_internal_*`` calls of ``csrc/darb_internal.h``.  ``libdarb_baselines.so`` holds
 the cuSPARSE comparison products of ``include/darb_baselines.h``; it is a
 separate library so that libdarb never links the vendor sparse library.
 """

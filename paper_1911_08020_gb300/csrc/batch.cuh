@@ -627,6 +627,7 @@ cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, 
     if constexpr (MODE == kModeY) grid_shape<LPR, CPL>(f, tiles, resident_per_sm<BF16, LPR, CPL, MODE>(), &level, &split);
     else grid_shape_rnn<LPR, CPL>(f, tiles, &level, &split);
     const dim3 grid(static_cast<unsigned>(f.nitems[level][split]), static_cast<unsigned>(tiles));
+    last_kernel() = kKernelBatch;
     return launch_ex(batch_kernel<BF16, LPR, CPL, MODE>, grid, dim3(kThreads), smem, stream, 1u << split, true, f,
                      f.items[level][split], X, ldx, batch, Y, ldy, xmap, hmap, ra, use_tma, early ? 1 : 0);
 }

@@ -513,6 +513,8 @@ bool overlaps(const void *a, size_t abytes, const void *b, size_t bbytes) {
 
 extern "C" {
 
+int darb_internal_last_kernel(void) { return darb::last_kernel(); }
+
 const char *darb_status_string(darb_status_t s) {
     switch (s) {
         case DARB_OK: return "DARB_OK";

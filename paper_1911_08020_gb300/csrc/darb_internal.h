@@ -208,15 +208,27 @@ cudaError_t launch_gru_sequence(const Format &f, const int32_t *row_m, int64_t T
 struct RnnArgs;
 // Batch > 4 RNN steps (rnn_batch.cu); mode is kModeLstm or kModeGru.
 cudaError_t launch_rnn_batch(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream);
+// What it is expected to take, ns.
+double rnn_batch_ns(const Format &f, const RnnArgs &ra, int mode);
 
-// The same with the cell local to the CTA of a unit (rnn_step.cu);
-// cudaErrorNotSupported when the call does not fit it.
-cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream);
+// A step with the cell local to the CTA of a unit (rnn_step.cu), any batch up
+// to 1024; cudaErrorNotSupported when the call does not fit it or is not
+// expected to take less than limit_ns.
+cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, double limit_ns,
+                            cudaStream_t stream);
 
 // The product on the same kernel (rnn_step.cu); cudaErrorNotSupported when it
 // does not fit or is not expected to take less than limit_ns.
 cudaError_t launch_spmm_rows(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,
                              bool early, double limit_ns, cudaStream_t stream);
+
+// Which of these kernels the calling thread launched last, for tests that have
+// to know which one a call reaches.
+enum Kernel : int { kKernelNone, kKernelRowlane, kKernelRows, kKernelBatch, kKernelXres, kKernelXresPlain };
+inline int &last_kernel() {
+    static thread_local int k = kKernelNone;
+    return k;
+}
 
 // Batch-tile width the RNN step kernels use for a batch of B (sizes the counters).
 int rnn_batch_tile(int64_t B);
@@ -245,3 +257,6 @@ darb_status_t lstm_step_view(darb_handle_t h, int64_t I, int64_t H, int64_t B, c
                              const float *h_out, const float *c_out, Format *f);
 
 }  // namespace darb
+
+// Exported beside the C ABI, for the tests: last_kernel().
+extern "C" DARB_API int darb_internal_last_kernel(void);

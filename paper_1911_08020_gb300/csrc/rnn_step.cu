@@ -4,12 +4,13 @@
 
 namespace darb {
 
-cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, cudaStream_t stream) {
+cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool early, double limit_ns,
+                            cudaStream_t stream) {
     if (mode == kModeLstm)
-        return f.bf16 ? step::launch<true, kModeLstm>(f, ra, early, stream)
-                      : step::launch<false, kModeLstm>(f, ra, early, stream);
-    return f.bf16 ? step::launch<true, kModeGru>(f, ra, early, stream)
-                  : step::launch<false, kModeGru>(f, ra, early, stream);
+        return f.bf16 ? step::launch<true, kModeLstm>(f, ra, early, stream, 0, 0, limit_ns)
+                      : step::launch<false, kModeLstm>(f, ra, early, stream, 0, 0, limit_ns);
+    return f.bf16 ? step::launch<true, kModeGru>(f, ra, early, stream, 0, 0, limit_ns)
+                  : step::launch<false, kModeGru>(f, ra, early, stream, 0, 0, limit_ns);
 }
 
 cudaError_t launch_spmm_rows(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,

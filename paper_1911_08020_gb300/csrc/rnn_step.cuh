@@ -460,6 +460,7 @@ cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem,
         if (make(&mx, ra.x, ra.I, p.bxh, ldx) && (MODE == kModeY || make(&mh, ra.h, ra.H, p.bhh, ra.B)))
             p.staging = kStageBoxes;
     }
+    last_kernel() = kKernelRows;
     return launch_ex(kernel, dim3(static_cast<unsigned>(p.ntiles * p.members)), dim3(kThreads), smem, stream, 1, true,
                      f, ra, mx, mh, p);
 }
@@ -468,8 +469,8 @@ cudaError_t launch_tile(const Format &f, const RnnArgs &ra, Plan p, size_t smem,
 // staged tile does not fit beside the CTA's rows even at 4 columns, or no tile
 // width is expected to take less than limit_ns.
 template <bool BF16, int MODE>
-cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream, int64_t ldx = 0,
-                   int64_t ldy = 0, double limit_ns = 1e300) {
+cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream, int64_t ldx, int64_t ldy,
+                   double limit_ns) {
     constexpr int kGates = MODE == kModeLstm ? 4 : MODE == kModeGru ? 3 : 1;
     const int64_t K = MODE == kModeY ? ra.I : int64_t(ra.I) + ra.H;
     if (K > 60000 || ra.B > 1024 || f.nitems[0][0] <= 0) return cudaErrorNotSupported;

@@ -276,6 +276,7 @@ cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, 
     const dim3 grid(static_cast<unsigned>(f.ngroups) * ksc);
     // X rows are the slice's BT-wide rows back to back: one bulk copy per round
     const int x_contig = (MODE == kModeY && batch == BT && ldx == BT && reinterpret_cast<uintptr_t>(X) % 16 == 0) ? 1 : 0;
+    last_kernel() = kKernelRowlane;
     return launch_ex(rowlane_kernel<BF16, BT, MODE>, grid, dim3(kWarps * 32), smem, stream, ksc, true, f, X, ldx, batch,
                      Y, ldy, ra, early ? 1 : 0, x_contig);
 }

@@ -816,6 +816,7 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
                                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorNotSupported;
     }
+    last_kernel() = PLAIN ? kKernelXresPlain : kKernelXres;
     return launch_ex(xres_kernel<BF16, T, PLAIN>, dim3(static_cast<unsigned>(nrun * p.C)), dim3(kThreads), smem, stream,
                      static_cast<unsigned>(p.C), true, f, X, ldx, batch, Y, ldy, xmap, p);
 }

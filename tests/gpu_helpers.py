@@ -23,6 +23,15 @@ TOL = {"f32": 1e-5, "bf16": 2e-3}
 TRANSCENDENTAL_SLACK = 2e-6
 
 
+# csrc/darb_internal.h, enum Kernel
+ROWLANE, ROWS, BATCH, XRES, XRES_PLAIN = 1, 2, 3, 4, 5
+
+
+def last_kernel():
+    """Which of these kernels this thread launched last."""
+    return darb.lib().darb_internal_last_kernel()
+
+
 def dev():
     return torch.device("cuda:0")
 

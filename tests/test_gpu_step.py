@@ -10,7 +10,7 @@ import torch
 import oracle
 from paper_1911_08020_gb300 import darb, synth
 
-from .gpu_helpers import TOL, dev, encode_both, gru_bound, lstm_bounds, t
+from .gpu_helpers import (BATCH, ROWLANE, ROWS, TOL, dev, encode_both, gru_bound, last_kernel, lstm_bounds, t)
 
 pytestmark = pytest.mark.gpu
 
@@ -94,6 +94,47 @@ def test_step_of_units_sorted_by_block_size(cell, I, H, B):
             darb.darb_gru_step(h, I, H, B, xd, t(hp), None, None, ho)
             hr, ga = oracle.gru_step(ref, I, H, x if I else None, hp, None, None)
             assert np.all(np.abs(ho.cpu().numpy() - hr) <= gru_bound(ga, hp, hr, TOL["f32"]))
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
+# (cell, I, H, block sizes, batch, kernel): steps of large matrices whose times on
+# the kernels differ by 20% or more
+RULE = [
+    ("lstm", 256, 1024, (4, 8, 16, 32), 32, ROWS), ("lstm", 7000, 1192, (10, 15, 20, 30), 1, ROWLANE),
+    ("lstm", 4096, 4096, (16, 32, 64), 2, ROWS), ("lstm", 7000, 1192, (10, 15, 20, 30), 4, ROWS), ("lstm", 7000, 1192, (10, 15, 20, 30), 64, BATCH),
+    ("lstm", 4096, 4096, (16, 32, 64), 32, BATCH), ("lstm", 4096, 4096, (16, 32, 64), 13, ROWS),
+    ("gru", 2048, 2048, (8, 16, 32, 64), 32, ROWS), ("gru", 2048, 2048, (8, 16, 32, 64), 64, ROWS),
+]
+
+
+@pytest.mark.parametrize("cell,I,H,mset,B,kernel", RULE)
+def test_large_steps_run_on_the_faster_kernel(cell, I, H, mset, B, kernel):
+    """... and agree with one-column steps, which add in another order: two fp32
+    sums of up to 820 products each within 820 * 2^-24 of sum |w x| (at most some
+    20 here) of the exact one, through a cell that contracts."""
+    gates = 4 if cell == "lstm" else 3
+    gen = torch.Generator(device=dev()).manual_seed(4)
+    w = (0.02 * torch.randn((gates * H, I + H), device=dev(), generator=gen)).to(torch.bfloat16)
+    h = darb.darb_encode(w, np.random.default_rng(82).choice(np.asarray(mset, np.int32), gates * H))
+    del w
+    try:
+        x, hp, cp = (torch.randn((n, B), device=dev(), generator=gen) for n in (I, H, H))
+
+        def step(x, hp, cp):
+            ho, co = torch.empty_like(hp), torch.zeros_like(hp)
+            if cell == "lstm":
+                darb.darb_lstm_step(h, I, H, hp.shape[1], x, hp, cp, None, ho, co)
+            else:
+                darb.darb_gru_step(h, I, H, hp.shape[1], x, hp, None, None, ho)
+            return ho, co
+
+        ho, co = step(x, hp, cp)
+        assert last_kernel() == kernel
+        for j in {0, B - 1}:
+            for whole, one in zip((ho, co), step(*(v[:, j:j + 1].contiguous() for v in (x, hp, cp)))):
+                assert torch.max(torch.abs(whole[:, j:j + 1] - one)).item() < 2e-3
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
