@@ -961,8 +961,8 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     a.x_tiles = a.x_mode != kXBulk ? nullptr : x_in_place ? a.x : xws;
     const int64_t warps = H + (pre || x_copy ? T * I : 0);
     const unsigned grid = static_cast<unsigned>(std::min<int64_t>((warps + 7) / 8, int64_t(sm_count()) * 16));
-    prep_kernel<<<grid, 256, 0, stream>>>(a, s.lbt, h0, x_copy ? xws : nullptr, pre ? xws : nullptr, ldx, nwords);
-    e = cudaGetLastError();
+    e = launch_ex(prep_kernel, dim3(grid), dim3(256), 0, stream, 1, false, a, s.lbt, h0, x_copy ? xws : nullptr,
+                  pre ? xws : nullptr, ldx, nwords);
     if (pre) {
         float *gx = reinterpret_cast<float *>(reinterpret_cast<char *>(xws) + up(size_t(I + H) * ldx * 4));
         if (e == cudaSuccess) {

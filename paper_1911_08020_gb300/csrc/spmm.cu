@@ -12,6 +12,7 @@
 #include "launch.cuh"
 #include "rowlane.cuh"
 
+#include <cstdlib>
 #include <mutex>
 #include <set>
 
@@ -51,7 +52,13 @@ cudaError_t stream_alloc(void **p, size_t bytes, cudaStream_t stream) {
     } else {
         cudaGetLastError();
     }
-    return cudaMallocAsync(p, bytes, stream);
+    // Test hook: with DARB_TEST_POOL_LIMIT=n a request of more than n bytes becomes
+    // one that no device can meet, so that the runtime refuses it
+    if (const char *limit = std::getenv("DARB_TEST_POOL_LIMIT"))
+        if (bytes > std::strtoull(limit, nullptr, 10)) bytes = size_t(1) << 60;
+    const cudaError_t e = cudaMallocAsync(p, bytes, stream);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by a later launch's check
+    return e;
 }
 
 int sm_count() {

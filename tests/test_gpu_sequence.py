@@ -360,3 +360,24 @@ def test_barrier_timeout_of_a_wide_tile(monkeypatch):
     """The same where h is exchanged behind the barrier (tiles of more than 32 KB)
     instead of with tags."""
     test_barrier_timeout_is_reported_and_the_device_stays_usable("lstm", 20, 1100, 8, monkeypatch)
+
+
+def test_call_after_a_refused_allocation(monkeypatch):
+    """A call whose workspace the pool refuses says so, and the refusal is not
+    found again by the next call's check of its own launch."""
+    g = np.random.default_rng(48)
+    T, I, H, B = 3, 7, 33, 3
+    stored, m = _gate_matrix(g, 4, I, H, "f32", (2, 4, 8))
+    h, ref = encode_both(stored, m, "f32")
+    try:
+        xs = synth.activations(T * I, B, seed=5).reshape(T, I, B)
+        h0, c0 = synth.state(H, B, seed=6), synth.state(H, B, seed=7)
+        monkeypatch.setenv("DARB_TEST_POOL_LIMIT", "1")
+        with pytest.raises(darb.DarbError) as e:
+            darb.darb_lstm_sequence(h, T, I, H, B, t(xs), t(h0), t(c0), None, torch.empty((T, H, B), device=dev()))
+        assert e.value.status == darb.ERR_OOM
+        monkeypatch.delenv("DARB_TEST_POOL_LIMIT")
+        _check_lstm_sequence(h, ref, T, I, H, B, xs, h0, c0, None, TOL["f32"])
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
