@@ -70,7 +70,7 @@ struct Ranges {
 // Where x_t comes from.
 constexpr int kXNone = 0;    // its products are precomputed (gx)
 constexpr int kXBulk = 1;    // tile-major rows (x_tiles), bulk copies
-constexpr int kXPlain = 2;   // the caller's x, plain loads (its tile-major copy would be too large)
+constexpr int kXPlain = 2;   // the caller's x, plain loads (there is no room for its tile-major copy)
 
 struct SeqArgs {
     int I, H, T;
@@ -937,7 +937,8 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     a.skip_cta = -1;
     sequence_test_hook(&a.barrier_ns, &a.skip_cta);
     // x_t is read in place when its rows are already tile-major; else from a
-    // tile-major copy, or by plain loads where that copy would be too large
+    // tile-major copy, or by plain loads where that copy would be too large (or
+    // cannot be had, below)
     const bool x_in_place = I % 4 == 0 && B == bt && reinterpret_cast<uintptr_t>(a.x) % 16 == 0;
     const size_t xt_bytes = size_t(T) * size_t(a.ntiles) * size_t(a.irows) * bt * 4;
     a.x_mode = pre || I == 0 ? kXNone : x_in_place || xt_bytes <= (size_t(1) << 30) ? kXBulk : kXPlain;
@@ -948,10 +949,15 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     const size_t bar_bytes = up(size_t(nwords) * 4);
     const size_t cbytes = kGru || a.c_on_chip || c_last ? 0 : up(size_t(H) * size_t(B) * 4);
     const size_t hx_bytes = up(2 * size_t(a.ntiles) * size_t(a.hrows) * bt * (a.tagged ? 8 : 4));
-    const bool x_copy = a.x_mode == kXBulk && !x_in_place;
-    const size_t ws_bytes = bar_bytes + cbytes + hx_bytes + (pre ? pre_bytes : 0) + (x_copy ? up(xt_bytes) : 0);
+    bool x_copy = a.x_mode == kXBulk && !x_in_place;
+    const size_t base_bytes = bar_bytes + cbytes + hx_bytes + (pre ? pre_bytes : 0);
     char *ws = nullptr;
-    cudaError_t e = stream_alloc(reinterpret_cast<void **>(&ws), ws_bytes, stream);
+    cudaError_t e = stream_alloc(reinterpret_cast<void **>(&ws), base_bytes + (x_copy ? up(xt_bytes) : 0), stream);
+    if (e == cudaErrorMemoryAllocation && x_copy) {   // no room for the copy of x: the steps read it in place
+        x_copy = false;
+        a.x_mode = kXPlain;
+        e = stream_alloc(reinterpret_cast<void **>(&ws), base_bytes, stream);
+    }
     if (e != cudaSuccess) return e;
     a.bar = reinterpret_cast<unsigned *>(ws);
     a.abort_flag = reinterpret_cast<int *>(ws + size_t(a.ngroups) * kBarWords * 4);

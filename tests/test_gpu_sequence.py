@@ -381,3 +381,35 @@ def test_call_after_a_refused_allocation(monkeypatch):
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
+
+
+@pytest.mark.parametrize("cell,I,H,B", [("lstm", 20, 50, 9), ("gru", 30, 90, 3)])
+def test_no_room_for_the_copy_of_x(cell, I, H, B, monkeypatch):
+    """Where the pool has the rest of the workspace (4 to 16 KB here) but not the
+    tile-major copy of x (60 steps, 23 KB and more), the steps read x in place;
+    a call that needs more than the pool has still says so."""
+    g = np.random.default_rng(49)
+    gates = 4 if cell == "lstm" else 3
+    T = 60
+    stored, m = _gate_matrix(g, gates, I, H, "f32", (2, 4, 8))
+    h, ref = encode_both(stored, m, "f32")
+    try:
+        xs = synth.activations(T * I, B, seed=5).reshape(T, I, B)
+        h0, c0 = synth.state(H, B, seed=6), synth.state(H, B, seed=7)
+        b1, b2 = synth.bias(gates * H, seed=1), synth.bias(gates * H, seed=2)
+
+        def check():
+            if cell == "lstm":
+                return _check_lstm_sequence(h, ref, T, I, H, B, xs, h0, c0, b1, TOL["f32"])[0]
+            return _check_gru_sequence(h, ref, T, I, H, B, xs, h0, b1, b2, TOL["f32"])
+
+        copied = check()
+        monkeypatch.setenv("DARB_TEST_POOL_LIMIT", "20000")
+        np.testing.assert_array_equal(check(), copied)   # the same sums in the same order
+        monkeypatch.setenv("DARB_TEST_POOL_LIMIT", "256")
+        with pytest.raises(darb.DarbError) as e:
+            check()
+        assert e.value.status == darb.ERR_OOM
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
