@@ -413,3 +413,31 @@ def test_no_room_for_the_copy_of_x(cell, I, H, B, monkeypatch):
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
+
+
+def test_planning_does_not_divide_per_row_and_candidate():
+    """Host time of a one-step call on a large cell over one on a small cell (the
+    least of many): 8 us when planning looks a row's counts up by its block
+    size, 130 us when it works them out for every row and every tile width and
+    group count it tries."""
+    import time
+
+    def host_us(I, H, B):
+        h = darb.darb_encode(torch.randn((4 * H, I + H), device=dev()),
+                             np.random.default_rng(50).choice(np.array([10, 15, 20, 30], np.int32), 4 * H))
+        try:
+            x, z = torch.zeros((1, I, B), device=dev()), torch.zeros((H, B), device=dev())
+            hs, cl = torch.empty((1, H, B), device=dev()), torch.empty((H, B), device=dev())
+            least = 1e9
+            for _ in range(60):
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                darb.darb_lstm_sequence(h, 1, I, H, B, x, z, z, None, hs, None, cl)
+                least = min(least, 1e6 * (time.perf_counter() - t0))
+            darb.darb_sync_status(h)
+            return least
+        finally:
+            darb.darb_destroy(h)
+
+    small = host_us(64, 128, 2)
+    assert host_us(1500, 1500, 20) - small < 60
