@@ -25,8 +25,8 @@
  *  - Work is enqueued on the caller's stream.  Only darb_encode, darb_import,
  *    darb_export, darb_sync_status, darb_rnn_reserve and darb_destroy
  *    synchronise; the product, step and sequence calls are asynchronous.
- *    darb_spmm allocates nothing; the step calls use scratch owned by the
- *    handle (darb_rnn_reserve sizes it up front).
+ *    darb_spmm allocates nothing; the step calls on large matrices or batches
+ *    use scratch owned by the handle (darb_rnn_reserve sizes it up front).
  *  - Only two opt-in calls take scratch from the device's stream-ordered
  *    memory pool: darb_spmm_ex with DARB_PATH_TENSOR_CORES and the sequence
  *    calls.  They return it to the pool on the same stream.  The first such
@@ -243,10 +243,15 @@ DARB_API darb_status_t darb_spmm_path(darb_handle_t h, int64_t batch, darb_path_
  *   h_prev, c_prev   device fp32, H x B
  *   bias   device fp32 [4H] added to the gate pre-activations, or NULL
  *   h_out, c_out     device fp32, H x B; must not overlap any input
- * Uses scratch owned by the handle (4H x B floats of gate sums and H counters),
- * allocated by the first step call that needs more than the handle holds (that
- * call synchronises); call darb_rnn_reserve first to size it up front.  Step
- * calls on one handle must be ordered on one stream.
+ * Most steps keep their gate sums on chip and need no scratch.  A step whose
+ * stacked input is too tall for that (from some 14000 rows), whose batch is
+ * above 1024, or that is faster on the kernels that exchange gate sums through
+ * memory (large matrices; decided by the sizes, the dtype and the alignment)
+ * uses scratch owned by the handle (4H x B floats of gate sums and at most
+ * H x ceil(B / t) counters, t = 1, 2, 4 or 8 by batch), allocated by the first such call that
+ * needs more than the handle holds (that call synchronises); call
+ * darb_rnn_reserve first to size it up front.  Step calls on one handle must
+ * be ordered on one stream.
  * Errors: DARB_ERR_INVALID_ARG (null, shape mismatch, B <= 0); DARB_ERR_OOM;
  * DARB_ERR_CUDA.
  */
@@ -326,21 +331,21 @@ DARB_API darb_status_t darb_gru_sequence(darb_handle_t h, int64_t T, int64_t I, 
 
 /*
  * darb_lstm_step without any allocation: the same step, same arguments and
- * same results, with its scratch (gate sums and arrival counters) in one
- * fixed array of 4 MiB inside this library instead of memory owned by the
- * handle.  It is for callers that cannot let a library call cudaMalloc at step
+ * same results, with the scratch of the steps that need some (gate sums and
+ * arrival counters) in one fixed array of 4 MiB inside this library instead of
+ * memory owned by the handle.  It is for callers that cannot let a library call cudaMalloc at step
  * time -- a serving loop with a fixed memory budget, code that must not
  * synchronise the device mid-stream, or allocations that must all go through
  * the caller's own pool.  The paper has no counterpart; it is a property of
  * this library's interface only.
  *   - Limit: 4H*B floats (rounded up to 256 bytes) plus H*ceil(B/t) counters
- *     (t = 1, 2, 4 or 8 by batch) must fit in 4 MiB; larger calls return
- *     DARB_ERR_UNSUPPORTED and do nothing.
+ *     (t = 1, 2, 4 or 8 by batch) must fit in 4 MiB, whether or not the step
+ *     uses them; larger calls return DARB_ERR_UNSUPPORTED and do nothing.
  *   - Every GPU that loads the library holds the 4 MiB until the process exits.
  *   - The first call on each device looks up the array's device address (one
  *     cudaGetSymbolAddress); make that first call before any stream capture.
  *   - All calls on a device share the one array, which keeps the last call's
- *     contents; each call clears the counters it needs on `stream`.  Calls that
+ *     contents; a call that uses it clears its counters on `stream`.  Calls that
  *     overlap on the GPU (other streams, or unordered launches) race on it.
  * Errors as darb_lstm_step, plus DARB_ERR_UNSUPPORTED for the size limit.
  */

@@ -498,6 +498,22 @@ size_t gate_floats_for(const darb_handle_s *h, int64_t B, bool gru) {
     return static_cast<size_t>(h->rows) * static_cast<size_t>(B) * (gru ? 2 : 1);
 }
 
+// A step: launch(scratch) with the scratch that the handle has, or with none;
+// the kernel that most steps take uses none.  Grown to what the call needs only
+// when launch says that it needs some.
+template <class Launch>
+darb_status_t run_step(darb_handle_s *h, size_t gate_floats, size_t counter_ints, Launch launch) {
+    darb::RnnScratch sc{};
+    if (gate_floats <= h->gates_cap && counter_ints <= h->counters_cap) sc = {h->d_gates, h->d_counters};
+    cudaError_t e = launch(sc);
+    if (e == cudaErrorNotSupported && sc.gates == nullptr) {
+        const darb_status_t st = ensure_scratch(h, gate_floats, counter_ints);
+        if (st != DARB_OK) return st;
+        e = launch(darb::RnnScratch{h->d_gates, h->d_counters});
+    }
+    return cuda_status(e);
+}
+
 size_t counter_ints_for(int64_t H, int64_t B) {
     const int bt = darb::rnn_batch_tile(B);
     return static_cast<size_t>(H) * static_cast<size_t>(ceil_div(B, bt));
@@ -814,11 +830,10 @@ darb_status_t darb_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, c
         if (overlaps(h_out, hb, ins[i], inb[i]) || overlaps(c_out, hb, ins[i], inb[i]))
             return DARB_ERR_INVALID_ARG;
     if (overlaps(h_out, hb, c_out, hb)) return DARB_ERR_INVALID_ARG;
-    st = ensure_scratch(h, gate_floats_for(h, B, false), counter_ints_for(H, B));
-    if (st != DARB_OK) return st;
-    darb::RnnScratch sc{h->d_gates, h->d_counters};
-    return cuda_status(darb::launch_lstm_step(format_of(h), I, H, B, x, h_prev, c_prev, bias,
-                                              h_out, c_out, sc, stream, early_ok(h, stream)));
+    const bool early = early_ok(h, stream);
+    return run_step(h, gate_floats_for(h, B, false), counter_ints_for(H, B), [&](darb::RnnScratch sc) {
+        return darb::launch_lstm_step(format_of(h), I, H, B, x, h_prev, c_prev, bias, h_out, c_out, sc, stream, early);
+    });
 }
 
 darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
@@ -834,11 +849,10 @@ darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, co
                            static_cast<size_t>(3 * H) * 4};
     for (int i = 0; i < 4; ++i)
         if (overlaps(h_out, hb, ins[i], inb[i])) return DARB_ERR_INVALID_ARG;
-    st = ensure_scratch(h, gate_floats_for(h, B, true), counter_ints_for(H, B));
-    if (st != DARB_OK) return st;
-    darb::RnnScratch sc{h->d_gates, h->d_counters};
-    return cuda_status(darb::launch_gru_step(format_of(h), I, H, B, x, h_prev, b_ih, b_hh, h_out,
-                                             sc, stream, early_ok(h, stream)));
+    const bool early = early_ok(h, stream);
+    return run_step(h, gate_floats_for(h, B, true), counter_ints_for(H, B), [&](darb::RnnScratch sc) {
+        return darb::launch_gru_step(format_of(h), I, H, B, x, h_prev, b_ih, b_hh, h_out, sc, stream, early);
+    });
 }
 
 // Arrival counts of the sequence kernels' barrier stay below 2^32.

@@ -153,7 +153,8 @@ struct EncodeTarget {
     int64_t rows, cols;
 };
 
-// Scratch for the fused RNN steps: gate sums and per-(unit, batch tile) arrival counters.
+// Scratch of the RNN steps on rowlane_kernel and batch_kernel: gate sums and
+// per-(unit, batch tile) arrival counters.
 struct RnnScratch {
     float *gates;      // rows x B (LSTM) or 2 x rows x B (GRU: x part then h part)
     int32_t *counters; // units x batch tiles, zero between launches
@@ -185,7 +186,8 @@ cudaError_t launch_spmm(const Format &f, const float *X, int64_t ldx, int64_t ba
                         int64_t ldy, bool early, int path, cudaStream_t stream);
 
 // `early` as for launch_spmm (the handle's values may be read before the
-// previous kernel on the stream finishes).
+// previous kernel on the stream finishes).  With null scratch a step that needs
+// some launches nothing and returns cudaErrorNotSupported.
 cudaError_t launch_lstm_step(const Format &f, int64_t I, int64_t H, int64_t B, const float *x,
                              const float *h_prev, const float *c_prev, const float *bias,
                              float *h_out, float *c_out, RnnScratch s, cudaStream_t stream,

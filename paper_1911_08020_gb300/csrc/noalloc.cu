@@ -1,13 +1,14 @@
 // noalloc.cu -- an LSTM step that allocates no device memory.
 //
-// darb_lstm_step keeps its gate sums and per-unit arrival counters in scratch
-// that the handle owns and allocates with cudaMalloc the first time a step
-// needs more than it holds.  Some callers cannot let a library allocate at
+// Large steps of darb_lstm_step keep their gate sums and per-unit arrival
+// counters in scratch that the handle owns and allocates with cudaMalloc the
+// first time one needs more than it holds (smaller steps take a kernel that
+// needs none, rnn_step.cuh).  Some callers cannot let a library allocate at
 // that point: a serving loop running under a fixed memory budget, where any
 // cudaMalloc outside start-up can fail or stall every stream on the device;
 // code that must not synchronise the device mid-stream (cudaMalloc and
 // cudaFree can); and callers whose allocations all go through their own pool.
-// darb_lstm_step_noalloc runs the same kernel with that scratch in one fixed
+// darb_lstm_step_noalloc runs the same kernels, with that scratch in one fixed
 // array compiled into this library instead, so nothing is allocated at call
 // time (or ever, apart from the array itself, which every GPU that loads the
 // library holds until the process exits).
@@ -72,12 +73,15 @@ extern "C" darb_status_t darb_lstm_step_noalloc(darb_handle_t h, int64_t I, int6
     darb::RnnScratch sc;
     sc.gates = static_cast<float *>(base);
     sc.counters = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(base) + gate_span);
-    // the array keeps whatever the last call left: counters must start at zero
-    if (cudaMemsetAsync(sc.counters, 0, counter_bytes, stream) != cudaSuccess) {
-        cudaGetLastError();
-        return DARB_ERR_CUDA;
+    // most steps take the kernel that needs no scratch
+    cudaError_t e = darb::launch_lstm_step(f, I, H, B, x, h_prev, c_prev, bias, h_out, c_out, darb::RnnScratch{}, stream);
+    if (e == cudaErrorNotSupported) {
+        // the array keeps whatever the last call left: counters must start at zero
+        if (cudaMemsetAsync(sc.counters, 0, counter_bytes, stream) != cudaSuccess) {
+            cudaGetLastError();
+            return DARB_ERR_CUDA;
+        }
+        e = darb::launch_lstm_step(f, I, H, B, x, h_prev, c_prev, bias, h_out, c_out, sc, stream);
     }
-    return darb::launch_lstm_step(f, I, H, B, x, h_prev, c_prev, bias, h_out, c_out, sc, stream) == cudaSuccess
-               ? DARB_OK
-               : DARB_ERR_CUDA;
+    return e == cudaSuccess ? DARB_OK : DARB_ERR_CUDA;
 }

@@ -44,7 +44,7 @@ template <int MODE>
 static cudaError_t launch_step(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream) {
     const double others_ns = ra.B <= 4 ? rowlane_ns(f, ra.B) : rnn_batch_ns(f, ra, MODE);
     const cudaError_t e = launch_rnn_step(f, ra, MODE, early, others_ns, stream);
-    if (e != cudaErrorNotSupported) return e;
+    if (e != cudaErrorNotSupported || ra.counters == nullptr) return e;
     if (ra.B <= 4)
         return f.bf16 ? rowlane::launch_any<true, MODE>(f, nullptr, 0, ra.B, nullptr, 0, ra, early, stream)
                       : rowlane::launch_any<false, MODE>(f, nullptr, 0, ra.B, nullptr, 0, ra, early, stream);
@@ -65,7 +65,7 @@ cudaError_t launch_gru_step(const Format &f, int64_t I, int64_t H, int64_t B, co
                             const float *h_prev, const float *b_ih, const float *b_hh,
                             float *h_out, RnnScratch s, cudaStream_t stream, bool early) {
     RnnArgs ra{};
-    ra.x = x; ra.h = h_prev; ra.gx = s.gates; ra.gh = s.gates + f.rows * B; ra.counters = s.counters;
+    ra.x = x; ra.h = h_prev; ra.gx = s.gates; ra.gh = s.gates ? s.gates + f.rows * B : nullptr; ra.counters = s.counters;
     ra.b_ih = b_ih; ra.b_hh = b_hh; ra.h_out = h_out;
     ra.I = static_cast<int>(I); ra.H = static_cast<int>(H); ra.B = B;
     return launch_step<kModeGru>(f, ra, early, stream);

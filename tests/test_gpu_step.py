@@ -140,6 +140,41 @@ def test_large_steps_run_on_the_faster_kernel(cell, I, H, mset, B, kernel):
         darb.darb_destroy(h)
 
 
+def test_step_takes_scratch_only_for_the_kernels_that_use_it():
+    """The local-cell kernel needs no gate sums or counters: a handle that only
+    runs such steps holds no memory for them (and none is allocated in a capture
+    of a first step); a step on the other kernels adds it."""
+    g = np.random.default_rng(83)
+    I, H, B = 40, 64, 8
+    w = (0.3 * g.standard_normal((4 * H, I + H))).astype(np.float32)
+    h, ref = encode_both(w, np.full(4 * H, 8, np.int32), "f32")
+    try:
+        x, hp, cp = synth.activations(I, B, seed=1), synth.state(H, B, seed=2), synth.state(H, B, seed=3)
+        xd, hd, cd = t(x), t(hp), t(cp)
+        ho, co = torch.empty((H, B), device=dev()), torch.empty((H, B), device=dev())
+        held = darb.darb_info(h)["device_bytes"]
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            darb.darb_lstm_step(h, I, H, B, xd, hd, cd, None, ho, co)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert last_kernel() == ROWS
+        assert darb.darb_info(h)["device_bytes"] == held
+        hr, cr, ga = oracle.lstm_step(ref, I, H, x, hp, cp, None)
+        bc, bh = lstm_bounds(ga, cp, TOL["f32"])
+        assert np.all(np.abs(co.cpu().numpy() - cr) <= bc)
+        assert np.all(np.abs(ho.cpu().numpy() - hr) <= bh)
+        wide = [torch.randn((n, 1028), device=dev()) for n in (I, H, H)]
+        out = [torch.empty((H, 1028), device=dev()) for _ in range(2)]
+        darb.darb_lstm_step(h, I, H, 1028, *wide, None, *out)
+        assert last_kernel() == BATCH
+        assert darb.darb_info(h)["device_bytes"] > held
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
 def test_gru_step_infinite_weight_in_a_block_across_the_boundary():
     """Block [4, 8) of a row holds x columns 4, 5 and h columns 6, 7 (I = 6); an
     infinite weight on one side must not meet the other side's zeros."""
