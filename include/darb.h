@@ -157,7 +157,7 @@ DARB_API darb_status_t darb_reencode_host(darb_handle_t h, const void *W, int64_
 
 /* Synchronise `stream` and report what the handle's kernels recorded on the
  * device since the last call, then clear it: DARB_ERR_TIMEOUT if a bounded
- * device wait (for a bulk copy, or at a sequence call's grid barrier) gave up
+ * device wait (for a bulk copy, or of a sequence call for another CTA) gave up
  * -- results of that call are not valid, the device stays usable -- else
  * DARB_ERR_NONFINITE if a (re)encode met a NaN, else DARB_OK.                */
 DARB_API darb_status_t darb_sync_status(darb_handle_t h, cudaStream_t stream);
@@ -279,10 +279,12 @@ DARB_API darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int6
 /*
  * T consecutive LSTM steps (the cell of darb_lstm_step) in one persistent
  * launch: the recurrence of an RNN layer over a whole input sequence (the
- * LSTM models of Sec. 4.1 run one step per token).  Each CTA keeps its share
- * of the gate matrix decoded in shared memory for all T steps and the steps
- * are separated by a grid-wide barrier, so W is read from memory once per
- * call instead of once per step.
+ * LSTM models of Sec. 4.1 run one step per token).  The batch columns are cut
+ * into groups, each run by its own CTAs; a CTA keeps its share of the gate
+ * matrix decoded in shared memory for all T steps, so W is read from memory
+ * once per call instead of once per step.  The steps of a group are separated
+ * by a barrier over its CTAs, or, where a column tile of h is at most 32 KB, by
+ * the values of h themselves, which carry the number of their step.
  *   x_seq  device fp32, T x I x B (step t at x_seq + t*I*B); NULL allowed when I == 0
  *   h0, c0 device fp32, H x B: the state before the first step
  *   bias   device fp32 [4H] or NULL
@@ -298,14 +300,25 @@ DARB_API darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int6
  * W [x_0 .. x_{T-1}; 0] of T * B columns (darb_spmm's kernels and numerics,
  * the CUDA-core gather); the recurrence then stages and
  * multiplies only h_{t-1}.
- * Resources: one cooperative launch of one CTA per SM (at most H CTAs); a
- * stream-ordered workspace of 256 bytes, plus H x B floats when c_last is
- * NULL and the cell state does not fit on chip, plus (I + H + 4H) x T*B
- * floats when the x parts are precomputed.  A barrier wait longer than 1 s
- * ends the launch and is reported by darb_sync_status as DARB_ERR_TIMEOUT.
- * For testing that path, the environment variable DARB_TEST_BARRIER_TIMEOUT=1
- * (read at every launch) shortens the limit to 1 ms and makes CTA 0 withhold
- * its first arrival, so the launch times out on purpose.
+ * Resources: a preparing launch and one cooperative launch of at most one CTA
+ * per SM, and a stream-ordered workspace of
+ *   - 128 bytes for every column group (at most one a CTA), and 128 more;
+ *   - H x B floats when c_last is NULL and the cell state does not fit on chip;
+ *   - two buffers of h, H rounded up to 4 rows x B rounded up to whole column
+ *     tiles (of 1 to 32 columns): 4 bytes an element, 8 where a tile of h is at
+ *     most 32 KB;
+ *   - when the x parts are precomputed, (I + H + 4H) x T*B floats (T*B rounded
+ *     up to 4); else, unless I is 0 or x_seq is laid out so already (I a multiple
+ *     of 4, B one whole tile, a 16-byte aligned base), a copy of x_seq with I
+ *     rounded up to 4 rows and B to whole tiles, if that is at most 1 GiB and
+ *     the memory pool can supply it; x_seq is read in place if not.
+ * DARB_ERR_OOM if the pool cannot supply the rest.  A wait of more than 1 s for
+ * another CTA ends the launch and is reported by darb_sync_status as
+ * DARB_ERR_TIMEOUT.  For testing that path, the environment variable
+ * DARB_TEST_BARRIER_TIMEOUT=1 (read at every launch) shortens the limit to 1 ms
+ * and makes CTA 0 withhold its first arrival or its first values of h, so the
+ * launch times out on purpose; DARB_TEST_POOL_LIMIT=n makes the pool refuse
+ * workspaces of more than n bytes.
  * Errors: DARB_ERR_INVALID_ARG (shape mismatch, null, overlap, T < 0);
  * DARB_ERR_UNSUPPORTED when a CTA's share of the decoded matrix plus one
  * column tile of [x_t; h_{t-1}] does not fit in shared memory, or cols > 65535;

@@ -105,8 +105,8 @@ struct SeqArgs {
     unsigned *bar;          // arrival counters of the groups, kBarWords apart, zero at launch
     int *abort_flag;        // zero at launch
     int32_t *status;
-    unsigned long long barrier_ns;   // time limit of a barrier wait (kWaitLimitNs unless a test shortens it)
-    int skip_cta;           // test hook: this CTA does not arrive at the first barrier (-1: none)
+    unsigned long long barrier_ns;   // time limit of a wait for another CTA (kWaitLimitNs unless a test shortens it)
+    int skip_cta;           // test hook: this CTA does not arrive, or publish, after the first step (-1: none)
 };
 
 // Byte offsets of the regions of a CTA's dynamic shared memory.
@@ -743,13 +743,15 @@ __global__ void __launch_bounds__(256) prep_kernel(SeqArgs a, int lbt, const flo
 
 namespace {
 
-// Test hook for the failure path of the grid barrier.  With the environment
-// variable DARB_TEST_BARRIER_TIMEOUT=1 a launch's barrier waits give up after
-// 1 ms and CTA 0 withholds its arrival at the first barrier: every CTA's wait
-// runs out, the launch records DARB_ERR_TIMEOUT (read by darb_sync_status),
-// raises the abort flag and ends.  Only the barrier is affected -- no copy is
-// in flight while a CTA waits there -- and the results of that call are not
-// valid.  Read on every launch so that a test can set and clear it.
+// Test hook for the failure path of the waits between CTAs.  With the
+// environment variable DARB_TEST_BARRIER_TIMEOUT=1 a launch's waits for another
+// CTA give up after 1 ms, and CTA 0 withholds its arrival at the first barrier
+// (or, where h is exchanged with tags, its first values): the waits of its
+// column group run out, the launch records DARB_ERR_TIMEOUT (read by
+// darb_sync_status), raises the abort flag, which ends every wait, and
+// ends; a CTA whose copy of x is in flight waits for it first.  The results of
+// that call are not valid.  Read on every launch so that a test can set and
+// clear it.
 void sequence_test_hook(unsigned long long *barrier_ns, int *skip_cta) {
     const char *v = std::getenv("DARB_TEST_BARRIER_TIMEOUT");
     if (v != nullptr && v[0] == '1' && v[1] == '\0') {
