@@ -511,7 +511,7 @@ darb_status_t run_step(darb_handle_s *h, size_t gate_floats, size_t counter_ints
         if (st != DARB_OK) return st;
         e = launch(darb::RnnScratch{h->d_gates, h->d_counters});
     }
-    return cuda_status(e);
+    return e == cudaErrorNotSupported ? DARB_ERR_UNSUPPORTED : cuda_status(e);   // a given kernel cannot take it
 }
 
 size_t counter_ints_for(int64_t H, int64_t B) {
@@ -530,6 +530,11 @@ bool overlaps(const void *a, size_t abytes, const void *b, size_t bbytes) {
 extern "C" {
 
 int darb_internal_last_kernel(void) { return darb::last_kernel(); }
+
+void darb_internal_last_sequence(int32_t cut[6]) {
+    static_assert(sizeof(darb::SequenceCut) == 6 * sizeof(int32_t), "six words");
+    std::memcpy(cut, &darb::last_sequence(), sizeof(darb::SequenceCut));
+}
 
 const char *darb_status_string(darb_status_t s) {
     switch (s) {
@@ -677,11 +682,8 @@ darb_status_t darb_spmm(darb_handle_t h, const float *X, int64_t ldx, int64_t ba
     return darb_spmm_ex(h, X, ldx, batch, Y, ldy, DARB_PATH_AUTO, stream);
 }
 
-darb_status_t darb_spmm_ex(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y,
-                           int64_t ldy, darb_path_t path, cudaStream_t stream) {
-    DARB_TRACE("darb_spmm_ex");
-    if (path != DARB_PATH_AUTO && path != DARB_PATH_CUDA_CORES && path != DARB_PATH_TENSOR_CORES)
-        return DARB_ERR_INVALID_ARG;
+static darb_status_t check_spmm(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, const float *Y,
+                                int64_t ldy) {
     if (!live(h) || X == nullptr || Y == nullptr || batch <= 0 || ldx < batch || ldy < batch)
         return DARB_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(X) % 4 != 0 || reinterpret_cast<uintptr_t>(Y) % 4 != 0)
@@ -690,7 +692,10 @@ darb_status_t darb_spmm_ex(darb_handle_t h, const float *X, int64_t ldx, int64_t
     if (overlaps(X, static_cast<size_t>((h->cols - 1) * ldx + batch) * 4, Y,
                  static_cast<size_t>((h->rows - 1) * ldy + batch) * 4))
         return DARB_ERR_INVALID_ARG;
-    const cudaError_t e = darb::launch_spmm(format_of(h), X, ldx, batch, Y, ldy, early_ok(h, stream), path, stream);
+    return DARB_OK;
+}
+
+static darb_status_t launch_status(cudaError_t e) {
     if (e == cudaErrorNotSupported) {
         cudaGetLastError();
         return DARB_ERR_UNSUPPORTED;
@@ -700,6 +705,24 @@ darb_status_t darb_spmm_ex(darb_handle_t h, const float *X, int64_t ldx, int64_t
         return DARB_ERR_OOM;
     }
     return cuda_status(e);
+}
+
+darb_status_t darb_spmm_ex(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y,
+                           int64_t ldy, darb_path_t path, cudaStream_t stream) {
+    DARB_TRACE("darb_spmm_ex");
+    if (path != DARB_PATH_AUTO && path != DARB_PATH_CUDA_CORES && path != DARB_PATH_TENSOR_CORES)
+        return DARB_ERR_INVALID_ARG;
+    const darb_status_t st = check_spmm(h, X, ldx, batch, Y, ldy);
+    if (st != DARB_OK) return st;
+    return launch_status(darb::launch_spmm(format_of(h), X, ldx, batch, Y, ldy, early_ok(h, stream), path, stream));
+}
+
+darb_status_t darb_internal_spmm(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,
+                                 int kernel, cudaStream_t stream) {
+    const darb_status_t st = check_spmm(h, X, ldx, batch, Y, ldy);
+    if (st != DARB_OK) return st;
+    return launch_status(darb::launch_spmm_on(format_of(h), static_cast<darb::Kernel>(kernel), X, ldx, batch, Y, ldy,
+                                              early_ok(h, stream), stream));
 }
 
 darb_status_t darb_spmm_host(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,
@@ -816,10 +839,9 @@ static darb_status_t check_step(darb_handle_t h, int64_t I, int64_t H, int64_t B
     return DARB_OK;
 }
 
-darb_status_t darb_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
-                             const float *h_prev, const float *c_prev, const float *bias,
-                             float *h_out, float *c_out, cudaStream_t stream) {
-    DARB_TRACE("darb_lstm_step");
+static darb_status_t lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x, const float *h_prev,
+                               const float *c_prev, const float *bias, float *h_out, float *c_out, darb::Kernel kernel,
+                               cudaStream_t stream) {
     darb_status_t st = check_step(h, I, H, B, 4, x, h_prev);
     if (st != DARB_OK) return st;
     if (c_prev == nullptr || h_out == nullptr || c_out == nullptr) return DARB_ERR_INVALID_ARG;
@@ -832,14 +854,27 @@ darb_status_t darb_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, c
     if (overlaps(h_out, hb, c_out, hb)) return DARB_ERR_INVALID_ARG;
     const bool early = early_ok(h, stream);
     return run_step(h, gate_floats_for(h, B, false), counter_ints_for(H, B), [&](darb::RnnScratch sc) {
-        return darb::launch_lstm_step(format_of(h), I, H, B, x, h_prev, c_prev, bias, h_out, c_out, sc, stream, early);
+        return darb::launch_lstm_step(format_of(h), I, H, B, x, h_prev, c_prev, bias, h_out, c_out, sc, stream, early,
+                                      kernel);
     });
 }
 
-darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
-                            const float *h_prev, const float *b_ih, const float *b_hh,
-                            float *h_out, cudaStream_t stream) {
-    DARB_TRACE("darb_gru_step");
+darb_status_t darb_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                             const float *h_prev, const float *c_prev, const float *bias,
+                             float *h_out, float *c_out, cudaStream_t stream) {
+    DARB_TRACE("darb_lstm_step");
+    return lstm_step(h, I, H, B, x, h_prev, c_prev, bias, h_out, c_out, darb::kKernelNone, stream);
+}
+
+darb_status_t darb_internal_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                                      const float *h_prev, const float *c_prev, const float *bias, float *h_out,
+                                      float *c_out, int kernel, cudaStream_t stream) {
+    return lstm_step(h, I, H, B, x, h_prev, c_prev, bias, h_out, c_out, static_cast<darb::Kernel>(kernel), stream);
+}
+
+static darb_status_t gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x, const float *h_prev,
+                              const float *b_ih, const float *b_hh, float *h_out, darb::Kernel kernel,
+                              cudaStream_t stream) {
     darb_status_t st = check_step(h, I, H, B, 3, x, h_prev);
     if (st != DARB_OK) return st;
     if (h_out == nullptr) return DARB_ERR_INVALID_ARG;
@@ -851,8 +886,21 @@ darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, co
         if (overlaps(h_out, hb, ins[i], inb[i])) return DARB_ERR_INVALID_ARG;
     const bool early = early_ok(h, stream);
     return run_step(h, gate_floats_for(h, B, true), counter_ints_for(H, B), [&](darb::RnnScratch sc) {
-        return darb::launch_gru_step(format_of(h), I, H, B, x, h_prev, b_ih, b_hh, h_out, sc, stream, early);
+        return darb::launch_gru_step(format_of(h), I, H, B, x, h_prev, b_ih, b_hh, h_out, sc, stream, early, kernel);
     });
+}
+
+darb_status_t darb_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                            const float *h_prev, const float *b_ih, const float *b_hh,
+                            float *h_out, cudaStream_t stream) {
+    DARB_TRACE("darb_gru_step");
+    return gru_step(h, I, H, B, x, h_prev, b_ih, b_hh, h_out, darb::kKernelNone, stream);
+}
+
+darb_status_t darb_internal_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                                     const float *h_prev, const float *b_ih, const float *b_hh, float *h_out,
+                                     int kernel, cudaStream_t stream) {
+    return gru_step(h, I, H, B, x, h_prev, b_ih, b_hh, h_out, static_cast<darb::Kernel>(kernel), stream);
 }
 
 // Arrival counts of the sequence kernels' barrier stay below 2^32.

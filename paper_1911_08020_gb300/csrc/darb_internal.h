@@ -85,6 +85,31 @@ constexpr int kXresTables = 2;   // row-set tables of xres: 2 and 4 groups of th
 constexpr int kXresMaxGroups = 4;
 constexpr int kWorkSplits = 4;   // clusters of 1, 2, 4, 8 CTAs
 
+// The kernels that products from batch 5 on and steps choose from (the two of
+// xres: activations by tensor maps, and by plain copies); kKernelNone: the rule's
+// choice.
+enum Kernel : int { kKernelNone, kKernelRowlane, kKernelRows, kKernelBatch, kKernelXres, kKernelXresPlain };
+
+// Which of them the calling thread launched last, for tests that have to know
+// which one a call reaches.
+inline int &last_kernel() {
+    static thread_local int k = kKernelNone;
+    return k;
+}
+
+// How the calling thread's last sequence was cut, for the same purpose.
+struct SequenceCut {
+    int32_t tagged;          // h exchanged with tags, without barriers
+    int32_t tile, groups;    // columns of a tile; column groups
+    int32_t tiles_a_group;   // at most
+    int32_t c_on_chip;       // LSTM: cell state in shared memory
+    int32_t x_mode;          // seq::kX*
+};
+inline SequenceCut &last_sequence() {
+    static thread_local SequenceCut c{};
+    return c;
+}
+
 // What a unit of rnn_step.cuh is: a row, or a hidden unit of an LSTM (4 gate
 // rows) or a GRU (3).
 constexpr int kUnitRow = 0, kUnitLstm = 1, kUnitGru = 2, kUnitKinds = 3;
@@ -167,6 +192,11 @@ cudaError_t launch_encode(const EncodeTarget &t, const void *W, int64_t ldw, int
 cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y,
                               int64_t ldy, bool early, cudaStream_t stream);
 
+// The same product on one given kernel; cudaErrorNotSupported, nothing launched,
+// when that one cannot take the call.
+cudaError_t launch_spmm_on(const Format &f, Kernel kernel, const float *X, int64_t ldx, int64_t batch, float *Y,
+                           int64_t ldy, bool early, cudaStream_t stream);
+
 // Y = (the first col_limit columns of W_darb) (the first col_limit rows of X)
 // on xres; cudaErrorNotSupported, nothing launched, when it cannot take the call.
 cudaError_t launch_spmm_prefix(const Format &f, int64_t col_limit, const float *X, int64_t ldx, int64_t batch,
@@ -187,15 +217,18 @@ cudaError_t launch_spmm(const Format &f, const float *X, int64_t ldx, int64_t ba
 
 // `early` as for launch_spmm (the handle's values may be read before the
 // previous kernel on the stream finishes).  With null scratch a step that needs
-// some launches nothing and returns cudaErrorNotSupported.
+// some launches nothing and returns cudaErrorNotSupported, as does one that the
+// given kernel cannot take (rowlane_kernel takes batches up to 4, batch_kernel
+// those above).
 cudaError_t launch_lstm_step(const Format &f, int64_t I, int64_t H, int64_t B, const float *x,
                              const float *h_prev, const float *c_prev, const float *bias,
                              float *h_out, float *c_out, RnnScratch s, cudaStream_t stream,
-                             bool early = false);
+                             bool early = false, Kernel kernel = kKernelNone);
 
 cudaError_t launch_gru_step(const Format &f, int64_t I, int64_t H, int64_t B, const float *x,
                             const float *h_prev, const float *b_ih, const float *b_hh,
-                            float *h_out, RnnScratch s, cudaStream_t stream, bool early = false);
+                            float *h_out, RnnScratch s, cudaStream_t stream, bool early = false,
+                            Kernel kernel = kKernelNone);
 
 // T steps of an RNN layer in one persistent cooperative launch (sequence.cu).
 // row_m: the host copy of the per-row block sizes.  cudaErrorNotSupported
@@ -223,14 +256,6 @@ cudaError_t launch_rnn_step(const Format &f, const RnnArgs &ra, int mode, bool e
 // does not fit or is not expected to take less than limit_ns.
 cudaError_t launch_spmm_rows(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy,
                              bool early, double limit_ns, cudaStream_t stream);
-
-// Which of these kernels the calling thread launched last, for tests that have
-// to know which one a call reaches.
-enum Kernel : int { kKernelNone, kKernelRowlane, kKernelRows, kKernelBatch, kKernelXres, kKernelXresPlain };
-inline int &last_kernel() {
-    static thread_local int k = kKernelNone;
-    return k;
-}
 
 // Batch-tile width the RNN step kernels use for a batch of B (sizes the counters).
 int rnn_batch_tile(int64_t B);
@@ -260,5 +285,18 @@ darb_status_t lstm_step_view(darb_handle_t h, int64_t I, int64_t H, int64_t B, c
 
 }  // namespace darb
 
-// Exported beside the C ABI, for the tests: last_kernel().
-extern "C" DARB_API int darb_internal_last_kernel(void);
+// Exported beside the C ABI, for the tests: last_kernel(), last_sequence(), and darb_spmm,
+// darb_lstm_step and darb_gru_step on a given kernel (DARB_ERR_UNSUPPORTED when
+// it cannot take the call).
+extern "C" {
+DARB_API int darb_internal_last_kernel(void);
+DARB_API void darb_internal_last_sequence(int32_t cut[6]);
+DARB_API darb_status_t darb_internal_spmm(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y,
+                                          int64_t ldy, int kernel, cudaStream_t stream);
+DARB_API darb_status_t darb_internal_lstm_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                                               const float *h_prev, const float *c_prev, const float *bias,
+                                               float *h_out, float *c_out, int kernel, cudaStream_t stream);
+DARB_API darb_status_t darb_internal_gru_step(darb_handle_t h, int64_t I, int64_t H, int64_t B, const float *x,
+                                              const float *h_prev, const float *b_ih, const float *b_hh,
+                                              float *h_out, int kernel, cudaStream_t stream);
+}

@@ -41,10 +41,17 @@ static double rowlane_ns(const Format &f, int64_t B) {
 // batch 1 13.0 / 10.7 and at 64 82 / 60; but 6000 x 3000 at 64 25 / 39, and
 // batch 4 9.1 / 17.5 at 8000 x 4096.
 template <int MODE>
-static cudaError_t launch_step(const Format &f, const RnnArgs &ra, bool early, cudaStream_t stream) {
-    const double others_ns = ra.B <= 4 ? rowlane_ns(f, ra.B) : rnn_batch_ns(f, ra, MODE);
-    const cudaError_t e = launch_rnn_step(f, ra, MODE, early, others_ns, stream);
-    if (e != cudaErrorNotSupported || ra.counters == nullptr) return e;
+static cudaError_t launch_step(const Format &f, const RnnArgs &ra, bool early, Kernel kernel, cudaStream_t stream) {
+    if (kernel == kKernelNone || kernel == kKernelRows) {
+        const double limit_ns = kernel == kKernelRows ? 1e300
+                                : ra.B <= 4           ? rowlane_ns(f, ra.B)
+                                                      : rnn_batch_ns(f, ra, MODE);
+        const cudaError_t e = launch_rnn_step(f, ra, MODE, early, limit_ns, stream);
+        if (e != cudaErrorNotSupported || kernel == kKernelRows) return e;
+    } else if (kernel != (ra.B <= 4 ? kKernelRowlane : kKernelBatch)) {
+        return cudaErrorNotSupported;
+    }
+    if (ra.counters == nullptr) return cudaErrorNotSupported;
     if (ra.B <= 4)
         return f.bf16 ? rowlane::launch_any<true, MODE>(f, nullptr, 0, ra.B, nullptr, 0, ra, early, stream)
                       : rowlane::launch_any<false, MODE>(f, nullptr, 0, ra.B, nullptr, 0, ra, early, stream);
@@ -53,22 +60,23 @@ static cudaError_t launch_step(const Format &f, const RnnArgs &ra, bool early, c
 
 cudaError_t launch_lstm_step(const Format &f, int64_t I, int64_t H, int64_t B, const float *x,
                              const float *h_prev, const float *c_prev, const float *bias,
-                             float *h_out, float *c_out, RnnScratch s, cudaStream_t stream, bool early) {
+                             float *h_out, float *c_out, RnnScratch s, cudaStream_t stream, bool early,
+                             Kernel kernel) {
     RnnArgs ra{};
     ra.x = x; ra.h = h_prev; ra.gx = s.gates; ra.gh = nullptr; ra.counters = s.counters;
     ra.c_prev = c_prev; ra.bias = bias; ra.h_out = h_out; ra.c_out = c_out;
     ra.I = static_cast<int>(I); ra.H = static_cast<int>(H); ra.B = B;
-    return launch_step<kModeLstm>(f, ra, early, stream);
+    return launch_step<kModeLstm>(f, ra, early, kernel, stream);
 }
 
 cudaError_t launch_gru_step(const Format &f, int64_t I, int64_t H, int64_t B, const float *x,
                             const float *h_prev, const float *b_ih, const float *b_hh,
-                            float *h_out, RnnScratch s, cudaStream_t stream, bool early) {
+                            float *h_out, RnnScratch s, cudaStream_t stream, bool early, Kernel kernel) {
     RnnArgs ra{};
     ra.x = x; ra.h = h_prev; ra.gx = s.gates; ra.gh = s.gates ? s.gates + f.rows * B : nullptr; ra.counters = s.counters;
     ra.b_ih = b_ih; ra.b_hh = b_hh; ra.h_out = h_out;
     ra.I = static_cast<int>(I); ra.H = static_cast<int>(H); ra.B = B;
-    return launch_step<kModeGru>(f, ra, early, stream);
+    return launch_step<kModeGru>(f, ra, early, kernel, stream);
 }
 
 }  // namespace darb

@@ -981,6 +981,7 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     a.h_x = reinterpret_cast<float *>(ws + bar_bytes + cbytes);
     float *const xws = reinterpret_cast<float *>(ws + bar_bytes + cbytes + hx_bytes);
     a.x_tiles = a.x_mode != kXBulk ? nullptr : x_in_place ? a.x : xws;
+    last_sequence() = {a.tagged, bt, s.ngroups, s.tpg, a.c_on_chip, a.x_mode};
     const int64_t warps = H + (pre || x_copy ? T * I : 0);
     const unsigned grid = static_cast<unsigned>(std::min<int64_t>((warps + 7) / 8, int64_t(sm_count()) * 16));
     e = launch_ex(prep_kernel, dim3(grid), dim3(256), 0, stream, 1, false, a, s.lbt, h0, x_copy ? xws : nullptr,

@@ -55,6 +55,25 @@ cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int6
                   : batch::launch_any<false, kModeY>(f, X, ldx, batch, Y, ldy, none, early, stream);
 }
 
+cudaError_t launch_spmm_on(const Format &f, Kernel kernel, const float *X, int64_t ldx, int64_t batch, float *Y,
+                           int64_t ldy, bool early, cudaStream_t stream) {
+    const RnnArgs none{};
+    switch (kernel) {
+        case kKernelRows: return launch_spmm_rows(f, X, ldx, batch, Y, ldy, early, 1e300, stream);
+        case kKernelBatch:
+            return f.bf16 ? batch::launch_any<true, kModeY>(f, X, ldx, batch, Y, ldy, none, early, stream)
+                          : batch::launch_any<false, kModeY>(f, X, ldx, batch, Y, ldy, none, early, stream);
+        case kKernelXres:
+            if (!xres::maps(X, ldx)) return cudaErrorNotSupported;
+            return f.bf16 ? xres::launch_as<true, 32, false>(f, X, ldx, batch, Y, ldy, early, stream)
+                          : xres::launch_as<false, 32, false>(f, X, ldx, batch, Y, ldy, early, stream);
+        case kKernelXresPlain:
+            return f.bf16 ? xres::launch_as<true, 32, true>(f, X, ldx, batch, Y, ldy, early, stream)
+                          : xres::launch_as<false, 32, true>(f, X, ldx, batch, Y, ldy, early, stream);
+        default: return cudaErrorNotSupported;
+    }
+}
+
 cudaError_t launch_spmm_prefix(const Format &f, int64_t col_limit, const float *X, int64_t ldx, int64_t batch,
                                float *Y, int64_t ldy, bool early, cudaStream_t stream) {
     if (batch > 16 && col_limit > 0 && col_limit < f.cols) {

@@ -863,6 +863,11 @@ double expected_ns(const Format &f, int64_t batch, bool aligned) {
     return 2854.0 + (123.8 + (aligned ? 0.0 : 106.5)) * s.slice + 148.9 * s.gather + 1480.0 * s.units;
 }
 
+// Whether a tensor map can describe X: a 16-byte aligned base and rows.
+inline bool maps(const float *X, int64_t ldx) {
+    return reinterpret_cast<uintptr_t>(X) % 16 == 0 && (ldx * 4) % 16 == 0 && tensor_map_encoder() != nullptr;
+}
+
 // The slices arrive by tensor maps where X allows one (16-byte aligned base
 // and rows, a row pitch the encoder takes), else by 4-byte copies of the
 // consumer warps, 128 bytes of a row per warp.  A slice of 192 KB then takes
@@ -872,7 +877,7 @@ double expected_ns(const Format &f, int64_t batch, bool aligned) {
 template <bool BF16, int T>
 cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy, bool early,
                    cudaStream_t stream) {
-    if (reinterpret_cast<uintptr_t>(X) % 16 == 0 && (ldx * 4) % 16 == 0 && tensor_map_encoder() != nullptr) {
+    if (maps(X, ldx)) {
         const cudaError_t e = launch_as<BF16, T, false>(f, X, ldx, batch, Y, ldy, early, stream);
         if (e != cudaErrorNotSupported) return e;
     }

@@ -6,12 +6,15 @@ Tolerances (the bar every product is held to, from the arithmetic):
   S = sum_j |val_j * x_j| over the kept weights of that output (for S = 0, y
   must be 0).  tol = 1e-5 for fp32 weights and 2e-3 for bf16 weights; both
   kernels compute fp32 products of exactly widened weights and fp32 inputs and
-  add them in fp32, whose rounding error is far inside either bound;
+  add them in fp32, whose rounding error is far inside either bound (sum_tol is
+  the bound of that arithmetic, for either dtype);
 * RNN cells: the gate pre-activation errors (tol * S per gate, S including
   |bias|) pushed through the cell with |sigmoid'| <= 1/4, |tanh'| <= 1 and
   |sigmoid|, |tanh| <= 1, plus 2e-6 for the fp32 expf / tanhf calls.
 """
 from __future__ import annotations
+
+import ctypes
 
 import numpy as np
 import torch
@@ -30,6 +33,46 @@ ROWLANE, ROWS, BATCH, XRES, XRES_PLAIN = 1, 2, 3, 4, 5
 def last_kernel():
     """Which of these kernels this thread launched last."""
     return darb.lib().darb_internal_last_kernel()
+
+
+def last_sequence():
+    """How this thread's last sequence was cut (csrc/darb_internal.h, SequenceCut)."""
+    cut = (ctypes.c_int32 * 6)()
+    darb.lib().darb_internal_last_sequence(cut)
+    return dict(zip(("tagged", "tile", "groups", "tiles_a_group", "c_on_chip", "x_mode"), cut))
+
+
+def _p(a):
+    return ctypes.c_void_p(a.data_ptr() if a is not None else None)
+
+
+def spmm_on(kernel, h, X, Y):
+    """darb_spmm on one given kernel."""
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    st = darb.lib().darb_internal_spmm(h.ptr, _p(X), ctypes.c_int64(X.stride(0)), ctypes.c_int64(X.shape[1]), _p(Y),
+                                       ctypes.c_int64(Y.stride(0)), kernel, stream)
+    assert st == darb.OK, darb.status_string(st)
+    assert last_kernel() == kernel
+
+
+def step_on(kernel, cell, h, I, H, B, x, hp, cp, b1, b2, ho, co):
+    """darb_lstm_step or darb_gru_step on one given kernel."""
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    dims = (ctypes.c_int64(I), ctypes.c_int64(H), ctypes.c_int64(B))
+    L = darb.lib()
+    st = (L.darb_internal_lstm_step(h.ptr, *dims, _p(x), _p(hp), _p(cp), _p(b1), _p(ho), _p(co), kernel, stream)
+          if cell == "lstm" else
+          L.darb_internal_gru_step(h.ptr, *dims, _p(x), _p(hp), _p(b1), _p(b2), _p(ho), kernel, stream))
+    assert st == darb.OK, darb.status_string(st)
+    assert last_kernel() == kernel
+
+
+def sum_tol(n):
+    """A bound for fp32 sums of n products of exactly widened weights, in any
+    order, in units of sum |w x|: each term meets at most n roundings of 2^-24
+    (its product's and n - 1 additions'); and no more than the bar of fp32
+    weights."""
+    return min(TOL["f32"], (n + 1) * 2.0 ** -24)
 
 
 def dev():

@@ -1,6 +1,6 @@
 """Products on the kernel whose CTAs own rows (small and middling calls from batch
 5 on), and around the limits of the rule that picks it, against the oracle.
-Bounds as for every product (gpu_helpers)."""
+Bounds: fp32 sums (gpu_helpers.sum_tol)."""
 from __future__ import annotations
 
 import numpy as np
@@ -10,7 +10,7 @@ import torch
 import oracle
 from paper_1911_08020_gb300 import darb, synth
 
-from .gpu_helpers import TOL, assert_product_close, dev, encode_both, t
+from .gpu_helpers import assert_product_close, dev, encode_both, sum_tol, t
 
 pytestmark = pytest.mark.gpu
 
@@ -46,7 +46,7 @@ def test_product(rows, cols, mset, B, padx, pady, shift, dtype):
         for _ in range(2):   # with the records read early, and right after a re-encode
             full = torch.full((rows, B + pady), -7.0, device=dev())
             darb.darb_spmm(h, Xd, full[:, :B])
-            assert_product_close(full[:, :B].cpu().numpy(), Yr, A, TOL[dtype])
+            assert_product_close(full[:, :B].cpu().numpy(), Yr, A, sum_tol(-(-cols // m.min())))
             assert torch.all(full[:, B:] == -7.0)
             darb.darb_reencode(h, Wd)
         darb.darb_sync_status(h)
@@ -68,7 +68,7 @@ def test_unselected_activations_do_not_matter(B):
         Yr, A = oracle.darb_spmm(ref, X, with_absdot=True)
         X[1::8], X[2::8] = np.inf, np.nan
         Y = darb.darb_spmm(h, t(X)).cpu().numpy()
-        assert_product_close(Y, Yr, A, TOL["f32"])
+        assert_product_close(Y, Yr, A, sum_tol(cols // 8))
     finally:
         darb.darb_destroy(h)
 
@@ -90,6 +90,6 @@ def test_product_of_rows_sorted_by_block_size(rows, cols, sizes, B, dtype):
         Y = darb.darb_spmm(h, t(X)).cpu().numpy()
         darb.darb_sync_status(h)
         Yr, A = oracle.darb_spmm(ref, X, with_absdot=True)
-        assert_product_close(Y, Yr, A, TOL["f32"])
+        assert_product_close(Y, Yr, A, sum_tol(-(-cols // min(m for m, _ in sizes))))
     finally:
         darb.darb_destroy(h)

@@ -14,7 +14,7 @@ import torch
 
 import oracle
 from paper_1911_08020_gb300 import darb, synth
-from tests.gpu_helpers import TOL, dev, encode_both, gru_bound, lstm_bounds, t
+from tests.gpu_helpers import TOL, dev, encode_both, gru_bound, last_sequence, lstm_bounds, t
 
 pytestmark = pytest.mark.gpu
 
@@ -410,6 +410,40 @@ def test_no_room_for_the_copy_of_x(cell, I, H, B, monkeypatch):
         with pytest.raises(darb.DarbError) as e:
             check()
         assert e.value.status == darb.ERR_OOM
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
+# (cell, I, H, B, block sizes): several tiles a column group, exchanged behind the
+# barrier; x parts precomputed, x copied, and none; a ragged last tile; the
+# cell state on chip and off
+SEVERAL_TILES = [("lstm", 800, 1500, 61, (10, 20, 30), 1), ("lstm", 200, 1500, 61, (10, 20, 30), 1),
+                 ("lstm", 0, 1500, 61, (10, 20, 30), 1), ("gru", 800, 1500, 125, (10, 20, 30), 1),
+                 ("gru", 200, 1500, 61, (10, 20, 30), 1), ("gru", 0, 1500, 125, (10, 20, 30), 1),
+                 ("lstm", 100, 700, 1100, (16, 32, 64), 0)]
+
+
+@pytest.mark.parametrize("cell,I,H,B,mset,c_on_chip", SEVERAL_TILES)
+def test_sequence_of_several_tiles_a_group_behind_barriers(cell, I, H, B, mset, c_on_chip):
+    g = np.random.default_rng(51)
+    T = 3
+    gates = 4 if cell == "lstm" else 3
+    stored, m = _gate_matrix(g, gates, I, H, "f32", mset)
+    h, ref = encode_both(stored, m, "f32")
+    try:
+        xs = synth.activations(T * max(I, 1), B, seed=8).reshape(T, max(I, 1), B)[:, :I].copy()
+        h0, c0 = synth.state(H, B, seed=9), synth.state(H, B, seed=10)
+        b1, b2 = synth.bias(gates * H, seed=1), synth.bias(gates * H, seed=2)
+        if cell == "lstm":
+            _check_lstm_sequence(h, ref, T, I, H, B, xs, h0, c0, b1, TOL["f32"])
+        else:
+            _check_gru_sequence(h, ref, T, I, H, B, xs, h0, b1, b2, TOL["f32"])
+        cut = last_sequence()
+        assert not cut["tagged"] and cut["tiles_a_group"] > 1
+        assert cut["x_mode"] == (1 if 0 < 2 * I < H else 0)
+        if cell == "lstm":
+            assert cut["c_on_chip"] == c_on_chip
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
