@@ -41,7 +41,8 @@ struct darb_handle_s {
     int32_t xset_first[darb::kXresTables] = {}, nxsets[darb::kXresTables] = {};
     std::vector<int64_t> xset_prefix[darb::kXresTables];
     darb::SetGeo *d_xsets = nullptr;
-    darb::UnitSplits splits[darb::kUnitKinds];            // of rnn_step.cuh
+    std::vector<int64_t> row_cost;                        // of rnn_step.cuh: prefix sums
+    darb::UnitSplits splits[darb::kUnitKinds];
     int64_t val_elems = 0, off_words = 0;
     // device memory: one allocation holding the layout, values and offsets
     void *dmem = nullptr;
@@ -156,19 +157,15 @@ void build_layout(darb_handle_s *h, const int32_t *m) {
     h->off_words = off;
     build_work_tables(h);
     // a row costs its chunks, and about one more to form its outputs
-    std::vector<int32_t> row_cost(static_cast<size_t>(rows));
-    for (int64_t r = 0; r < rows; ++r)
-        row_cost[static_cast<size_t>(r)] =
-            (h->groups[static_cast<size_t>(h->rowloc[static_cast<size_t>(r)] / kSlots)].n + kChunk - 1) / kChunk + 1;
+    h->row_cost.assign(1, 0);
+    h->row_cost.reserve(static_cast<size_t>(rows) + 1);
+    for (int64_t r = 0; r < rows; ++r) {
+        const Group &g = h->groups[static_cast<size_t>(h->rowloc[static_cast<size_t>(r)] / kSlots)];
+        h->row_cost.push_back(h->row_cost.back() + (g.n + kChunk - 1) / kChunk + 1);
+    }
     for (int kind = 0; kind < darb::kUnitKinds; ++kind) {
-        const int64_t gates = kind == darb::kUnitRow ? 1 : kind == darb::kUnitLstm ? 4 : 3;
-        if (rows % gates != 0) continue;
-        const int64_t units = rows / gates;
-        h->splits[kind].build(units, [&](int64_t u) {
-            int64_t c = 0;
-            for (int64_t q = 0; q < gates; ++q) c += row_cost[static_cast<size_t>(q * units + u)];
-            return c;
-        });
+        const int gates = kind == darb::kUnitRow ? 1 : kind == darb::kUnitLstm ? 4 : 3;
+        if (rows % gates == 0) h->splits[kind].set(h->row_cost.data(), rows / gates, gates);
     }
     // tiles of tb(m) blocks, every row in order; tb a multiple of the chunk
     auto tiles_of = [h, rows, cols](std::vector<darb::EncTile> &out, int (*tb_of)(int)) {

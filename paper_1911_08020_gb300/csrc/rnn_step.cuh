@@ -507,6 +507,19 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
         Plan p{};
         p.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
         p.members = std::max(1, std::min({sms / p.ntiles, ra.H, kMaxMembers}));
+        const TileCost &cost = (MODE == kModeY ? kProductCost : kStepCost)[l - kMinLbt];
+        const bool ragged = ra.B % bt != 0;
+        const double per_byte = !aligned            ? cost.stage4
+                                : l == 5 && !ragged ? cost.boxes
+                                                    : cost.stage16 + (ragged ? cost.ragged : 0) +
+                                                          (p.ntiles > 1 ? cost.part : 0);
+        const int waves = (p.ntiles * p.members + sms - 1) / sms;
+        auto expected_ns = [&](double busiest, double units) {
+            return cost.fixed + waves * (double(K) * bt * 4 * per_byte + busiest * kChunk * cost.weight +
+                                         units * bt * cost.output);
+        };
+        // no split goes below the means
+        if (!(expected_ns(double(splits.total()) / p.members, double(ra.H) / p.members) < best_ns)) continue;
         UnitSplit local;
         const UnitSplit &split = splits.get(p.members, local);
         // ranges by cost give some members many light units, whose rows and partial
@@ -516,15 +529,7 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
             const size_t bytes = lay_out(p, r.most_units, bt);
             if (bytes == 0 || bytes > kSmemCap) continue;
             p.by_cost = by_cost;
-            const TileCost &cost = (MODE == kModeY ? kProductCost : kStepCost)[l - kMinLbt];
-            const bool ragged = ra.B % bt != 0;
-            const double per_byte = !aligned            ? cost.stage4
-                                    : l == 5 && !ragged ? cost.boxes
-                                                        : cost.stage16 + (ragged ? cost.ragged : 0) +
-                                                              (p.ntiles > 1 ? cost.part : 0);
-            const int waves = (p.ntiles * p.members + sms - 1) / sms;
-            const double ns = cost.fixed + waves * (double(K) * bt * 4 * per_byte + double(r.busiest) * kChunk * cost.weight +
-                                                    double(r.most_units) * bt * cost.output);
+            const double ns = expected_ns(double(r.busiest), double(r.most_units));
             if (ns < best_ns) {
                 best_ns = ns;
                 best = p;

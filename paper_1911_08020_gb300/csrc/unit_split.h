@@ -13,7 +13,6 @@
 #include <atomic>
 #include <cstdint>
 #include <new>
-#include <vector>
 
 namespace darb {
 
@@ -41,20 +40,18 @@ public:
         for (auto &s : kept_) delete s.load(std::memory_order_relaxed);
     }
 
-    // cost(u): of unit u, at least 1
-    template <class Cost>
-    void build(int64_t units, Cost cost) {
-        prefix_.resize(static_cast<size_t>(units) + 1);
-        prefix_[0] = 0;
-        for (int64_t u = 0; u < units; ++u)
-            prefix_[static_cast<size_t>(u) + 1] = prefix_[static_cast<size_t>(u)] + cost(u);
+    // Units of `gates` rows, unit u rows u, units + u, 2 units + u ...; prefix[r]:
+    // the cost of rows [0, r), at least 1 each, kept by the caller.
+    void set(const int64_t *prefix, int64_t units, int gates) {
+        prefix_ = prefix;
+        units_ = units;
+        gates_ = gates;
     }
 
-    int64_t units() const { return static_cast<int64_t>(prefix_.size()) - 1; }
-    int64_t total() const { return prefix_.back(); }
+    int64_t total() const { return prefix_[units_ * gates_]; }
 
     // The split over `members` (1 .. min(units, kMaxMembers)).  Worked out by the
-    // first call that asks for it (some microseconds) and kept; any thread may
+    // first call that asks for it (about a microsecond) and kept; any thread may
     // call.  Without memory to keep it, it is worked out in `local`.
     const UnitSplit &get(int members, UnitSplit &local) const {
         std::atomic<UnitSplit *> &slot = kept_[members];
@@ -73,25 +70,39 @@ public:
 
 private:
     void work_out(int members, UnitSplit &s) const {
-        const int64_t n = units(), all = total();
-        const int64_t *const p = prefix_.data();
+        const int64_t n = units_, all = total();
+        auto p = [&](int64_t u) {   // the cost of units [0, u)
+            int64_t c = prefix_[u];
+            for (int q = 1; q < gates_; ++q) c += prefix_[q * n + u] - prefix_[q * n];
+            return c;
+        };
         s.equal = {0, static_cast<int32_t>((n + members - 1) / members)};
-        for (int q = 0; q < members; ++q)
-            s.equal.busiest = std::max(s.equal.busiest, p[n * (q + 1) / members] - p[n * q / members]);
+        for (int64_t q = 0, before = 0; q < members; ++q) {
+            const int64_t upto = p(n * (q + 1) / members);
+            s.equal.busiest = std::max(s.equal.busiest, upto - before);
+            before = upto;
+        }
         // by cost: a member ends with the unit that brings the running sum nearest
         // to its share, and leaves one unit for every later member
         s.by_cost = {0, 0};
         s.start[0] = 0;
+        int64_t before = 0;
+        int64_t length = n / members;   // of the range before: about that of the next
         for (int q = 0; q < members; ++q) {
             const int64_t from = s.start[q], last = n - (members - 1 - q);
             int64_t to = last;
             if (q + 1 < members) {
                 const int64_t share = all / members * (q + 1) + all % members * (q + 1) / members;
-                to = std::lower_bound(p + from + 1, p + last, share) - p;
-                if (to > from + 1 && p[to] - share > share - p[to - 1]) --to;
+                to = std::min(from + std::max<int64_t>(length, 1), last);   // the first unit past the share
+                while (to < last && p(to) < share) ++to;
+                while (to > from + 1 && p(to - 1) >= share) --to;
+                if (to > from + 1 && p(to) - share > share - p(to - 1)) --to;
             }
+            length = to - from;
             s.start[q + 1] = static_cast<int32_t>(to);
-            s.by_cost.busiest = std::max(s.by_cost.busiest, p[to] - p[from]);
+            const int64_t upto = p(to);
+            s.by_cost.busiest = std::max(s.by_cost.busiest, upto - before);
+            before = upto;
             s.by_cost.most_units = std::max(s.by_cost.most_units, static_cast<int32_t>(to - from));
         }
         // Equal numbers unless the busiest member gets 5% less: their members have
@@ -99,7 +110,9 @@ private:
         s.prefer_by_cost = s.by_cost.busiest * 20 < s.equal.busiest * 19;
     }
 
-    std::vector<int64_t> prefix_ = {0};
+    const int64_t *prefix_ = nullptr;
+    int64_t units_ = 0;
+    int gates_ = 1;
     mutable std::atomic<UnitSplit *> kept_[kMaxMembers + 1] = {};
 };
 
