@@ -29,19 +29,22 @@
 // with the launch) and, for wide matrices, the gather.  A step (us, in a graph
 // of steps) against the kernels whose gate sums meet through clusters, scratch
 // and counters (rowlane_kernel, batch_kernel): LSTM 4096 x 1280 fp32 at batch
-// 1 / 8 / 32 / 64: 6.3 / 5.8 / 7.6 / 10.5 against 7.8 / 17.0 / 25.0 / 30.3; GRU
-// 3072 x 2048 bf16 at batch 64: 10.9 against 32.3; LSTM 6000 x 3000 bf16 at
-// batch 20: 16.0 against 37.9, fp32 at batch 37: 27.5 against 212.  Those kernels
-// remain for inputs too tall to stage at 4 columns (some 14000 rows).
+// 1 / 8 / 32 / 64: 6.1 / 5.7 / 7.2 / 10.4 against 7.6 / 16.9 / 25.0 / 29.4; GRU
+// 3072 x 2048 bf16 at batch 64: 11.0 against 32.8; LSTM 6000 x 3000 bf16 at
+// batch 20: 16.0 against 36.8, fp32 at batch 37: 23.2 against 78.5.  Those
+// kernels remain for inputs too tall to stage at 4 columns (some 14000 rows),
+// for more than 1024 columns, and where they are expected to be faster
+// (rnn.cu): above some 3600 stacked rows the tiles are narrow.
 //
 // A plain product (kModeY; the rows are the units, X the whole input) takes
 // this kernel from batch 5 on while it is expected to be faster than the
-// kernels that stream through clusters, whose fixed part is larger but whose
-// gather is cheaper.  us against what those took: 1024 x 1024 fp32 at batch 6 /
-// 8 / 24 / 64: 4.0 / 3.7 / 4.0 / 4.4 against 27.6 / 4.9 / 10.2 / 10.1; 6000 x
-// 3000 fp32 at 6 / 8 / 16: 8.7 / 7.4 / 9.7 against 80 / 15 / 14, but 16.2 against
-// 11.8 at 32; 2000 x 2500 fp32 at 24 / 64: 6.3 / 9.1 against 12.2 / 11.7, but
-// 13.4 against 13.0 at 100; 4096 x 4096 bf16 at 8: 5.6 against 8.2.
+// kernels that stream through clusters (spmm_batch.cu), whose fixed part is
+// larger but whose gather is cheaper.  us against the faster of those: 1024 x
+// 1024 fp32 at batch 6 / 8 / 24 / 64: 3.6 / 3.4 / 3.6 / 4.1 against 10.7 / 4.7 /
+// 6.8 / 7.6; 6000 x 3000 fp32 at 6 / 8 / 16: 8.3 / 7.1 / 8.9 against 12.9 / 13.0 /
+// 13.0, but 14.8 against 11.6 at 32; 2000 x 2500 fp32 at 24 / 64: 6.0 / 8.6
+// against 6.5 / 8.8; 4096 x 4096 bf16 at 8: 5.2 against 7.9, but 8.5 against 7.4
+// at 16.
 #pragma once
 
 #include "kernels_common.cuh"

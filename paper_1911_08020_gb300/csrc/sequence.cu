@@ -35,8 +35,8 @@
 // staging 2500, the cell 1800.  One column group instead of one a tile stages
 // every column in every CTA: GRU 3072 x 2048 at batch 64 took 11.0 against 8.7
 // us a step.  Against one lane a column, tensor-map staging and all CTAs in one
-// barrier, whole calls went from 3131 to 1505 us (that GRU, 200 steps), 507 to
-// 329 (the LSTM above, 35 steps), 520 to 309 (LSTM 4096 x 1280 fp32, batch 1,
+// barrier, whole calls went from 3131 to 1491 us (that GRU, 200 steps), 507 to
+// 325 (the LSTM above, 35 steps), 520 to 307 (LSTM 4096 x 1280 fp32, batch 1,
 // 100 steps), and 2592 to 545 where the batch is no multiple of 4 (GRU 2100 x
 // 1000, batch 37, 100 steps).
 #include "darb_internal.h"
@@ -853,8 +853,10 @@ static cudaError_t launch_seq_t(const Format &f, const int32_t *row_m, seq::SeqA
     // staging of in_rows rows and the gather of the CTA's kept weights.  A
     // narrow tile stages less but keeps more weights a CTA, each of which
     // costs its own share of a load, and a quarter-warp's staged rows then
-    // share banks (cycles per weight: measured on the gate matrices of
-    // 4096 x 1280 fp32 and 6000 x 3000 bf16).
+    // share banks (cycles per weight: measured on two gate matrices only,
+    // 4096 x 1280 fp32 and 6000 x 3000 bf16; of 240 sequences of other sizes, 64
+    // to 1500 units at batches 1 to 128, none took longer than with one lane a
+    // column behind one barrier).
     Shape shapes[(kMaxLbt + 1) * 80];
     int nshapes = 0;
     for (int lbt = 0; lbt <= kMaxLbt && (lbt == 0 || (1 << (lbt - 1)) < B); ++lbt) {

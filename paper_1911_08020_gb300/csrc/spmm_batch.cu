@@ -26,9 +26,8 @@ cudaError_t launch_spmm_batch(const Format &f, const float *X, int64_t ldx, int6
     // The rows kernel has to be expected to take 5% less.  Over 611 products of
     // 47 shapes, block sizes mixed and in runs, at 26 batches from 5 to 256,
     // each timed on every kernel, the choice is on average 2% above the fastest;
-    // 9 were more than 3% above the cluster kernel, the worst 14% (4096 x 4096
-    // fp32 at batch 16, half the rows in blocks of 8 and half of 64: 12.3 us
-    // against 11.0).
+    // 9 were more than 3% above the cluster kernel, the worst 14% (700 x 6000 fp32
+    // at batch 32: 9.3 us against 8.1).
     const bool aligned = reinterpret_cast<uintptr_t>(X) % 16 == 0 && ldx % 4 == 0;
     const bool streams = batch <= 16 && aligned;   // batch_kernel, else xres
     const double kept = double(f.set_prefix[0][f.nitems[0][0]]) * kSlots * kChunk;
