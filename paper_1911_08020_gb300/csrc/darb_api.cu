@@ -528,6 +528,8 @@ extern "C" {
 
 int darb_internal_last_kernel(void) { return darb::last_kernel(); }
 
+int darb_internal_last_split(void) { return darb::last_split(); }
+
 void darb_internal_last_sequence(int32_t cut[6]) {
     static_assert(sizeof(darb::SequenceCut) == 6 * sizeof(int32_t), "six words");
     std::memcpy(cut, &darb::last_sequence(), sizeof(darb::SequenceCut));

@@ -97,6 +97,12 @@ inline int &last_kernel() {
     return k;
 }
 
+// The column split of the calling thread's last product on xres.
+inline int &last_split() {
+    static thread_local int c = 0;
+    return c;
+}
+
 // How the calling thread's last sequence was cut, for the same purpose.
 struct SequenceCut {
     int32_t tagged;          // h exchanged with tags, without barriers
@@ -285,11 +291,12 @@ darb_status_t lstm_step_view(darb_handle_t h, int64_t I, int64_t H, int64_t B, c
 
 }  // namespace darb
 
-// Exported beside the C ABI, for the tests: last_kernel(), last_sequence(), and darb_spmm,
+// Exported beside the C ABI, for the tests: last_kernel(), last_split(), last_sequence(), and darb_spmm,
 // darb_lstm_step and darb_gru_step on a given kernel (DARB_ERR_UNSUPPORTED when
 // it cannot take the call).
 extern "C" {
 DARB_API int darb_internal_last_kernel(void);
+DARB_API int darb_internal_last_split(void);
 DARB_API void darb_internal_last_sequence(int32_t cut[6]);
 DARB_API darb_status_t darb_internal_spmm(darb_handle_t h, const float *X, int64_t ldx, int64_t batch, float *Y,
                                           int64_t ldy, int kernel, cudaStream_t stream);

@@ -660,14 +660,18 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
     // splits with kMinStages or more, the one whose clusters occupy the most
     // SMs, then the deeper ring, then the smaller split; a shallower ring only
     // when no split has that.  Where that leaves its clusters with fewer than
-    // two units, most SMs idle while a unit runs: a finer split that is expected
-    // to take the least time then, if it is well below (in group-chunks of
-    // multiplying, 137 ns: the load of the slice, and the units of a cluster,
-    // each its share of the set's work and a fixed cost; more where partial sums
-    // cross CTAs).  1000 x 7000 bf16 at batch 24: 8.5 us against 10.8, 2000 x
-    // 5000 at 64: 10.4 against 11.2.  By that estimate alone 5000 x 700 at
-    // batch 256 went from 18.0 to 20.1, and a coarser split has longer chains
-    // of fp32 additions (1500 x 1500 at 100: 1.38 times the error).
+    // two units, most SMs idle while a unit runs: a finer split then, the one of
+    // the least estimated time (in group-chunks of multiplying, 137 ns: the load
+    // of the slice, and the units of a cluster, each its share of the set's work
+    // and a fixed cost; more where partial sums cross CTAs), if its longest run
+    // is below too (`longest`).  us, finer against coarser: 1000 x 7000 bf16 at
+    // batch 24 8.5 / 10.8, 1834 x 3097 bf16 at 24 7.1 / 8.5, 445 x 939 bf16 with a
+    // tenth of the rows in blocks of 4 and the rest of 64 at 44 5.3 / 15.2.  By the
+    // estimate alone, where it is 15% below, 5 of 60 calls took 4 to 22% longer
+    // (739 x 2652 at batch 256 11.5 / 9.4: a finer split has fewer clusters, and
+    // two units that are not the mean may meet in one); by the longest run one of
+    // 76, by 4%.  Of 639 products 3 are 15 to 19% above the finer split they could
+    // have had.
     struct Split {
         Plan p;
         uint32_t smem;
@@ -715,18 +719,59 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
         }
         if (least.sms == 0 || (s.deep != least.deep ? s.deep : s.cost < least.cost)) least = s;
     }
-    const Split &best = few && least.p.C > most.p.C && least.deep == most.deep && least.cost < 0.85 * most.cost ? least : most;
-    Plan p = best.p;
-    const uint32_t smem = best.smem;
-    const int64_t best_sms = best.sms;
-    if (best_sms <= 0) return cudaErrorNotSupported;
-    const int64_t occ = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(p.C, smem), kMaxClusters);
     // Row sets of about 4 heaviest groups (table 1: 128 rows, the consumers'
     // efficient layout) when they still give every cluster 2 units or more;
     // else sets of about 2 (table 0), whose finer units balance better.  (At
     // 3 units a cluster FC6 batch 64 took table 0 on clusters of 6: 20.3
     // against 18.8 us; at 1, FC7 batch 64 took table 1: 13.8 against 12.8.)
-    const int table = tiles * f.nxsets[1] >= 2 * occ ? 1 : 0;
+    auto table_of = [&](int64_t ncl) { return tiles * f.nxsets[1] >= 2 * ncl ? 1 : 0; };
+    // The ranks of a cluster go through a unit together, so a unit costs what its
+    // busiest rank streams -- its set's groups times the most chunks any slice's
+    // blocks touch -- plus a fixed cost per unit (the hand-off of its partial
+    // sums and the start of its rounds): prefix sums over the sets.
+    auto unit_costs = [&](const Plan &q, int table, std::vector<int64_t> &cost) {
+        const SetGeo *hs = f.xsets_host[table];
+        const int nsets = f.nxsets[table];
+        cost.assign(static_cast<size_t>(nsets) + 1, 0);
+        int64_t most = 0;
+        for (int s = 0; s < nsets; ++s) {
+            // (the same for the sets of a bin, which are neighbours)
+            if (s == 0 || hs[s].m != hs[s - 1].m) most = 0;
+            for (int qq = 0; qq < q.C && (s == 0 || hs[s].m != hs[s - 1].m); ++qq) {
+                const int64_t lo = int64_t(qq) * q.S, hi = lo + q.S;
+                const int64_t j0 = std::min<int64_t>(hs[s].n, (lo + hs[s].m - 1) / hs[s].m);
+                const int64_t j1 = std::min<int64_t>(hs[s].n, (hi + hs[s].m - 1) / hs[s].m);
+                if (j1 > j0) most = std::max<int64_t>(most, (j1 + kChunk - 1) / kChunk - j0 / kChunk);
+            }
+            cost[static_cast<size_t>(s) + 1] = cost[static_cast<size_t>(s)] + hs[s].ng * most + kUnitCost;
+        }
+    };
+    thread_local std::vector<int64_t> cost;   // host; reused across calls
+    // A bound from below of a split's longest run, with its slice's load, in
+    // group-chunks: the heaviest unit, or where some clusters take two units the
+    // lightest neighbours and the mean of the clusters.
+    auto longest = [&](const Split &q) {
+        const int64_t ncl = q.sms / q.p.C;
+        const int table = table_of(ncl), nsets = f.nxsets[table];
+        unit_costs(q.p, table, cost);
+        int64_t unit = 0, pair = INT64_MAX;
+        for (int s = 0; s < nsets; ++s) {
+            unit = std::max(unit, cost[s + 1] - cost[s]);
+            if (s + 2 <= nsets) pair = std::min(pair, cost[s + 2] - cost[s]);
+        }
+        if (nsets == 1) pair = 2 * unit;
+        double run = double(unit);
+        if (tiles * nsets > ncl) run = std::max({run, double(pair), double(cost[nsets]) * double(tiles) / double(ncl)});
+        return double(q.p.nboxes) * q.p.box_rows * (T * 4 / (77.0 * 137.0)) + run + (q.p.C > 1 ? kClusterCost : 0);
+    };
+    const bool finer = few && least.p.C > most.p.C && least.deep == most.deep && longest(least) < 0.9 * longest(most);
+    const Split &best = finer ? least : most;
+    Plan p = best.p;
+    const uint32_t smem = best.smem;
+    const int64_t best_sms = best.sms;
+    if (best_sms <= 0) return cudaErrorNotSupported;
+    const int64_t occ = std::min<int64_t>(max_clusters<BF16, T, PLAIN>(p.C, smem), kMaxClusters);
+    const int table = table_of(occ);
     const int nsets = f.nxsets[table];
     const int64_t units = tiles * nsets;
     p.table = table;
@@ -734,29 +779,13 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
     const int ncl = static_cast<int>(std::min<int64_t>(occ, units));
     if (ncl <= 0) return cudaErrorNotSupported;
     // Contiguous runs of units, at most ncl of them, whose longest is as short
-    // as it can be.  The ranks of a cluster go through a unit together, so a
-    // unit costs what its busiest rank streams -- its set's groups times the
-    // most chunks any slice's blocks touch -- plus a fixed cost per unit (the
-    // hand-off of its partial sums and the start of its rounds); a run that
-    // crosses into the next batch tile also pays for the drain of its
-    // consumers and the load of the new slice.  kUnitCost and kSwitchCost
-    // were swept on FC6/FC7 at batch 64 and 256 (10 and 40 group-chunks of
-    // multiplying).  The bound on a run is found by bisection, each candidate
-    // tried by a greedy pass that closes a run where the next unit would pass
-    // it.
-    thread_local std::vector<int64_t> cost;   // host; reused across calls
-    const SetGeo *hs = f.xsets_host[table];
-    cost.assign(static_cast<size_t>(nsets) + 1, 0);
-    for (int s = 0; s < nsets; ++s) {
-        int64_t most = 0;
-        for (int qq = 0; qq < p.C; ++qq) {
-            const int64_t lo = int64_t(qq) * p.S, hi = lo + p.S;
-            const int64_t j0 = std::min<int64_t>(hs[s].n, (lo + hs[s].m - 1) / hs[s].m);
-            const int64_t j1 = std::min<int64_t>(hs[s].n, (hi + hs[s].m - 1) / hs[s].m);
-            if (j1 > j0) most = std::max<int64_t>(most, (j1 + kChunk - 1) / kChunk - j0 / kChunk);
-        }
-        cost[static_cast<size_t>(s) + 1] = cost[static_cast<size_t>(s)] + hs[s].ng * most + kUnitCost;
-    }
+    // as it can be.  A run that crosses into the next batch tile also pays for
+    // the drain of its consumers and the load of the new slice.  kUnitCost and
+    // kSwitchCost were swept on FC6/FC7 at batch 64 and 256 (10 and 40
+    // group-chunks of multiplying).  The bound on a run is found by bisection,
+    // each candidate tried by a greedy pass that closes a run where the next
+    // unit would pass it.
+    unit_costs(p, table, cost);
     const int64_t *pre = cost.data();
     // One greedy pass for a bound: a run takes its first unit whatever that
     // costs, then the following units while they fit, a unit that opens a
@@ -817,6 +846,7 @@ cudaError_t launch_as(const Format &f, const float *X, int64_t ldx, int64_t batc
             return cudaErrorNotSupported;
     }
     last_kernel() = PLAIN ? kKernelXresPlain : kKernelXres;
+    last_split() = p.C;
     return launch_ex(xres_kernel<BF16, T, PLAIN>, dim3(static_cast<unsigned>(nrun * p.C)), dim3(kThreads), smem, stream,
                      static_cast<unsigned>(p.C), true, f, X, ldx, batch, Y, ldy, xmap, p);
 }

@@ -35,6 +35,11 @@ def last_kernel():
     return darb.lib().darb_internal_last_kernel()
 
 
+def last_split():
+    """The column split of this thread's last product on the resident slices."""
+    return darb.lib().darb_internal_last_split()
+
+
 def last_sequence():
     """How this thread's last sequence was cut (csrc/darb_internal.h, SequenceCut)."""
     cut = (ctypes.c_int32 * 6)()

@@ -11,7 +11,7 @@ import oracle
 from paper_1911_08020_gb300 import darb, synth
 
 from .gpu_helpers import (BATCH, ROWLANE, ROWS, XRES, XRES_PLAIN, assert_product_close, dev, encode_both, gru_bound,
-                          last_kernel, lstm_bounds, spmm_on, step_on, sum_tol, t)
+                          last_kernel, last_split, lstm_bounds, spmm_on, step_on, sum_tol, t)
 
 pytestmark = pytest.mark.gpu
 
@@ -108,6 +108,31 @@ def test_rule(rows, cols, mset, dtype, B, pad, kernel):
         assert last_kernel() == kernel
         Yr, A = oracle.darb_spmm(ref, X, with_absdot=True)
         assert_product_close(Y, Yr, A, sum_tol(n))
+        darb.darb_sync_status(h)
+    finally:
+        darb.darb_destroy(h)
+
+
+# rows, cols, (block size, rows) in order, batch, and the columns' splits with and
+# without a finer one where clusters would have fewer than two units: a unit
+# each in the finer split (faster), two that meet in one (22% slower)
+@pytest.mark.parametrize("rows,cols,runs,B,finer", [
+    (1000, 7000, ((10, 250), (15, 250), (20, 250), (30, 250)), 24, True),
+    (739, 2652, ((16, 300), (32, 212), (64, 227)), 256, False),
+])
+def test_finer_split_only_where_its_longest_run_is_shorter(rows, cols, runs, B, finer):
+    g = np.random.default_rng(74)
+    w = (0.05 * g.standard_normal((rows, cols))).astype(np.float32)
+    m = np.concatenate([np.full(n, size, np.int32) for size, n in runs])
+    h, ref = encode_both(synth.f32_to_bf16_bits(w), m, "bf16")
+    try:
+        X, Xd = _x(cols, B, 0, 0)
+        Y = torch.empty((rows, B), device=dev())
+        spmm_on(XRES, h, Xd, Y)
+        fewest = -(-cols * 128 // (227 * 1024 - 16384))   # slices that leave room for the partial sums
+        assert last_split() > fewest + 1 if finer else last_split() <= fewest + 1
+        Yr, A = oracle.darb_spmm(ref, X, with_absdot=True)
+        assert_product_close(Y.cpu().numpy(), Yr, A, sum_tol(-(-cols // m.min())))
         darb.darb_sync_status(h)
     finally:
         darb.darb_destroy(h)
