@@ -75,9 +75,9 @@ def _costs(order, rows, cols):
     return -(-(-(-cols // m)) // 8) + 1
 
 
-@pytest.mark.parametrize("gates", [1, 3, 4])
-@pytest.mark.parametrize("members", [1, 2, 5, 19, 76, 152, 160])
-@pytest.mark.parametrize("rows,cols", [(160, 300), (300, 5000), (1024, 1024), (4096, 9216)])
+@pytest.mark.parametrize("gates", [1, 4])
+@pytest.mark.parametrize("members", [1, 19, 152])
+@pytest.mark.parametrize("rows,cols", [(160, 300), (1024, 1024), (4096, 9216)])
 @pytest.mark.parametrize("order", ["tenth", "tenth_last", "half", "sorted", "mixed", "equal", "extreme"])
 def test_no_member_has_much_more_than_the_mean(program, order, rows, cols, members, gates):
     by_row = np.concatenate([np.random.default_rng(q).permutation(_costs("mixed", rows, cols)) if q else
