@@ -482,8 +482,7 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
     const UnitSplits &splits = *f.splits[MODE == kModeLstm ? kUnitLstm : MODE == kModeGru ? kUnitGru : kUnitRow];
     const int sms = sm_count();
     const bool aligned = aligned16(ra, MODE == kModeY, MODE == kModeY ? ldx : ra.B);
-    int lbt = -1;
-    size_t smem = 0;
+    int lbt = -1, best_units = 0;
     Plan best{};
     double best_ns = limit_ns;
     // the places of a CTA's shared memory for members of up to `units` units, and
@@ -505,44 +504,62 @@ cudaError_t launch(const Format &f, const RnnArgs &ra, bool early, cudaStream_t 
         p.c_off = take(MODE == kModeLstm ? size_t(units) * bt * 4 : 0);
         return o;
     };
+    // The tile widths, each with the time it would take if its members' shares
+    // were equal: no split goes below that, so the widths are tried in the order
+    // of it, and splits are worked out (once a handle) only for those that could
+    // be the best.
+    struct Tile {
+        int l, ntiles, members;
+        double ns, staging, weight, output;
+        double expected_ns(double busiest, double units) const { return staging + busiest * weight + units * output; }
+    } tiles[kMaxLbt - kMinLbt + 1];
+    int ntiles = 0;
     for (int l = kMinLbt; l <= kMaxLbt && (l == kMinLbt || (1 << (l - 1)) < ra.B); ++l) {
         const int bt = 1 << l;
-        Plan p{};
-        p.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
-        p.members = std::max(1, std::min({sms / p.ntiles, ra.H, kMaxMembers}));
+        Tile &t = tiles[ntiles++];
+        t.l = l;
+        t.ntiles = static_cast<int>((ra.B + bt - 1) / bt);
+        t.members = std::max(1, std::min({sms / t.ntiles, ra.H, kMaxMembers}));
         const TileCost &cost = (MODE == kModeY ? kProductCost : kStepCost)[l - kMinLbt];
         const bool ragged = ra.B % bt != 0;
         const double per_byte = !aligned            ? cost.stage4
                                 : l == 5 && !ragged ? cost.boxes
                                                     : cost.stage16 + (ragged ? cost.ragged : 0) +
-                                                          (p.ntiles > 1 ? cost.part : 0);
-        const int waves = (p.ntiles * p.members + sms - 1) / sms;
-        auto expected_ns = [&](double busiest, double units) {
-            return cost.fixed + waves * (double(K) * bt * 4 * per_byte + busiest * kChunk * cost.weight +
-                                         units * bt * cost.output);
-        };
-        // no split goes below the means
-        if (!(expected_ns(double(splits.total()) / p.members, double(ra.H) / p.members) < best_ns)) continue;
+                                                          (t.ntiles > 1 ? cost.part : 0);
+        const int waves = (t.ntiles * t.members + sms - 1) / sms;
+        t.staging = cost.fixed + waves * double(K) * bt * 4 * per_byte;
+        t.weight = waves * kChunk * cost.weight;
+        t.output = waves * bt * cost.output;
+        t.ns = t.expected_ns(double(splits.total()) / t.members, double(ra.H) / t.members);
+    }
+    for (; ntiles > 0; --ntiles) {
+        Tile *const next =
+            std::min_element(tiles, tiles + ntiles, [](const Tile &p, const Tile &q) { return p.ns < q.ns; });
+        const Tile t = *next;
+        *next = tiles[ntiles - 1];
+        if (!(t.ns < best_ns)) break;
         UnitSplit local;
-        const UnitSplit &split = splits.get(p.members, local);
+        const UnitSplit &split = splits.get(t.members, local);
         // ranges by cost give some members many light units, whose rows and partial
         // sums may not fit; equal numbers then
         for (int by_cost = split.prefer_by_cost ? 1 : 0; by_cost >= 0; --by_cost) {
             const UnitRanges &r = by_cost ? split.by_cost : split.equal;
-            const size_t bytes = lay_out(p, r.most_units, bt);
+            const size_t bytes = lay_out(best, r.most_units, 1 << t.l);
             if (bytes == 0 || bytes > kSmemCap) continue;
-            p.by_cost = by_cost;
-            const double ns = expected_ns(double(r.busiest), double(r.most_units));
+            const double ns = t.expected_ns(double(r.busiest), double(r.most_units));
             if (ns < best_ns) {
                 best_ns = ns;
-                best = p;
-                lbt = l;
-                smem = bytes;
+                best.ntiles = t.ntiles;
+                best.members = t.members;
+                best.by_cost = by_cost;
+                best_units = r.most_units;
+                lbt = t.l;
             }
             break;
         }
     }
     if (lbt < 0) return cudaErrorNotSupported;
+    const size_t smem = lay_out(best, best_units, 1 << lbt);
     if (best.by_cost) {
         UnitSplit local;
         const UnitSplit &split = splits.get(best.members, local);
