@@ -904,7 +904,7 @@ inline bool maps(const float *X, int64_t ldx) {
 // ~1500 copy instructions of the SM's load unit (3 us) and no register
 // round trip: 3001 x 4099 fp32 at batch 999 takes 131 us, of which the gather's
 // bound is 76 (with batch_kernel's one producer warp loading X through
-// registers: 1160 to 2420 us on four boxes).
+// registers: 1160 to 2420 us in four runs).
 template <bool BF16, int T>
 cudaError_t launch(const Format &f, const float *X, int64_t ldx, int64_t batch, float *Y, int64_t ldy, bool early,
                    cudaStream_t stream) {
